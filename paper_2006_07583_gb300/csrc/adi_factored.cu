@@ -872,21 +872,10 @@ __device__ void fac_issue(const LineDesc<T> *__restrict__ descs, const FacGroup 
     }
 }
 
-// W consecutive shared-memory elements into registers (8-byte loads for float when the
-// source is 8-byte aligned).
+// W consecutive shared-memory elements into registers (the chunks' odd stride spreads the lanes
+// over the banks).
 template <typename T, int W>
 __device__ __forceinline__ void load_win(const T *src, T (&w)[W]) {
-    if constexpr (sizeof(T) == 4 && W % 2 == 0) {
-        if ((smem_addr(src) & 7u) == 0) {
-#pragma unroll
-            for (int k = 0; k < W; k += 2) {
-                const float2 q = *reinterpret_cast<const float2 *>(src + k);
-                w[k] = q.x;
-                w[k + 1] = q.y;
-            }
-            return;
-        }
-    }
 #pragma unroll
     for (int k = 0; k < W; ++k) w[k] = src[k];
 }
@@ -913,12 +902,13 @@ __device__ __forceinline__ void load_blk(const T *src, T (&M)[BS][BS]) {
 template <typename T, int BS>
 __device__ __forceinline__ void win_scan(bool forward, int c, int tact, int reach, const T *maps, const T *off,
                                          T (&z)[BS]) {
-#pragma unroll
-    for (int p = 0; p < BS; ++p) z[p] = T(0);
     const int k0 = forward ? max(0, c - reach) : min(tact - 1, c + reach);
     const int n = forward ? c - k0 : k0 - c;
+    // the first map of the window would act on zero: its chunk's value starts the recurrence
+#pragma unroll
+    for (int p = 0; p < BS; ++p) z[p] = n > 0 ? off[k0 * BS + p] : T(0);
 #pragma unroll 4
-    for (int t = 0; t < n; ++t) {
+    for (int t = 1; t < n; ++t) {
         const int k = forward ? k0 + t : k0 - t;
         T M[BS][BS];
         load_blk<T, BS>(maps + k * BS * BS, M);
@@ -1034,23 +1024,23 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
     // Row r < NR1 belongs to the head, r >= NR1 to the tail; within an end, HZ rows come first.
     constexpr int NR1 = E::HMAX + (BS == 3 ? E::HMAX + 2 : 0), NR = 2 * NR1;
     T *scr = lb + gr.scr;
+    auto row_win = [&](int r) {
+        const bool tail = r >= NR1;
+        if (!(tail ? has_tail : has_head)) return;
+        const int q = tail ? r - NR1 : r;
+        const T *row = (tail ? eT : eH) + (q < E::HMAX ? E::HZ + q * Z : E::DZ + (q - E::HMAX) * Z);
+        T a0 = T(0), a1 = T(0);
+#pragma unroll
+        for (int k = 0; k < 2 * W; k += 2) {
+            a0 += row[k] * zval(tail, k);
+            a1 += row[k + 1] * zval(tail, k + 1);
+        }
+        scr[r] = a0 + a1;
+    };
     // Lines of at least three warps: the warps other than the head and tail warps compute the
     // rows after their local forward pass (below), while the end warps form KZ z.
     const bool scr_help = Tl >= 96;
     if (line_ok && !scr_help) {
-        auto row_win = [&](int r) {
-            const bool tail = r >= NR1;
-            if (!(tail ? has_tail : has_head)) return;
-            const int q = tail ? r - NR1 : r;
-            const T *row = (tail ? eT : eH) + (q < E::HMAX ? E::HZ + q * Z : E::DZ + (q - E::HMAX) * Z);
-            T a0 = T(0), a1 = T(0);
-#pragma unroll
-            for (int k = 0; k < 2 * W; k += 2) {
-                a0 += row[k] * zval(tail, k);
-                a1 += row[k + 1] * zval(tail, k + 1);
-            }
-            scr[r] = a0 + a1;
-        };
         const int stride = Tl >= NR ? Tl / NR : 1;
         if (stride > 1) {
             if (c % stride == 0 && c / stride < NR) row_win(c / stride);
@@ -1274,27 +1264,35 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
         }
     }
 
-    // ---- window parts of the end-region rows by the middle warps (one row per half-warp,
-    // one or two terms per lane, then a half-warp sum) ----
+    // ---- window parts of the end-region rows by the middle warps.  A line with five or more takes one
+    // row per half-warp (one or two terms per lane, then a half-warp sum): one to three passes.  A
+    // shorter line's two to four would make up to 18, which took 2300 of a 128-thread line's 9600
+    // cycles: there two of them take one row per lane, head and tail ----
     if (scr_help && line_ok) {
         const int tw = (tact - 1) >> 5;  // the tail warp (tact > 64, so 2 <= tw)
         if (wl != 0 && wl != tw) {
             const int hi = wl - 1 - (wl > tw ? 1 : 0), nh = (Tl >> 5) - 2;
-            const int half = lane >> 4, k = lane & 15;
-            for (int r0 = 2 * hi; r0 < NR; r0 += 2 * nh) {  // warp-uniform trip count
-                const int r = r0 + half;
-                const bool tail = r >= NR1;
-                const int q = tail ? r - NR1 : r;
-                T a = T(0);
-                const bool here = r < NR && (tail ? has_tail : has_head);
-                if (here) {
-                    const T *row = (tail ? eT : eH) + (q < E::HMAX ? E::HZ + q * Z : E::DZ + (q - E::HMAX) * Z);
-                    a = row[k] * zval(tail, k);
-                    if (k + 16 < 2 * W) a += row[k + 16] * zval(tail, k + 16);
-                }
+            if (nh < 5) {
+                static_assert(NR1 <= 32, "an end's rows fit one warp");
+                if (hi == 0 && lane < NR1) row_win(lane);
+                if (hi == (nh > 1 ? 1 : 0) && lane < NR1) row_win(NR1 + lane);
+            } else {
+                const int half = lane >> 4, k = lane & 15;
+                for (int r0 = 2 * hi; r0 < NR; r0 += 2 * nh) {  // warp-uniform trip count
+                    const int r = r0 + half;
+                    const bool tail = r >= NR1;
+                    const int q = tail ? r - NR1 : r;
+                    T a = T(0);
+                    const bool here = r < NR && (tail ? has_tail : has_head);
+                    if (here) {
+                        const T *row = (tail ? eT : eH) + (q < E::HMAX ? E::HZ + q * Z : E::DZ + (q - E::HMAX) * Z);
+                        a = row[k] * zval(tail, k);
+                        if (k + 16 < 2 * W) a += row[k + 16] * zval(tail, k + 16);
+                    }
 #pragma unroll
-                for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-                if (k == 0 && here) scr[r] = a;
+                    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    if (k == 0 && here) scr[r] = a;
+                }
             }
         }
     }
@@ -1312,6 +1310,7 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
         }
         seg_scan<T, BS>(mp, true, Tl, yin, ssm);
     } else {
+        if (offb == offf) workers_sync();  // one offset buffer: the group before has read its values
         if (act)
 #pragma unroll
             for (int p = 0; p < BS; ++p) lofff[c * BS + p] = Y[MM - 1][p];
