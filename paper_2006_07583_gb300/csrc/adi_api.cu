@@ -637,6 +637,24 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
     std::vector<int4> gr[2][2];
     std::vector<FacGroup> fgr[2][kFacVariants];
     size_t words = 0;
+    const int sms = sm_count();
+    // Line groups of a factored launch: the fewest groups its lines need (as many lines each as a CTA
+    // takes) decide the rounds that the persistent CTAs make; the lines are then spread evenly over all
+    // the rounds' groups, so that no SM idles while others solve full groups.
+    int fmin[2][kFacVariants] = {}, frounds[2][kFacVariants] = {};
+    auto fac_cap = [&](const adi_sim *s, int N) {
+        const int nl = fac_lines_per_cta(s->g.method, N, esz);
+        return s->fac_nl_cap > 0 ? std::min(nl, s->fac_nl_cap) : nl;
+    };
+    for (const adi_sim *s : members)
+        for (int dir = 0; dir < 2; ++dir) {
+            const int N = dir == 0 ? s->g.nx : s->g.ny;
+            if (s->solver != ADI_SOLVER_FACTORED || fac_split_line(s->g.method, N)) continue;
+            const int nl = fac_cap(s, N);
+            fmin[dir][fac_variant(s->g.method, N)] += (s->nlines[dir] + nl - 1) / nl;
+        }
+    for (int dir = 0; dir < 2; ++dir)
+        for (int v = 0; v < kFacVariants; ++v) frounds[dir][v] = (fmin[dir][v] + sms - 1) / sms;
     for (adi_sim *s : members) {
         for (int dir = 0; dir < 2; ++dir) {
             if (s->solver == ADI_SOLVER_LINE) {
@@ -661,15 +679,16 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
                         p.fstage[dir][v] = std::max(p.fstage[dir][v], sb);
                     }
                 } else {
-                    int nl = fac_lines_per_cta(s->g.method, N, esz);
-                    if (s->fac_nl_cap > 0) nl = std::min(nl, s->fac_nl_cap);
-                    for (int st = 0; st < n; st += nl) {
-                        int cnt = std::min(nl, n - st);
+                    const int nl = fac_cap(s, N), need = (n + nl - 1) / nl;
+                    const int ng = (int)std::min<long long>(n, (long long)need * frounds[dir][v] * sms / fmin[dir][v]);
+                    for (int k = 0, st = 0; k < ng; ++k) {
+                        const int cnt = n / ng + (k < n % ng ? 1 : 0);
                         FacGroup fg = fac_group_of(s->g.method, N, first + st, cnt, 1.0 / s->h, 0.5 * s->dt);
                         // the scans this simulation's lines need, whatever else shares the launch
                         if (s->fac_reach > kFacMaxReach) fg.own |= kFacOwnFull;
                         fgr[dir][v].push_back(fg);
                         p.fstage[dir][v] = std::max(p.fstage[dir][v], fac_stage_bytes(s->g.method, N, cnt, esz));
+                        st += cnt;
                     }
                 }
                 if (s->fac_ring_cap > 0)
@@ -722,10 +741,13 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
             }
         }
         for (int v = 0; v < kFacVariants && !rc; ++v) {
+            // the groups with most threads first: the last round's are the small ones
+            std::stable_sort(fgr[dir][v].begin(), fgr[dir][v].end(),
+                             [](const FacGroup &a, const FacGroup &b) { return a.nl * a.T > b.nl * b.T; });
             p.nfgroups[dir][v] = (int)fgr[dir][v].size();
             p.fstages[dir][v] = fac_stages_for(p.fstage[dir][v], esz, (v == 0 || v == 3) ? ADI_CFD : ADI_MFD);
             if (p.fring[dir][v] > 0) p.fstages[dir][v] = std::min(p.fstages[dir][v], p.fring[dir][v]);
-            p.fgrid[dir][v] = std::min(p.nfgroups[dir][v], sm_count());
+            p.fgrid[dir][v] = std::min(p.nfgroups[dir][v], sms);
             if (p.nfgroups[dir][v] && !p.fstages[dir][v]) { rc = ADI_ENOTSUP; break; }
             if (!fgr[dir][v].empty()) {
                 rc = dev_alloc(p.fgroups[dir][v], fgr[dir][v].size() * sizeof(FacGroup));
