@@ -62,6 +62,8 @@ __host__ __device__ inline size_t fac_static_smem(size_t esz, int bs) {
 // two code paths of the same output round differently.
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 // ---------------------------------------------------------------------------------------
 // Geometry of a line for the factored solver.
@@ -1024,23 +1026,23 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
     // Row r < NR1 belongs to the head, r >= NR1 to the tail; within an end, HZ rows come first.
     constexpr int NR1 = E::HMAX + (BS == 3 ? E::HMAX + 2 : 0), NR = 2 * NR1;
     T *scr = lb + gr.scr;
-    auto row_win = [&](int r) {
-        const bool tail = r >= NR1;
-        if (!(tail ? has_tail : has_head)) return;
-        const int q = tail ? r - NR1 : r;
-        const T *row = (tail ? eT : eH) + (q < E::HMAX ? E::HZ + q * Z : E::DZ + (q - E::HMAX) * Z);
-        T a0 = T(0), a1 = T(0);
-#pragma unroll
-        for (int k = 0; k < 2 * W; k += 2) {
-            a0 += row[k] * zval(tail, k);
-            a1 += row[k + 1] * zval(tail, k + 1);
-        }
-        scr[r] = a0 + a1;
-    };
     // Lines of at least three warps: the warps other than the head and tail warps compute the
     // rows after their local forward pass (below), while the end warps form KZ z.
     const bool scr_help = Tl >= 96;
     if (line_ok && !scr_help) {
+        auto row_win = [&](int r) {
+            const bool tail = r >= NR1;
+            if (!(tail ? has_tail : has_head)) return;
+            const int q = tail ? r - NR1 : r;
+            const T *row = (tail ? eT : eH) + (q < E::HMAX ? E::HZ + q * Z : E::DZ + (q - E::HMAX) * Z);
+            T a0 = T(0), a1 = T(0);
+    #pragma unroll
+            for (int k = 0; k < 2 * W; k += 2) {
+                a0 += row[k] * zval(tail, k);
+                a1 += row[k + 1] * zval(tail, k + 1);
+            }
+            scr[r] = a0 + a1;
+        };
         const int stride = Tl >= NR ? Tl / NR : 1;
         if (stride > 1) {
             if (c % stride == 0 && c / stride < NR) row_win(c / stride);
@@ -1267,15 +1269,30 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
     // ---- window parts of the end-region rows by the middle warps.  A line with five or more takes one
     // row per half-warp (one or two terms per lane, then a half-warp sum): one to three passes.  A
     // shorter line's two to four would make up to 18, which took 2300 of a 128-thread line's 9600
-    // cycles: there two of them take one row per lane, head and tail ----
+    // cycles: there two of them take one row per lane, head and tail, adding the terms in the half-warp's order ----
     if (scr_help && line_ok) {
         const int tw = (tact - 1) >> 5;  // the tail warp (tact > 64, so 2 <= tw)
         if (wl != 0 && wl != tw) {
             const int hi = wl - 1 - (wl > tw ? 1 : 0), nh = (Tl >> 5) - 2;
             if (nh < 5) {
                 static_assert(NR1 <= 32, "an end's rows fit one warp");
-                if (hi == 0 && lane < NR1) row_win(lane);
-                if (hi == (nh > 1 ? 1 : 0) && lane < NR1) row_win(NR1 + lane);
+                auto row_tree = [&](bool tail) {
+                    if (!(tail ? has_tail : has_head) || lane >= NR1) return;
+                    const T *row = (tail ? eT : eH) + (lane < E::HMAX ? E::HZ + lane * Z : E::DZ + (lane - E::HMAX) * Z);
+                    T a[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        a[k] = mul_rn(row[k], zval(tail, k));
+                        if (k + 16 < 2 * W) a[k] = fma_rn(row[k + 16], zval(tail, k + 16), a[k]);
+                    }
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                        for (int k = 0; k < o; ++k) a[k] += a[k + o];
+                    scr[(tail ? NR1 : 0) + lane] = a[0];
+                };
+                if (hi == 0) row_tree(false);
+                if (hi == (nh > 1 ? 1 : 0)) row_tree(true);
             } else {
                 const int half = lane >> 4, k = lane & 15;
                 for (int r0 = 2 * hi; r0 < NR; r0 += 2 * nh) {  // warp-uniform trip count

@@ -1,0 +1,66 @@
+"""GPU: the sizes at which the step's kernels change their path or their tiles end, against the FP64 CPU oracle.
+
+Tolerances are the path's own (FP64 max |difference| <= 1e-12 x max |field|, FP32 relative L2 <= 1e-4), for
+the few steps taken here; where two GPU paths are compared they are derived beside the test.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2006_07583_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+CFD, MFD = wl.CFD, wl.MFD
+
+
+@pytest.fixture(scope="module")
+def adi():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2006_07583_gb300 import adi as _adi
+
+    _adi.lib()
+    return _adi
+
+
+def _case(method, nx, ny, seed, cfl=0.8):
+    rng = np.random.default_rng(seed)
+    su, sv, sw = wl.shapes(method, nx, ny)
+    h = 1.0 / max(nx, ny)
+    c = rng.uniform(0.6, 1.4, su)
+    U, V, W = rng.standard_normal(su), rng.standard_normal(sv), rng.standard_normal(sw)
+    return h, cfl * h / c.max(), c, U, V, W
+
+
+def _check(got, want, fp64):
+    for g, o in zip(got, want):
+        if fp64:
+            assert np.max(np.abs(g - o)) <= 1e-12 * np.max(np.abs(o))
+        else:
+            assert np.linalg.norm(g - o) <= 1e-4 * np.linalg.norm(o)
+
+
+# chunks per line on either side of: 32 | 33 (a line within a warp), 64 | 65 (end rows by the middle warps), 192 |
+# 193 and 224 | 225 (one row per lane or per half-warp; FP64 CTAs of 256 or 512 threads), and the last line lengths
+# of an MFD remainder of 0, 1 and 2 blocks; chunks are 9 nodes (CFD, N - 5 of them) or 9 cells (MFD, about N - 8)
+LINES = [(CFD, 5 + 9 * 32), (CFD, 5 + 9 * 33), (CFD, 5 + 9 * 64 + 8), (CFD, 5 + 9 * 65), (CFD, 5 + 9 * 192),
+         (CFD, 5 + 9 * 193), (CFD, 5 + 9 * 224 + 8), (CFD, 5 + 9 * 225), (MFD, 16), (MFD, 17), (MFD, 8 + 9 * 32),
+         (MFD, 8 + 9 * 33 + 4), (MFD, 8 + 9 * 65 + 7), (MFD, 8 + 9 * 193), (MFD, 8 + 9 * 224 + 8), (MFD, 8 + 9 * 225 + 1)]
+
+
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("method,n", LINES)
+def test_line_lengths_at_path_changes(adi, method, n, fp64):
+    nx, ny = (n, 20) if n % 2 else (20, n)  # the long lines along x or y
+    h, dt, c, U, V, W = _case(method, nx, ny, n)
+    src = (ny // 2, nx // 3, 0.01, 15.0, 0.0)
+    sim = adi.Sim(method, nx, ny, h, dt, c, U, V, W, precision=adi.ADI_FP64 if fp64 else adi.ADI_FP32)
+    assert sim.solver == adi.ADI_SOLVER_FACTORED
+    sim.set_source(*src)
+    sim.step(3)
+    G = sim.read()
+    sim.close()
+    _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, 3, source=src), fp64)
