@@ -651,7 +651,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
             const int N = dir == 0 ? s->g.nx : s->g.ny;
             if (s->solver != ADI_SOLVER_FACTORED || fac_split_line(s->g.method, N)) continue;
             const int nl = fac_cap(s, N);
-            fmin[dir][fac_variant(s->g.method, N)] += (s->nlines[dir] + nl - 1) / nl;
+            fmin[dir][fac_variant(s->g.method, N, esz)] += (s->nlines[dir] + nl - 1) / nl;
         }
     for (int dir = 0; dir < 2; ++dir)
         for (int v = 0; v < kFacVariants; ++v) frounds[dir][v] = (fmin[dir][v] + sms - 1) / sms;
@@ -666,7 +666,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
                 int first = (int)(fdv[0][dir].size() / dsz);
                 int n = s->nlines[dir];
                 int N = dir == 0 ? s->g.nx : s->g.ny;
-                int v = fac_variant(s->g.method, N);
+                int v = fac_variant(s->g.method, N, esz);
                 if (fac_split_line(s->g.method, N)) {
                     // lines longer than a CTA's chunks: sub-lines with a halo of the scan reach
                     FacGroup sub[kFacMaxSplit];
@@ -745,7 +745,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
             std::stable_sort(fgr[dir][v].begin(), fgr[dir][v].end(),
                              [](const FacGroup &a, const FacGroup &b) { return a.nl * a.T > b.nl * b.T; });
             p.nfgroups[dir][v] = (int)fgr[dir][v].size();
-            p.fstages[dir][v] = fac_stages_for(p.fstage[dir][v], esz, (v == 0 || v == 3) ? ADI_CFD : ADI_MFD);
+            p.fstages[dir][v] = fac_stages_for(p.fstage[dir][v], esz, fac_variant_method(v));
             if (p.fring[dir][v] > 0) p.fstages[dir][v] = std::min(p.fstages[dir][v], p.fring[dir][v]);
             p.fgrid[dir][v] = std::min(p.nfgroups[dir][v], sms);
             if (p.nfgroups[dir][v] && !p.fstages[dir][v]) { rc = ADI_ENOTSUP; break; }

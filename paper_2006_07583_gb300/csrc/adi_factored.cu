@@ -45,6 +45,7 @@
 namespace adi {
 
 constexpr int kFacThreads = 512;              // threads per CTA: 15 compute warps and one staging warp
+constexpr int kFacNarrow = 256;               // MFD in FP64, lines of at most 224 chunks: 7 compute warps (fac_narrow)
 constexpr int kFacWorkers = kFacThreads - 32; // threads that solve lines
 constexpr int kFacMaxT = kFacWorkers;         // chunks (threads) per line at most
 constexpr size_t kFacSmemLimit = 227 * 1024;  // shared memory per CTA
@@ -85,6 +86,14 @@ __host__ __device__ inline int fac_geom_T(int method, int N) {
     int T = 1;
     while (T < tact) T <<= 1;
     return T;
+}
+// MFD lines of at most 224 chunks run in FP64 in CTAs of 256 threads: twice the registers a thread (the
+// band form's 72 FP64 values do not fit 128 registers and spilled 0.5 KB a thread, more than the L1 beside the staged
+// lines holds), and seven warps keep the FP64 pipe as busy as fifteen: 1001 lines of 1001 cells 200 ->
+// 144 us with the band form.  CFD, whose lines of 512 cells then made two rounds instead of one, gained nothing (55.7
+// -> 58.0 us) and keeps the wide CTAs.
+__host__ __device__ inline bool fac_narrow(int method, int T, size_t esz) {
+    return method == kMFD && esz == 8 && T <= kFacNarrow - 32;
 }
 // Kernel variant (one compiled instance per chunk length and method, and for split lines).
 __host__ __device__ inline int fac_variant_of(int method, int N) {
@@ -177,8 +186,8 @@ int fac_stages_for(size_t stage_bytes, size_t esz, int method) {
 // Lines per CTA: as many as the CTA's threads cover, fewer where a two-stage ring of them
 // would not fit shared memory.
 int fac_lines_per_cta(int method, int N, size_t esz) {
-    const int T = fac_geom(method, N).T;
-    int nl = T >= kFacWorkers ? 1 : kFacWorkers / T;
+    const int T = fac_geom(method, N).T, workers = fac_narrow(method, T, esz) ? kFacNarrow - 32 : kFacWorkers;
+    int nl = T >= workers ? 1 : workers / T;
     while (nl > 1 && fac_stages_for(fac_stage_bytes(method, N, nl, esz), esz, method) < 2) --nl;
     return nl;
 }
@@ -196,7 +205,11 @@ bool fac_supported(int method, int N, size_t esz) {
 }
 size_t fac_words(int method, int N) { return (size_t)fac_rec(fac_geom(method, N)); }
 int fac_chunks(int method, int N) { return fac_geom(method, N).T; }
-int fac_variant(int method, int N) { return fac_variant_of(method, N); }
+int fac_variant(int method, int N, size_t esz) {
+    const int v = fac_variant_of(method, N);
+    return fac_narrow(method, fac_geom(method, N).T, esz) ? v + 4 : v;
+}
+int fac_variant_method(int v) { return v == 0 || v == 3 ? kCFD : kMFD; }
 size_t fac_ws_doubles() { return kFacWs; }
 static unsigned fac_tdiv(int T) {
     return T > 1 ? (unsigned)(((1ull << 32) + (unsigned long long)T - 1) / (unsigned long long)T) : 0u;
@@ -642,9 +655,11 @@ __device__ __forceinline__ void map_shfl(Map<T, BS> &dst, const Map<T, BS> &src,
     }
 }
 
-// Barrier of the compute warps (named barrier 1; the staging warp does not take part).
+// Barrier of the compute warps of a CTA of NT threads (named barrier 1; the staging warp does not take
+// part).
+template <int NT>
 __device__ __forceinline__ void workers_sync() {
-    asm volatile("bar.sync 1, %0;" ::"r"(kFacWorkers) : "memory");
+    asm volatile("bar.sync 1, %0;" ::"r"(NT - 32) : "memory");
 }
 
 // Scan buffers of a CTA: warp aggregates and warp prefixes.
@@ -659,7 +674,7 @@ struct ScanSmem {
 // shuffles only).  forward: z(c) = (a_{c-1} o ... o a_0)(0), the value entering chunk c;
 // backward: z(c) = (a_{c+1} o ... o a_{Tl-1})(0), the value after chunk c.  Every thread of
 // the CTA must call it with the same Tl.
-template <typename T, int BS>
+template <typename T, int BS, int NT>
 __device__ __forceinline__ void seg_scan(Map<T, BS> a, bool forward, int Tl, T (&z)[BS], ScanSmem<T, BS> &sm) {
     const int tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
@@ -682,9 +697,9 @@ __device__ __forceinline__ void seg_scan(Map<T, BS> a, bool forward, int Tl, T (
     }
     const int nw = Tl >> 5;          // warps per line
     const int wl = warp % nw;        // warp index within its line
-    const bool whole = (tid / Tl) < (kFacWorkers / Tl);  // inside a whole line of the CTA
+    const bool whole = (tid / Tl) < ((NT - 32) / Tl);  // inside a whole line of the CTA
     if (pos == 31) sm.agg[warp] = a;  // the warp's full composition
-    workers_sync();
+    workers_sync<NT>();
     if (whole && wl == 0 && lane == 0) {
         T p[BS];
 #pragma unroll
@@ -706,7 +721,7 @@ __device__ __forceinline__ void seg_scan(Map<T, BS> a, bool forward, int Tl, T (
             for (int i = 0; i < BS; ++i) p[i] = q[i];
         }
     }
-    workers_sync();
+    workers_sync<NT>();
 #pragma unroll
     for (int i = 0; i < BS; ++i) {
         T acc = ex.off[i];
@@ -717,13 +732,21 @@ __device__ __forceinline__ void seg_scan(Map<T, BS> a, bool forward, int Tl, T (
 }
 
 // Block inverse of the line kernel: the FP32 path takes the hardware reciprocal
-// approximation (relative error below 2^-22), FP64 an IEEE division.
+// approximation (relative error below 2^-22).
 __device__ __forceinline__ float fac_rcp(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-__device__ __forceinline__ double fac_rcp(double x) { return 1.0 / x; }
+// FP64: the hardware approximation r0 (about 20 bits) and one step of Householder's cubic iteration, r0 (1 + e
+// + e^2) with e = 1 - x r0: three FMAs against a division's ten or so operations on the FP64 pipe that bounds these kernels;
+// the error left is e^3 = 2^-60 and one rounding (measured against 1 / x: at most 1 ulp).
+__device__ __forceinline__ double fac_rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
 template <typename T, int BS>
 __device__ __forceinline__ void fac_inv(const T (&S)[BS][BS], T (&R)[BS][BS]) {
     if constexpr (BS == 2) {
@@ -927,11 +950,117 @@ __device__ __forceinline__ void win_scan(bool forward, int c, int tact, int reac
     }
 }
 
+// An MFD chunk in FP64, eliminated row by row as a band matrix.  Row k is 1 - s K_0 on the diagonal and -s K_d
+// at distance d = 1..3 (s = alpha beta / h^2, K the 7-point operator); Crout form: L_d the eliminated lower bands, q
+// = 1 / pivot, v_d the eliminated upper bands times q.  About 31 FP64 operations a cell for the factors and
+// the substitutions, against about 55 for 3 x 3 block products and inverses: the FP64 pipe bounds the kernel (1001
+// lines of 1001 cells: 200 -> 144 us together with the cheaper reciprocals and the 256-thread CTAs).
+// FP32 keeps the block form: three approximate reciprocals a block instead of one doubled its error (100 x 100 cells,
+// 25 steps: 1.3e-6 -> 3.4e-6 of the 64-bit result) for 1-3 %.
+template <int MM>
+struct MfdBand {
+    static constexpr int NC = 3 * MM;
+    double L1[NC], L2[NC], L3[NC], q[NC], v1[NC], v2[NC];  // the third upper band is L3 q
+    // Factors, and the block value y that leaves the chunk if none enters it.  S: the Schur complement of the
+    // chunk's first block; dB: the tail region's correction of its last block, or nullptr.
+    __device__ __forceinline__ void factor(const double (&al)[NC], double bh2, const double (&S)[3][3], const double *dB,
+                                           const double (&Y)[MM][3], double (&yend)[3]) {
+        double v3[NC], z[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const double sc = al[k] * bh2;
+            double di = 1.0 - sc * mim_DG(3);
+            double lo1 = -sc * mim_DG(2), lo2 = -sc * mim_DG(1), up1 = lo1, up2 = lo2;
+            L3[k] = -sc * mim_DG(0);
+            if (k < 3) {  // in-block entries
+                di = S[k][k];
+                if (k >= 1) lo1 = S[k][k >= 1 ? k - 1 : 0];
+                if (k == 2) lo2 = S[k][0];
+                if (k <= 1) up1 = S[k][k <= 1 ? k + 1 : 2];
+                if (k == 0) up2 = S[k][2];
+            } else if (k >= NC - 3 && dB) {
+                const int p = k - (NC - 3);
+                di -= dB[p * 3 + p];
+                if (p >= 1) lo1 -= dB[p * 3 + p - 1];
+                if (p == 2) lo2 -= dB[p * 3];
+                if (p <= 1) up1 -= dB[p * 3 + p + 1];
+                if (p == 0) up2 -= dB[2];
+            }
+            double zz = Y[k / 3][k % 3];
+            if (k >= 3) {
+                lo2 -= L3[k] * v1[k - 3];
+                lo1 -= L3[k] * v2[k - 3];
+                di -= L3[k] * v3[k - 3];
+                zz -= L3[k] * z[k - 3];
+            }
+            if (k >= 2) {
+                L2[k] = lo2;
+                lo1 -= lo2 * v1[k - 2];
+                di -= lo2 * v2[k - 2];
+                up1 -= lo2 * v3[k - 2];
+                zz -= lo2 * z[k - 2];
+            }
+            if (k >= 1) {
+                L1[k] = lo1;
+                di -= lo1 * v1[k - 1];
+                up1 -= lo1 * v2[k - 1];
+                up2 -= lo1 * v3[k - 1];
+                zz -= lo1 * z[k - 1];
+            }
+            q[k] = fac_rcp(di);
+            v1[k] = up1 * q[k];
+            v2[k] = up2 * q[k];
+            v3[k] = L3[k] * q[k];
+            z[k] = zz * q[k];
+        }
+        yend[2] = z[NC - 1];
+        yend[1] = z[NC - 2] - v1[NC - 2] * z[NC - 1];
+        yend[0] = z[NC - 3] - v1[NC - 3] * yend[1] - v2[NC - 3] * z[NC - 1];
+    }
+    // Y: r -> the true forward values, from the block value yin that enters; xfirst: x of the first block if
+    // nothing follows the chunk.
+    __device__ __forceinline__ void forward(const double (&al)[NC], double bh2, const double (&yin)[3], double (&Y)[MM][3],
+                                            double (&xfirst)[3]) {
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const double sc = al[m] * bh2;
+#pragma unroll
+            for (int p = m; p < 3; ++p) Y[0][m] += sc * mim_DG(p - m) * yin[p];
+        }
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            double a = Y[k / 3][k % 3];
+            if (k >= 3) a -= L3[k] * Y[(k - 3) / 3][(k - 3) % 3];
+            if (k >= 2) a -= L2[k] * Y[(k - 2) / 3][(k - 2) % 3];
+            if (k >= 1) a -= L1[k] * Y[(k - 1) / 3][(k - 1) % 3];
+            Y[k / 3][k % 3] = a * q[k];
+            L3[k] *= q[k];  // from here on the third upper band
+        }
+        double x1 = 0.0, x2 = 0.0, x3 = 0.0;
+#pragma unroll
+        for (int k = NC - 1; k >= 0; --k) {
+            const double x = Y[k / 3][k % 3] - L3[k] * x3 - v2[k] * x2 - v1[k] * x1;
+            x3 = x2; x2 = x1; x1 = x;
+        }
+        xfirst[0] = x1; xfirst[1] = x2; xfirst[2] = x3;
+    }
+    // Y -> x, from the x that follows the chunk.
+    __device__ __forceinline__ void backward(const double (&xin)[3], double (&Y)[MM][3]) {
+        double x1 = xin[0], x2 = xin[1], x3 = xin[2];
+#pragma unroll
+        for (int k = NC - 1; k >= 0; --k) {
+            const double x = Y[k / 3][k % 3] - L3[k] * x3 - v2[k] * x2 - v1[k] * x1;
+            Y[k / 3][k % 3] = x;
+            x3 = x2; x2 = x1; x1 = x;
+        }
+    }
+};
+
 // ---------------------------------------------------------------------------------------
 // One line group from its staged inputs: nl lines of one simulation and direction, Tl
 // threads per line; thread (l, c) = (tid / Tl, tid % Tl) owns middle blocks [c MM, c MM + MM).
 // ---------------------------------------------------------------------------------------
-template <typename T, int BS, int MM, bool SPLIT>
+template <typename T, int BS, int MM, bool SPLIT, int NT>
 __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural, ScanSmem<T, BS> &ssm,
                                           T *offf, T *offb) {
     static_assert(MM >= 2, "chunks of at least two blocks");
@@ -1179,8 +1308,19 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
     };
 
     // ---- factorisation and local forward pass ----
-    T Si[MM][BS][BS];
-    if (act) {
+    constexpr bool kBand = BS == 3 && sizeof(T) == 8;
+    T Si[kBand ? 1 : MM][BS][BS];
+    [[maybe_unused]] MfdBand<BS == 3 ? MM : 2> band;  // MFD in FP64
+    T yend[BS], xfirst[BS];  // the chunk's y at its end if none enters it; x at its start if none follows
+#pragma unroll
+    for (int p = 0; p < BS; ++p) yend[p] = xfirst[p] = T(0);
+    if constexpr (kBand) {
+        if (act) {
+            T S[BS][BS];
+            load_blk<T, BS>(sR + c * B2, S);
+            band.factor(aw, beta * ih * ih, S, is_tail ? eT + E::DB : nullptr, Y, yend);
+        }
+    } else if (act) {
         T G[BS][BS];
 #pragma unroll
         for (int i = 0; i < MM; ++i) {
@@ -1264,6 +1404,8 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
                 }
             }
         }
+#pragma unroll
+        for (int p = 0; p < BS; ++p) yend[p] = Y[MM - 1][p];
     }
 
     // ---- window parts of the end-region rows by the middle warps.  A line with five or more takes one
@@ -1321,20 +1463,22 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
         if (act) {
             load_blk<T, BS>(sR + gr.part + c * B2, mp.m);
 #pragma unroll
-            for (int p = 0; p < BS; ++p) mp.off[p] = Y[MM - 1][p];
+            for (int p = 0; p < BS; ++p) mp.off[p] = yend[p];
         } else {
             map_id<T, BS>(mp);
         }
-        seg_scan<T, BS>(mp, true, Tl, yin, ssm);
+        seg_scan<T, BS, NT>(mp, true, Tl, yin, ssm);
     } else {
-        if (offb == offf) workers_sync();  // one offset buffer: the group before has read its values
+        if (offb == offf) workers_sync<NT>();  // one offset buffer: the group before has read its values
         if (act)
 #pragma unroll
-            for (int p = 0; p < BS; ++p) lofff[c * BS + p] = Y[MM - 1][p];
-        workers_sync();
+            for (int p = 0; p < BS; ++p) lofff[c * BS + p] = yend[p];
+        workers_sync<NT>();
         if (act) win_scan<T, BS>(true, c, tact, (int)sinfo[0], sR + gr.part, lofff, yin);
     }
-    if (act) {
+    if constexpr (kBand) {
+        if (act) band.forward(aw, beta * ih * ih, yin, Y, xfirst);
+    } else if (act) {
         T dl[BS];
 #pragma unroll
         for (int p = 0; p < BS; ++p) dl[p] = yin[p];
@@ -1355,6 +1499,8 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
 #pragma unroll
             for (int p = 0; p < BS; ++p) Y[i][p] += u[p];
         }
+#pragma unroll
+        for (int p = 0; p < BS; ++p) xfirst[p] = Y[0][p];
     }
 
     // ---- backward scan: the true x after the chunk; correction ----
@@ -1364,20 +1510,22 @@ __device__ __forceinline__ void fac_group(unsigned char *stage_raw, int natural,
         if (act) {
             load_blk<T, BS>(sR + 2 * gr.part + c * B2, mp.m);
 #pragma unroll
-            for (int p = 0; p < BS; ++p) mp.off[p] = Y[0][p];
+            for (int p = 0; p < BS; ++p) mp.off[p] = xfirst[p];
         } else {
             map_id<T, BS>(mp);
         }
-        seg_scan<T, BS>(mp, false, Tl, xin, ssm);
+        seg_scan<T, BS, NT>(mp, false, Tl, xin, ssm);
     } else {
-        if (offb == offf) workers_sync();  // one offset buffer: the forward reads are done
+        if (offb == offf) workers_sync<NT>();  // one offset buffer: the forward reads are done
         if (act)
 #pragma unroll
-            for (int p = 0; p < BS; ++p) loffb[c * BS + p] = Y[0][p];
-        workers_sync();
+            for (int p = 0; p < BS; ++p) loffb[c * BS + p] = xfirst[p];
+        workers_sync<NT>();
         if (act) win_scan<T, BS>(false, c, tact, (int)sinfo[1], sR + 2 * gr.part, loffb, xin);
     }
-    if (act) {
+    if constexpr (kBand) {
+        if (act) band.backward(xin, Y);
+    } else if (act) {
         T ep[BS];
 #pragma unroll
         for (int p = 0; p < BS; ++p) ep[p] = xin[p];
@@ -1620,8 +1768,8 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-template <typename T, int BS, int MM, bool SPLIT>
-__global__ void __launch_bounds__(kFacThreads, 1)
+template <typename T, int BS, int MM, bool SPLIT, int NT>
+__global__ void __launch_bounds__(NT, 1)
 line_solve_factored_kernel(const LineDesc<T> *__restrict__ descs, const FacGroup *__restrict__ groups, int ngroups,
                            int natural, unsigned stage_bytes, int stages, int *fault) {
     extern __shared__ __align__(128) unsigned char fac_smem[];
@@ -1629,18 +1777,18 @@ line_solve_factored_kernel(const LineDesc<T> *__restrict__ descs, const FacGroup
     __shared__ __align__(8) unsigned long long full[kFacMaxStages], empty[kFacMaxStages];
     // chunk offsets of the windowed scans: forward and backward buffers for FP32, one for FP64
     constexpr int kBufs = sizeof(T) == 4 ? 2 : 1;
-    __shared__ T offs[kBufs][kFacThreads * BS];
+    __shared__ T offs[kBufs][NT * BS];
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) {
         for (int k = 0; k < kFacMaxStages; ++k) {
             mbar_init(&full[k], 1);
-            mbar_init(&empty[k], kFacWorkers / 32);
+            mbar_init(&empty[k], (NT - 32) / 32);
         }
         mbar_fence_init();
     }
     __syncthreads();
     // the it-th group of this CTA goes to stage it % stages, as that stage's use-th group
-    if (tid >= kFacWorkers) {  // the staging warp; every lane runs the same loop
+    if (tid >= NT - 32) {  // the staging warp; every lane runs the same loop
         int last[kFacMaxStages];
         for (int k = 0; k < kFacMaxStages; ++k) last[k] = -1;
         int st = 0, use = 0;
@@ -1675,7 +1823,7 @@ line_solve_factored_kernel(const LineDesc<T> *__restrict__ descs, const FacGroup
     int st = 0, use = 0;
     for (int gi = blockIdx.x; gi < ngroups; gi += gridDim.x) {
         if (!mbar_wait(&full[st], (unsigned)(use & 1))) atomicExch(fault, 1);
-        fac_group<T, BS, MM, SPLIT>(fac_smem + (size_t)st * stage_bytes, natural, ssm, offs[0], offs[kBufs - 1]);
+        fac_group<T, BS, MM, SPLIT, NT>(fac_smem + (size_t)st * stage_bytes, natural, ssm, offs[0], offs[kBufs - 1]);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[st]);
         if (++st == stages) { st = 0; ++use; }
@@ -1689,10 +1837,10 @@ cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, double *ws, 
     return cudaGetLastError();
 }
 
-template <typename T, int BS, int MM, bool SPLIT>
+template <typename T, int BS, int MM, bool SPLIT, int NT>
 cudaError_t launch_fac_inst(const LineDesc<T> *d, const FacGroup *groups, int ngroups, size_t stage_bytes, int stages,
                             int grid, int natural, int *fault, cudaStream_t s) {
-    auto kern = line_solve_factored_kernel<T, BS, MM, SPLIT>;
+    auto kern = line_solve_factored_kernel<T, BS, MM, SPLIT, NT>;
     // the host sizes the ring with fac_static_smem, an upper bound of the kernel's own static
     // shared memory: check it against the compiled kernel once
     static const bool static_ok = [&] {
@@ -1703,7 +1851,7 @@ cudaError_t launch_fac_inst(const LineDesc<T> *d, const FacGroup *groups, int ng
     const size_t dyn = (size_t)stages * stage_bytes;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kFacThreads, dyn, s>>>(d, groups, ngroups, natural, (unsigned)stage_bytes, stages, fault);
+    kern<<<grid, NT, dyn, s>>>(d, groups, ngroups, natural, (unsigned)stage_bytes, stages, fault);
     return cudaGetLastError();
 }
 
@@ -1714,12 +1862,20 @@ cudaError_t launch_line_solve_factored(const LineDesc<T> *d, const FacGroup *gro
     if (ngroups <= 0) return cudaSuccess;
     if (grid > ngroups) grid = ngroups;
     if (stages < 1 || stages > kFacMaxStages) return cudaErrorInvalidValue;
+    constexpr int W = kFacThreads;
     switch (variant) {
-    case 0: return launch_fac_inst<T, 2, 9, false>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 1: return launch_fac_inst<T, 3, 2, false>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 2: return launch_fac_inst<T, 3, 3, false>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 3: return launch_fac_inst<T, 2, 9, true>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 4: return launch_fac_inst<T, 3, 3, true>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    case 0: return launch_fac_inst<T, 2, 9, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    case 1: return launch_fac_inst<T, 3, 2, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    case 2: return launch_fac_inst<T, 3, 3, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    case 3: return launch_fac_inst<T, 2, 9, true, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    case 4: return launch_fac_inst<T, 3, 3, true, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    }
+    if constexpr (sizeof(T) == 8) {
+        constexpr int NR = kFacNarrow;
+        switch (variant) {
+        case 5: return launch_fac_inst<T, 3, 2, false, NR>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+        case 6: return launch_fac_inst<T, 3, 3, false, NR>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+        }
     }
     return cudaErrorInvalidValue;
 }

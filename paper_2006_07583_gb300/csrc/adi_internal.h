@@ -140,8 +140,10 @@ int fac_split_groups(int method, int N, int first, int halo, double inv_h, doubl
 bool fac_supported(int method, int N, size_t esz);  // chunks fit a CTA, stage fits smem
 size_t fac_words(int method, int N);     // elements of one line's record
 int fac_chunks(int method, int N);       // threads per line
-int fac_variant(int method, int N);      // compiled kernel instance: 0 CFD, 1-2 MFD, 3-4 split lines
-constexpr int kFacVariants = 5;
+// compiled kernel instance: 0 CFD, 1-2 MFD, 3-4 split lines, 5-6 as 1-2 in CTAs of 256 threads (FP64)
+int fac_variant(int method, int N, size_t esz);
+int fac_variant_method(int v);
+constexpr int kFacVariants = 7;
 int fac_lines_per_cta(int method, int N, size_t esz);
 size_t fac_stage_bytes(int method, int N, int nl, size_t esz);  // shared memory of one stage
 int fac_stages_for(size_t stage_bytes, size_t esz, int method);  // groups in flight that fit: 3, 2, 1 or 0

@@ -3,6 +3,10 @@
 Tolerances are the path's own (FP64 max |difference| <= 1e-12 x max |field|, FP32 relative L2 <= 1e-4), for
 the few steps taken here; where two GPU paths are compared they are derived beside the test.
 """
+import os
+import shutil
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -12,6 +16,8 @@ from paper_2006_07583_gb300 import workloads as wl
 pytestmark = pytest.mark.gpu
 
 CFD, MFD = wl.CFD, wl.MFD
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
 
 
 @pytest.fixture(scope="module")
@@ -64,3 +70,22 @@ def test_line_lengths_at_path_changes(adi, method, n, fp64):
     G = sim.read()
     sim.close()
     _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, 3, source=src), fp64)
+
+
+def test_fp64_reciprocal():
+    """The FP64 line kernels' reciprocal (fac_rcp) against CUDA's correctly rounded 1 / x: at most one unit in the
+    last place off, for 2^20 values over the exponents that pivots and determinants take."""
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    out = os.path.join(HERE, "_build")  # git-ignored
+    os.makedirs(out, exist_ok=True)
+    exe = os.path.join(out, "fac_rcp_check")
+    r = subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I" + os.path.join(ROOT, "include"),
+                        "-o", exe, os.path.join(HERE, "fac_rcp_check.cu")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "worst" in r.stdout, r.stdout[-500:] + r.stderr[-500:]
+    assert int(r.stdout.split()[1]) <= 1, r.stdout
