@@ -1061,13 +1061,16 @@ template <typename T>
 int run_precompute(adi_sim *s) {
     const LineDesc<T> *all = (const LineDesc<T> *)s->cold_all.p;
     int n = s->nlines[0] + s->nlines[1];
-    cudaError_t e = cudaMemsetAsync(s->status.p, 0, sizeof(int), s->stream);
-    if (e == cudaSuccess) e = launch_precompute<T>(all, n, (T *)s->tab.p, (int *)s->status.p, s->stream);
-    int st = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&st, s->status.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_status(e);
-    if (st) return ADI_ESINGULAR;
+    cudaError_t e = cudaSuccess;
+    if (s->solver != ADI_SOLVER_FACTORED) {  // the end tables of the other solvers
+        e = cudaMemsetAsync(s->status.p, 0, sizeof(int), s->stream);
+        if (e == cudaSuccess) e = launch_precompute<T>(all, n, (T *)s->tab.p, (int *)s->status.p, s->stream);
+        int st = 0;
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&st, s->status.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_status(e);
+        if (st) return ADI_ESINGULAR;
+    }
     if (s->solver == ADI_SOLVER_CHUNKED) {
         e = launch_precompute_sep<T>(all, n, s->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -1078,7 +1081,10 @@ int run_precompute(adi_sim *s) {
         if (rc) return rc;
         int out[2] = {0, 0};
         e = cudaMemsetAsync(s->status.p, 0, 2 * sizeof(int), s->stream);
-        if (e == cudaSuccess) e = launch_fac_precompute<T>(all, n, (double *)ws.p, (int *)s->status.p, s->stream);
+        for (int dir = 0, at = 0; dir < 2; at += s->nlines[dir++])
+            if (e == cudaSuccess)
+                e = launch_fac_precompute<T>(all + at, s->nlines[dir], s->g.method, dir == 0 ? s->g.nx : s->g.ny,
+                                             (double *)ws.p + (size_t)at * fac_ws_doubles(), (int *)s->status.p, s->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(out, s->status.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
         dev_free(ws);

@@ -51,7 +51,7 @@ constexpr int kFacMaxT = kFacWorkers;         // chunks (threads) per line at mo
 constexpr size_t kFacSmemLimit = 227 * 1024;  // shared memory per CTA
 constexpr size_t kFacStaticBase = 2048;       // reserve for the kernel's other static shared memory
 constexpr int kFacMaxStages = 3;              // staged groups in flight per CTA at most
-constexpr int kFacWs = 1024;                  // FP64 workspace of the precompute, per line
+constexpr int kFacWs = 1024;                  // FP64 workspace of one end's elimination
 // Static shared memory of the kernel for element size esz and block size bs, an upper bound:
 // the scan buffers (chunk offsets, two arrays for FP32, one for FP64) plus the rest (checked
 // against the compiled kernel before its first launch).
@@ -210,7 +210,7 @@ int fac_variant(int method, int N, size_t esz) {
     return fac_narrow(method, fac_geom(method, N).T, esz) ? v + 4 : v;
 }
 int fac_variant_method(int v) { return v == 0 || v == 3 ? kCFD : kMFD; }
-size_t fac_ws_doubles() { return kFacWs; }
+size_t fac_ws_doubles() { return 18; }
 static unsigned fac_tdiv(int T) {
     return T > 1 ? (unsigned)(((1ull << 32) + (unsigned long long)T - 1) / (unsigned long long)T) : 0u;
 }
@@ -301,46 +301,20 @@ struct FacEnd {
     static constexpr int HZ = BS * 2 * W, DZ = HZ + HMAX * Z, DB = DZ + (BS == 3 ? (HMAX + 2) * Z : 0);
 };
 
-// ---------------------------------------------------------------------------------------
-// Middle block b (A to block b-1, B, C to block b+1) in precision R from alpha values
-// al(k) along the pressure line.
-// ---------------------------------------------------------------------------------------
-template <typename R, int BS, typename AL>
-__device__ __forceinline__ void fac_block(const FacGeom &g, double beta, double ih, int b, AL al,
-                                          R (&A)[BS][BS], R (&B)[BS][BS], R (&C)[BS][BS]) {
-    if constexpr (BS == 2) {
-        const int j = g.first + b;
-        const R tb = R(3) * (R)beta * (R)ih;
-        A[0][0] = R(1); A[0][1] = -tb; A[1][0] = -R(3) * (R)ih * (R)al(j - 1); A[1][1] = R(1);
-        B[0][0] = R(4); B[0][1] = R(0); B[1][0] = R(0); B[1][1] = R(4);
-        C[0][0] = R(1); C[0][1] = tb; C[1][0] = R(3) * (R)ih * (R)al(j + 1); C[1][1] = R(1);
-    } else {
-        const int cb = g.first + 3 * b;
-        const R bh2 = (R)(beta * ih * ih);
-#pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            const R sc = (R)al(cb + m) * bh2;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                A[m][q] = (q >= m) ? -sc * (R)mim_DG(q - m) : R(0);
-                B[m][q] = (q == m ? R(1) : R(0)) - sc * (R)mim_DG(q - m + 3);
-                C[m][q] = (q <= m) ? -sc * (R)mim_DG(q - m + 6) : R(0);
-            }
-        }
-    }
+// Reciprocals.  FP32: the hardware approximation (relative error below 2^-22).
+__device__ __forceinline__ float fac_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
-
-template <typename R, int BS>
-__device__ __forceinline__ void f_mm(const R (&X)[BS][BS], const R (&Y)[BS][BS], R (&Z)[BS][BS]) {
-#pragma unroll
-    for (int i = 0; i < BS; ++i)
-#pragma unroll
-        for (int j = 0; j < BS; ++j) {
-            R acc = R(0);
-#pragma unroll
-            for (int k = 0; k < BS; ++k) acc += X[i][k] * Y[k][j];
-            Z[i][j] = acc;
-        }
+// FP64: the hardware approximation r0 (about 20 bits) and one step of Householder's cubic iteration, r0 (1 + e
+// + e^2) with e = 1 - x r0: three FMAs against a division's ten or so operations on the FP64 pipe that bounds these kernels;
+// the error left is e^3 = 2^-60 and one rounding (measured against 1 / x: at most 1 ulp).
+__device__ __forceinline__ double fac_rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -391,10 +365,58 @@ __device__ bool fac_rhs_coeffs(const LineDesc<TS> &d, int i, int op, int ov, int
     return ok;
 }
 
-// Dense elimination of one end region (end 0: head, 1: tail) into its table; dB of the end
-// (bs x bs, row-major) is also returned in dBo.  False if the region is singular.
+// Gauss-Jordan inverse with partial pivoting of an n x n matrix (n <= 13, destroyed) by one warp: lane
+// j holds column j of [A | R] (R starts as the identity); the same operations in the same order as
+// small_inverse.
+__device__ inline bool warp_inverse(double *A, int n, double *R, int lane) {
+    double scale = 0.0;
+    for (int i = lane; i < n * n; i += 32) {
+        R[i] = (i / n == i % n) ? 1.0 : 0.0;
+        scale = fmax(scale, fabs(A[i]));
+    }
+    for (int o = 16; o > 0; o >>= 1) scale = fmax(scale, __shfl_xor_sync(0xffffffffu, scale, o));
+    __syncwarp();
+    double *col = lane < n ? A + lane : R + (lane - n);  // this lane's column, stride n
+    const bool mine = lane < 2 * n;
+    for (int c = 0; c < n; ++c) {
+        double f[13];
+        int p = c;
+        double best = fabs(A[c * n + c]);
+#pragma unroll
+        for (int i = 0; i < 13; ++i) {
+            f[i] = i < n ? A[i * n + c] : 0.0;
+            if (i > c && i < n && fabs(f[i]) > best) { best = fabs(f[i]); p = i; }
+        }
+        if (!(best > 1e-13 * scale)) return false;  // uniform over the warp
+        __syncwarp();  // column c has been read
+        if (mine) {
+            const double ap = col[p * n], ac = col[c * n];
+            double fp = 0.0, fc = 0.0;
+#pragma unroll
+            for (int i = 0; i < 13; ++i) {
+                if (i == p) fp = f[i];
+                if (i == c) fc = f[i];
+            }
+            const double row = ap * (1.0 / fp);
+            if (p != c) col[p * n] = ac;
+            col[c * n] = row;
+#pragma unroll
+            for (int i = 0; i < 13; ++i) {
+                if (i >= n || i == c) continue;
+                const double fi = i == p ? fc : f[i];  // rows p and c are swapped
+                if (fi != 0.0) col[i * n] -= fi * row;
+            }
+        }
+        __syncwarp();
+    }
+    return true;
+}
+
+// Dense elimination of one end region (end 0: head, 1: tail) into its table by one warp, in its
+// shared workspace ws (kFacWs doubles); dB of the end (bs x bs, row-major) is also returned in FP64
+// in dBo (global memory).  False if the region is singular.
 template <typename TS>
-__device__ bool fac_end(const LineDesc<TS> &d, const FacGeom &g, int end, double *ws, TS *et, double *dBo) {
+__device__ bool fac_end(const LineDesc<TS> &d, const FacGeom &g, int end, double *ws, TS *et, double *dBo, int lane) {
     const int N = d.N, bs = g.bs, W = g.win, Z = fac_zlen(g);
     const int nunk = d.method == kCFD ? 2 * N : N;
     const int m = end == 0 ? g.hu : g.tu;
@@ -404,64 +426,61 @@ __device__ bool fac_end(const LineDesc<TS> &d, const FacGeom &g, int end, double
     const int op = end == 0 ? 0 : pl + 1 - W, ov = end == 0 ? 0 : N + 1 - W;
     double *H = ws, *Hi = H + m * m, *E = Hi + m * m, *F = E + m * bs, *Rm = F + bs * m;
     double *HiE = Rm + m * 2 * W, *K = HiE + m * bs, *HZ = K + bs * m;
-    for (int i = 0; i < m; ++i)
-        for (int j = 0; j < m; ++j) H[i * m + j] = line_entry(d, r0 + i, r0 + j);
-    for (int i = 0; i < m; ++i)
-        for (int j = 0; j < bs; ++j) E[i * bs + j] = line_entry(d, r0 + i, j0 + j);
-    for (int i = 0; i < bs; ++i)
-        for (int j = 0; j < m; ++j) F[i * m + j] = line_entry(d, j0 + i, r0 + j);
-    if (!small_inverse(H, m, Hi)) return false;
-    for (int i = 0; i < m; ++i)
-        for (int j = 0; j < bs; ++j) {
-            double acc = 0.0;
-            for (int k = 0; k < m; ++k) acc += Hi[i * m + k] * E[k * bs + j];
-            HiE[i * bs + j] = acc;
-        }
-    for (int i = 0; i < bs; ++i)
-        for (int j = 0; j < m; ++j) {
-            double acc = 0.0;
-            for (int k = 0; k < m; ++k) acc += F[i * m + k] * Hi[k * m + j];
-            K[i * m + j] = acc;
-        }
-    for (int i = 0; i < bs; ++i)
-        for (int j = 0; j < bs; ++j) {
-            double acc = 0.0;
-            for (int k = 0; k < m; ++k) acc += F[i * m + k] * HiE[k * bs + j];
-            dBo[i * bs + j] = acc;
-        }
+    for (int i = lane; i < m * m; i += 32) H[i] = line_entry(d, r0 + i / m, r0 + i % m);
+    for (int i = lane; i < m * bs; i += 32) E[i] = line_entry(d, r0 + i / bs, j0 + i % bs);
+    for (int i = lane; i < bs * m; i += 32) F[i] = line_entry(d, j0 + i / m, r0 + i % m);
     bool ok = true;
-    for (int q = 0; q < m; ++q) ok = fac_rhs_coeffs(d, r0 + q, op, ov, W, Rm + q * 2 * W, Rm + q * 2 * W + W) && ok;
+    if (lane < m) ok = fac_rhs_coeffs(d, r0 + lane, op, ov, W, Rm + lane * 2 * W, Rm + lane * 2 * W + W);
+    ok = __all_sync(0xffffffffu, ok);
+    __syncwarp();
+    if (!warp_inverse(H, m, Hi, lane)) return false;
+    for (int i = lane; i < m * bs; i += 32) {
+        double acc = 0.0;
+        for (int k = 0; k < m; ++k) acc += Hi[(i / bs) * m + k] * E[k * bs + i % bs];
+        HiE[i] = acc;
+    }
+    for (int i = lane; i < bs * m; i += 32) {
+        double acc = 0.0;
+        for (int k = 0; k < m; ++k) acc += F[(i / m) * m + k] * Hi[k * m + i % m];
+        K[i] = acc;
+    }
     const double nan = __longlong_as_double(0x7ff8000000000000ULL);
     const int e_stride = fac_e_stride(g);
-    for (int i = 0; i < e_stride; ++i) et[i] = (TS)0;
-    // KZ = -K R
-    for (int p = 0; p < bs; ++p)
-        for (int k = 0; k < 2 * W; ++k) {
-            double acc = 0.0;
-            for (int q = 0; q < m; ++q) acc -= K[p * m + q] * Rm[q * 2 * W + k];
-            et[p * 2 * W + k] = (TS)(ok ? acc : nan);
-        }
-    // HZ = [Hinv R | -Hinv E]
-    for (int q = 0; q < m; ++q) {
-        for (int k = 0; k < 2 * W; ++k) {
-            double acc = 0.0;
-            for (int q2 = 0; q2 < m; ++q2) acc += Hi[q * m + q2] * Rm[q2 * 2 * W + k];
-            HZ[q * Z + k] = acc;
-        }
-        for (int b = 0; b < bs; ++b) HZ[q * Z + 2 * W + b] = -HiE[q * bs + b];
-        for (int k = 0; k < Z; ++k) et[fac_e_hz(g) + q * Z + k] = (TS)(ok ? HZ[q * Z + k] : nan);
+    for (int i = lane; i < e_stride; i += 32) et[i] = (TS)0;
+    __syncwarp();
+    for (int i = lane; i < bs * bs; i += 32) {
+        double acc = 0.0;
+        for (int k = 0; k < m; ++k) acc += F[(i / bs) * m + k] * HiE[k * bs + i % bs];
+        dBo[i] = acc;
+        et[fac_e_db(g) + i] = (TS)acc;
     }
-    for (int i = 0; i < bs * bs; ++i) et[fac_e_db(g) + i] = (TS)dBo[i];
+    // KZ = -K R
+    for (int i = lane; i < bs * 2 * W; i += 32) {
+        double acc = 0.0;
+        for (int q = 0; q < m; ++q) acc -= K[(i / (2 * W)) * m + q] * Rm[q * 2 * W + i % (2 * W)];
+        et[i] = (TS)(ok ? acc : nan);
+    }
+    // HZ = [Hinv R | -Hinv E]
+    for (int i = lane; i < m * Z; i += 32) {
+        const int q = i / Z, k = i % Z;
+        double acc = 0.0;
+        if (k < 2 * W) {
+            for (int q2 = 0; q2 < m; ++q2) acc += Hi[q * m + q2] * Rm[q2 * 2 * W + k];
+        } else {
+            acc = -HiE[q * bs + k - 2 * W];
+        }
+        HZ[i] = acc;
+        et[fac_e_hz(g) + i] = (TS)(ok ? acc : nan);
+    }
+    __syncwarp();
     if (d.method != kMFD) return true;
-    // MFD: h (G u)_j at the end's velocity nodes as maps of z (cells through HZ)
+    // MFD: h (G u)_j at the end's velocity nodes as maps of z (cells through HZ), lane = entry of z
     const int qb = g.first + 3 * (g.nb - 1);  // first cell of the last middle block
     const int jlo = end == 0 ? 0 : qb + 1, jhi = end == 0 ? g.hu + 1 : N;
     const int cell_lo = end == 0 ? 1 : N - g.tu + 1;  // first eliminated cell
     const int adj = end == 0 ? g.hu + 1 : qb;         // first cell of the adjacent block
     for (int j = jlo; j <= jhi; ++j) {
-        double *row = HZ + m * Z;  // scratch row after HZ
-        for (int k = 0; k < Z; ++k) row[k] = 0.0;
-        double gw[8];
+        double gw[8], row = 0.0;
         int g0;
         const int ng = mfd_G_row(N, j, &g0, gw);
         bool rok = ok;
@@ -469,140 +488,354 @@ __device__ bool fac_end(const LineDesc<TS> &d, const FacGeom &g, int end, double
             const int cc = g0 + t;
             if (cc == 0 || cc == N + 1) {
                 const int wi = cc - op;
-                if (wi < 0 || wi >= W) rok = false; else row[wi] += gw[t];
+                if (wi < 0 || wi >= W) rok = false; else if (lane == wi) row += gw[t];
             } else if (cc >= cell_lo && cc < cell_lo + m) {
-                for (int k = 0; k < Z; ++k) row[k] += gw[t] * HZ[(cc - cell_lo) * Z + k];
+                if (lane < Z) row += gw[t] * HZ[(cc - cell_lo) * Z + lane];
             } else if (cc >= adj && cc < adj + bs) {
-                row[2 * W + cc - adj] += gw[t];
+                if (lane == 2 * W + cc - adj) row += gw[t];
             } else {
                 rok = false;
             }
         }
-        for (int k = 0; k < Z; ++k) et[fac_e_dz(g) + (j - jlo) * Z + k] = (TS)(rok ? row[k] : nan);
+        if (lane < Z) et[fac_e_dz(g) + (j - jlo) * Z + lane] = (TS)(rok ? row : nan);
     }
     return true;
 }
 
-template <typename TS, int BS>
-__device__ bool fac_chunks_fp64(const LineDesc<TS> &d, const FacGeom &g, const double *dBh, const double *dBt, TS *rec) {
-    constexpr int B2 = BS * BS;
+// The end tables: one warp per (line, end).  With one thread per line and its workspace in global memory
+// the eliminations were a chain of scattered accesses and most of the 15.4 ms that the records of a
+// 4096 x 4096 grid took.
+constexpr int kFacEndWarps = 4;
+template <typename TS>
+__global__ void __launch_bounds__(32 * kFacEndWarps) fac_ends_kernel(const LineDesc<TS> *__restrict__ descs, int nlines,
+                                                                     double *dB, int *status) {
+    __shared__ double ws[kFacEndWarps][kFacWs];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int job = blockIdx.x * kFacEndWarps + warp, line = job >> 1, end = job & 1;
+    if (line >= nlines) return;
+    const LineDesc<TS> &d = descs[line];
+    const FacGeom g = fac_geom(d.method, d.N);
+    TS *et = d.sep + fac_chunk_elems(g) + end * fac_e_stride(g);
+    if (!fac_end(d, g, end, ws[warp], et, dB + (size_t)job * 9, lane) && lane == 0) atomicExch(status, 1);
+}
+
+// Block LU of the middle blocks [b0, b1) of a line (whole chunks), from G = G_{b0-1}; on return G =
+// G_{b1-1}.  STORE: write the chunks' records.  False if a block is singular.  The FP64 pipe bounds it (one
+// warp instruction in 19 cycles an SM), so the products visit the coupling blocks' nonzero entries only and none
+// of their units (the blocks as in fac_group); each sum keeps the order and the roundings of the full block products,
+// so that leaving entries out changes no bit.
+__device__ __forceinline__ bool fac_pivot_ok(double det) { return fabs(det) > 0.0 && isfinite(det); }
+
+template <typename TS, bool STORE>
+__device__ bool fac_run(const LineDesc<TS> &d, const FacGeom &g, const double *dBh, const double *dBt, TS *rec, int b0,
+                        int b1, double (&G)[2][2]) {
     TS *recS = rec, *recF = rec + fac_part(g), *recH = rec + (size_t)2 * fac_part(g);
-    auto al = [&](int k) -> double { return (double)d.alpha[(long long)k * d.sp]; };
-    double G[BS][BS], Fp[BS][BS], Hp[BS][BS];
-    for (int p = 0; p < BS; ++p)
-        for (int q = 0; q < BS; ++q) { G[p][q] = 0.0; Fp[p][q] = Hp[p][q] = (p == q) ? 1.0 : 0.0; }
-    for (int b = 0; b < g.nb; ++b) {
-        double A[BS][BS], B[BS][BS], C[BS][BS];
-        fac_block<double, BS>(g, d.beta, d.inv_h, b, al, A, B, C);
-        if (b == 0)
-            for (int p = 0; p < BS; ++p)
-                for (int q = 0; q < BS; ++q) { B[p][q] -= dBh[p * BS + q]; A[p][q] = 0.0; }
-        if (b == g.nb - 1)
-            for (int p = 0; p < BS; ++p)
-                for (int q = 0; q < BS; ++q) { B[p][q] -= dBt[p * BS + q]; C[p][q] = 0.0; }
-        double S[BS][BS], Si[BS][BS], Gn[BS][BS], T1[BS][BS];
-        for (int p = 0; p < BS; ++p)
-            for (int q = 0; q < BS; ++q) {
-                double acc = B[p][q];
-                for (int k = 0; k < BS; ++k) acc -= A[p][k] * G[k][q];
-                S[p][q] = acc;
-            }
-        double det = BS == 2 ? S[0][0] * S[1][1] - S[0][1] * S[1][0]
-                             : S[0][0] * (S[1][1] * S[2][2] - S[1][2] * S[2][1]) -
-                                   S[0][1] * (S[1][0] * S[2][2] - S[1][2] * S[2][0]) +
-                                   S[0][2] * (S[1][0] * S[2][1] - S[1][1] * S[2][0]);
-        if (!(fabs(det) > 0.0) || !isfinite(det)) return false;
-        mat_inv<double, BS>(S, Si);
-        f_mm<double, BS>(Si, C, Gn);
-        const int c = b / g.mm, i = b % g.mm;
-        if (i == 0) {
-            for (int p = 0; p < BS; ++p)
-                for (int q = 0; q < BS; ++q) {
-                    recS[(size_t)c * B2 + p * BS + q] = (TS)S[p][q];
-                    Fp[p][q] = Hp[p][q] = (p == q) ? 1.0 : 0.0;
-                }
+    const double tb = 3.0 * d.beta * d.inv_h, c3 = 3.0 * d.inv_h;
+    const TS *__restrict__ al = d.alpha;
+    const long long sp = d.sp;
+    const int j0 = g.first;
+    double am = c3 * (double)al[(j0 + b0 - 1) * sp], a0 = c3 * (double)al[(j0 + b0) * sp];
+    double F[2][2] = {}, H[2][2] = {};
+    int c = b0 / g.mm, i = 0;
+    for (int b = b0; b < b1; ++b) {
+        const double ap = c3 * (double)al[(j0 + b + 1) * sp];
+        const bool first = b == 0, last = b == g.nb - 1;
+        double S[2][2] = {{4.0, 0.0}, {0.0, 4.0}};
+        if (first)
+            for (int p = 0; p < 2; ++p)
+                for (int q = 0; q < 2; ++q) S[p][q] -= dBh[p * 2 + q];
+        if (last)
+            for (int p = 0; p < 2; ++p)
+                for (int q = 0; q < 2; ++q) S[p][q] -= dBt[p * 2 + q];
+        if (!first) {  // S -= A G, A = [[1, -tb], [-am, 1]]
+            S[0][0] = fma_rn(tb, G[1][0], __dsub_rn(S[0][0], G[0][0]));
+            S[0][1] = fma_rn(tb, G[1][1], __dsub_rn(S[0][1], G[0][1]));
+            S[1][0] = __dsub_rn(fma_rn(am, G[0][0], S[1][0]), G[1][0]);
+            S[1][1] = __dsub_rn(fma_rn(am, G[0][1], S[1][1]), G[1][1]);
         }
-        // Fp <- (-Si A) Fp ;  Hp <- Hp (-Gn)
-        double Fb[BS][BS];
-        f_mm<double, BS>(Si, A, Fb);
-        f_mm<double, BS>(Fb, Fp, T1);
-        for (int p = 0; p < BS; ++p)
-            for (int q = 0; q < BS; ++q) Fp[p][q] = -T1[p][q];
-        f_mm<double, BS>(Hp, Gn, T1);
-        for (int p = 0; p < BS; ++p)
-            for (int q = 0; q < BS; ++q) Hp[p][q] = -T1[p][q];
-        if (i == g.mm - 1)
-            for (int p = 0; p < BS; ++p)
-                for (int q = 0; q < BS; ++q) {
-                    recF[(size_t)c * B2 + p * BS + q] = (TS)Fp[p][q];
-                    recH[(size_t)c * B2 + p * BS + q] = (TS)Hp[p][q];
-                }
-        for (int p = 0; p < BS; ++p)
-            for (int q = 0; q < BS; ++q) G[p][q] = Gn[p][q];
+        const double det = S[0][0] * S[1][1] - S[0][1] * S[1][0];
+        if (!fac_pivot_ok(det)) return false;
+        double R[2][2];
+        mat_inv<double, 2>(S, R);
+        // G = R C, C = [[1, tb], [ap, 1]]
+        G[0][0] = last ? 0.0 : fma_rn(R[0][1], ap, R[0][0]);
+        G[0][1] = last ? 0.0 : __dadd_rn(mul_rn(R[0][0], tb), R[0][1]);
+        G[1][0] = last ? 0.0 : fma_rn(R[1][1], ap, R[1][0]);
+        G[1][1] = last ? 0.0 : __dadd_rn(mul_rn(R[1][0], tb), R[1][1]);
+        if constexpr (STORE) {
+            // E = -R A
+            double E[2][2] = {{-fma_rn(R[0][1], -am, R[0][0]), -__dadd_rn(mul_rn(R[0][0], -tb), R[0][1])},
+                              {-fma_rn(R[1][1], -am, R[1][0]), -__dadd_rn(mul_rn(R[1][0], -tb), R[1][1])}};
+            if (first) E[0][0] = E[0][1] = E[1][0] = E[1][1] = 0.0;
+            if (i == 0) {
+                for (int p = 0; p < 2; ++p)
+                    for (int q = 0; q < 2; ++q) {
+                        recS[(size_t)c * 4 + p * 2 + q] = (TS)S[p][q];
+                        F[p][q] = E[p][q];
+                        H[p][q] = -G[p][q];
+                    }
+            } else {
+                double f[2][2], h[2][2];
+                for (int p = 0; p < 2; ++p)
+                    for (int q = 0; q < 2; ++q) {
+                        f[p][q] = fma_rn(E[p][1], F[1][q], mul_rn(E[p][0], F[0][q]));
+                        h[p][q] = -fma_rn(H[p][1], G[1][q], mul_rn(H[p][0], G[0][q]));
+                    }
+                for (int p = 0; p < 2; ++p)
+                    for (int q = 0; q < 2; ++q) { F[p][q] = f[p][q]; H[p][q] = h[p][q]; }
+            }
+            if (++i == g.mm) {
+                for (int p = 0; p < 2; ++p)
+                    for (int q = 0; q < 2; ++q) {
+                        recF[(size_t)c * 4 + p * 2 + q] = (TS)F[p][q];
+                        recH[(size_t)c * 4 + p * 2 + q] = (TS)H[p][q];
+                    }
+                i = 0;
+                ++c;
+            }
+        }
+        am = a0;
+        a0 = ap;
     }
     return true;
 }
 
-// Reach of the windowed scans (see the header): the largest, over the chunks, of the number
-// of consecutive stored transfers (forward: F_e F_{e-1} ..., backward: H_s H_{s+1} ...) whose
-// product first has infinity norm at most tau, or that reaches the end of the line; at most
-// kFacMaxReach + 1 (which selects the full scan).
-template <typename TS, int BS>
-__device__ int fac_reach(const TS *maps, int tact, double tau, bool forward) {
-    constexpr int B2 = BS * BS;
-    int reach = 0;
-    for (int e = 0; e < tact - 1; ++e) {
-        const int first = forward ? e : e + 1;  // chunk whose transfer the window starts with
-        double P[BS][BS];
-        for (int p = 0; p < BS; ++p)
-            for (int q = 0; q < BS; ++q) P[p][q] = p == q ? 1.0 : 0.0;
-        int r = 0;
-        for (;;) {
-            const int k = forward ? first - r : first + r;
-            double M[BS][BS], T1[BS][BS];
-            for (int p = 0; p < BS; ++p)
-                for (int q = 0; q < BS; ++q) M[p][q] = (double)maps[(size_t)k * B2 + p * BS + q];
-            f_mm<double, BS>(P, M, T1);
-            double nrm = 0.0;
-            for (int p = 0; p < BS; ++p) {
-                double rs = 0.0;
-                for (int q = 0; q < BS; ++q) { P[p][q] = T1[p][q]; rs += fabs(T1[p][q]); }
-                nrm = fmax(nrm, rs);
+template <typename TS, bool STORE>
+__device__ bool fac_run(const LineDesc<TS> &d, const FacGeom &g, const double *dBh, const double *dBt, TS *rec, int b0,
+                        int b1, double (&G)[3][3]) {
+    TS *recS = rec, *recF = rec + fac_part(g), *recH = rec + (size_t)2 * fac_part(g);
+    const double bh2 = d.beta * d.inv_h * d.inv_h;
+    const TS *__restrict__ al = d.alpha;
+    const long long sp = d.sp;
+    double F[3][3] = {}, H[3][3] = {};
+    int c = b0 / g.mm, i = 0;
+    for (int b = b0; b < b1; ++b) {
+        const bool first = b == 0, last = b == g.nb - 1;
+        const int cb = g.first + 3 * b;
+        double sc[3], S[3][3], R[3][3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) sc[m] = (double)al[(cb + m) * sp] * bh2;
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) S[p][q] = fma_rn(-sc[p], mim_DG(q - p + 3), p == q ? 1.0 : 0.0);
+        if (first)
+            for (int p = 0; p < 3; ++p)
+                for (int q = 0; q < 3; ++q) S[p][q] -= dBh[p * 3 + q];
+        if (last)
+            for (int p = 0; p < 3; ++p)
+                for (int q = 0; q < 3; ++q) S[p][q] -= dBt[p * 3 + q];
+        if (!first)  // S -= A G, A[p][k] = -s_p K_(3 + p - k) for k >= p
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+#pragma unroll
+                for (int k = p; k < 3; ++k) {
+                    const double ak = mul_rn(sc[p], mim_DG(k - p));
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) S[p][q] = fma_rn(ak, G[k][q], S[p][q]);
+                }
+        const double det = S[0][0] * (S[1][1] * S[2][2] - S[1][2] * S[2][1]) - S[0][1] * (S[1][0] * S[2][2] - S[1][2] * S[2][0]) +
+                           S[0][2] * (S[1][0] * S[2][1] - S[1][1] * S[2][0]);
+        if (!fac_pivot_ok(det)) return false;
+        mat_inv<double, 3>(S, R);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {  // G = R C, C[k][q] = -s_k K_(3 + q - k) for q <= k
+            double t[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int k = q; k < 3; ++k) {
+                const double ck = -mul_rn(sc[k], mim_DG(q - k + 6));
+#pragma unroll
+                for (int p = 0; p < 3; ++p) t[p] = fma_rn(R[p][k], ck, t[p]);
             }
-            ++r;
-            const bool at_end = forward ? (k == 0) : (k == tact - 1);
-            if (nrm <= tau || at_end || r > kFacMaxReach) break;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) G[p][q] = last ? 0.0 : t[p];
         }
+        if constexpr (STORE) {
+            double E[3][3];  // -R A
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                double t[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+                for (int k = 0; k <= q; ++k) {
+                    const double ak = mul_rn(sc[k], mim_DG(q - k));
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) t[p] = fma_rn(R[p][k], ak, t[p]);
+                }
+#pragma unroll
+                for (int p = 0; p < 3; ++p) E[p][q] = first ? 0.0 : t[p];
+            }
+            if (i == 0) {
+                for (int p = 0; p < 3; ++p)
+                    for (int q = 0; q < 3; ++q) {
+                        recS[(size_t)c * 9 + p * 3 + q] = (TS)S[p][q];
+                        F[p][q] = E[p][q];
+                        H[p][q] = -G[p][q];
+                    }
+            } else {
+                double f[3][3], h[3][3];
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        f[p][q] = fma_rn(E[p][2], F[2][q], fma_rn(E[p][1], F[1][q], mul_rn(E[p][0], F[0][q])));
+                        h[p][q] = -fma_rn(H[p][2], G[2][q], fma_rn(H[p][1], G[1][q], mul_rn(H[p][0], G[0][q])));
+                    }
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) { F[p][q] = f[p][q]; H[p][q] = h[p][q]; }
+            }
+            if (++i == g.mm) {
+                for (int p = 0; p < 3; ++p)
+                    for (int q = 0; q < 3; ++q) {
+                        recF[(size_t)c * 9 + p * 3 + q] = (TS)F[p][q];
+                        recH[(size_t)c * 9 + p * 3 + q] = (TS)H[p][q];
+                    }
+                i = 0;
+                ++c;
+            }
+        }
+    }
+    return true;
+}
+
+// Reach of the windowed scans over the windows that start at the chunks [e0, e1) (see the header): the
+// largest number of consecutive stored transfers (forward: F_e F_{e-1} ..., backward: H_s H_{s+1} ...)
+// whose product first has infinity norm at most tau, or that reaches the end of the line; at most
+// kFacMaxReach + 1 (which selects the full scan).
+// A window's products are formed in FP32, and in FP64 only where a norm comes so near tau that FP32's rounding could
+// decide (the FP64 pipe is what the records wait for).
+template <typename TS, int BS, typename R>
+__device__ int fac_window(const TS *maps, int tact, double tau, bool forward, int first, bool &unsure) {
+    constexpr int B2 = BS * BS;
+    R P[BS][BS];
+#pragma unroll
+    for (int p = 0; p < BS; ++p)
+#pragma unroll
+        for (int q = 0; q < BS; ++q) P[p][q] = p == q ? R(1) : R(0);
+    unsure = false;
+    const R lo = (R)(tau * 0.999), hi = (R)(tau * 1.001);
+    for (int r = 0;;) {
+        const int k = forward ? first - r : first + r;
+        R M[BS][BS], T1[BS][BS], nrm = R(0);
+#pragma unroll
+        for (int p = 0; p < BS; ++p)
+#pragma unroll
+            for (int q = 0; q < BS; ++q) M[p][q] = (R)maps[(size_t)k * B2 + p * BS + q];
+#pragma unroll
+        for (int p = 0; p < BS; ++p) {
+            R rs = R(0);
+#pragma unroll
+            for (int q = 0; q < BS; ++q) {
+                R t = R(0);
+#pragma unroll
+                for (int m = 0; m < BS; ++m) t += P[p][m] * M[m][q];
+                T1[p][q] = t;
+                rs += t < R(0) ? -t : t;
+            }
+            nrm = rs > nrm ? rs : nrm;
+        }
+#pragma unroll
+        for (int p = 0; p < BS; ++p)
+#pragma unroll
+            for (int q = 0; q < BS; ++q) P[p][q] = T1[p][q];
+        ++r;
+        const bool at_end = forward ? (k == 0) : (k == tact - 1);
+        if (nrm > lo && nrm < hi) unsure = true;
+        if (nrm <= (R)tau || at_end || r > kFacMaxReach) return r;
+    }
+}
+template <typename TS, int BS>
+__device__ int fac_reach(const TS *maps, int tact, double tau, bool forward, int e0, int e1) {
+    int reach = 0;
+    for (int e = e0; e < e1 && e < tact - 1 && reach <= kFacMaxReach; ++e) {
+        const int first = forward ? e : e + 1;  // chunk whose transfer the window starts with
+        bool unsure;
+        int r = fac_window<TS, BS, float>(maps, tact, tau, forward, first, unsure);
+        if (unsure) r = fac_window<TS, BS, double>(maps, tact, tau, forward, first, unsure);
         reach = max(reach, r);
-        if (reach > kFacMaxReach) break;
     }
     return reach;
 }
 
-template <typename TS>
-__global__ void fac_precompute_kernel(const LineDesc<TS> *__restrict__ descs, int nlines, double *ws,
-                                      int *status) {
-    const int line = blockIdx.x * blockDim.x + threadIdx.x;
-    if (line >= nlines) return;
-    const LineDesc<TS> d = descs[line];
-    const FacGeom g = fac_geom(d.method, d.N);
-    double *w = ws + (size_t)line * kFacWs;
+// The chunk records of the lines of one direction (all of N cells): segs threads per line, each the
+// block LU of a run of whole chunks.  A run inside the line starts fac_warm blocks earlier from G = 0:
+// the recursion forgets its start by the square of what the chunk transfers decay (on the seismic grids
+// 0.4 a CFD block, 4e-26 over 64, and 0.01 an MFD block, 1e-32 over 16: the same bits as from the head).  Whether it did is checked, not assumed: the G it reached at
+// its first block must agree with the G of the run before to kFacWarmTol of its size, else one thread
+// does the line again from its head (weakly decaying lines, as with very large time steps).
+constexpr int kFacRecThreads = 128;
+__host__ __device__ inline int fac_warm(int method) { return method == kCFD ? 64 : 16; }
+constexpr double kFacWarmTol = 1e-15;
+template <typename TS, int BS>
+__device__ void fac_records(const LineDesc<TS> &d, const FacGeom &g, const double *dB, int segs, int seg, bool mine,
+                            double (*gs)[9], double (*ge)[9], int *bad, int *status) {
+    const int c0 = (int)((long long)g.tact * seg / segs), c1 = (int)((long long)g.tact * (seg + 1) / segs);
     TS *rec = d.sep;
-    TS *eH = rec + fac_chunk_elems(g), *eT = eH + fac_e_stride(g);
-    double dBh[9], dBt[9];
-    bool ok = fac_end(d, g, 0, w, eH, dBh) && fac_end(d, g, 1, w, eT, dBt);
-    if (ok) ok = d.method == kCFD ? fac_chunks_fp64<TS, 2>(d, g, dBh, dBt, rec)
-                                  : fac_chunks_fp64<TS, 3>(d, g, dBh, dBt, rec);
-    if (!ok) { atomicExch(status, 1); return; }
+    const int t = threadIdx.x;
+    bool ok = true;
+    if (seg == 0) *bad = 0;
+    if (mine) {
+        double G[BS][BS] = {};
+        const int b0 = c0 * g.mm;
+        if (b0 > 0) ok = fac_run<TS, false>(d, g, dB, dB + 9, rec, max(0, b0 - fac_warm(d.method)), b0, G);
+        for (int p = 0; p < BS; ++p)
+            for (int q = 0; q < BS; ++q) gs[t][p * BS + q] = G[p][q];
+        if (ok) ok = fac_run<TS, true>(d, g, dB, dB + 9, rec, b0, c1 * g.mm, G);
+        for (int p = 0; p < BS; ++p)
+            for (int q = 0; q < BS; ++q) ge[t][p * BS + q] = G[p][q];
+    }
+    __syncthreads();
+    if (mine) {
+        if (seg > 0) {
+            double diff = 0.0, size = 0.0;
+            for (int i = 0; i < BS * BS; ++i) {
+                diff = fmax(diff, fabs(gs[t][i] - ge[t - 1][i]));
+                size = fmax(size, fabs(ge[t - 1][i]));
+            }
+            ok = ok && diff <= kFacWarmTol * size;  // false for NaN
+        }
+        if (!ok) atomicExch(bad, 1);
+    }
+    __syncthreads();
+    if (mine && seg == 0 && *bad) {
+        double G[BS][BS] = {};
+        if (!fac_run<TS, true>(d, g, dB, dB + 9, rec, 0, g.nb, G)) atomicExch(status, 1);
+    }
+    __syncthreads();  // the line's F and H are written (to global memory, by this block)
+    if (!mine) return;
     const double tau = sizeof(TS) == 4 ? 0x1p-40 : 0x1p-70;
-    const TS *F = rec + fac_part(g), *H = rec + (size_t)2 * fac_part(g);
-    const int rf = d.method == kCFD ? fac_reach<TS, 2>(F, g.tact, tau, true) : fac_reach<TS, 3>(F, g.tact, tau, true);
-    const int rb = d.method == kCFD ? fac_reach<TS, 2>(H, g.tact, tau, false) : fac_reach<TS, 3>(H, g.tact, tau, false);
-    TS *info = rec + fac_info(g);
+    const int rf = fac_reach<TS, BS>(rec + fac_part(g), g.tact, tau, true, c0, c1);
+    const int rb = fac_reach<TS, BS>(rec + (size_t)2 * fac_part(g), g.tact, tau, false, c0, c1);
+    gs[t][0] = rf;
+    ge[t][0] = rb;
+}
+
+template <typename TS>
+__global__ void __launch_bounds__(kFacRecThreads) fac_records_kernel(const LineDesc<TS> *__restrict__ descs, int nlines,
+                                                                     int segs, const double *dB, int *status) {
+    __shared__ double gs[kFacRecThreads][9], ge[kFacRecThreads][9];
+    __shared__ int bad[kFacRecThreads];
+    const int per = kFacRecThreads / segs, t = threadIdx.x;
+    const int l = t / segs, seg = t % segs, line = blockIdx.x * per + l;
+    const bool mine = line < nlines;
+    const LineDesc<TS> &d = descs[mine ? line : 0];
+    const FacGeom g = fac_geom(d.method, d.N);
+    const double *db = dB + (size_t)(mine ? line : 0) * 18;
+    if (d.method == kCFD) fac_records<TS, 2>(d, g, db, segs, seg, mine, gs, ge, bad + l, status);
+    else fac_records<TS, 3>(d, g, db, segs, seg, mine, gs, ge, bad + l, status);
+    __syncthreads();
+    if (!mine || seg != 0) return;
+    double rf = 0.0, rb = 0.0;
+    for (int k = 0; k < segs; ++k) {
+        rf = fmax(rf, gs[t + k][0]);
+        rb = fmax(rb, ge[t + k][0]);
+    }
+    TS *info = d.sep + fac_info(g);
     info[0] = (TS)rf;
     info[1] = (TS)rb;
     info[2] = info[3] = (TS)0;
-    atomicMax(status + 1, max(rf, rb));
+    atomicMax(status + 1, (int)fmax(rf, rb));
 }
 
 // ---------------------------------------------------------------------------------------
@@ -731,22 +964,7 @@ __device__ __forceinline__ void seg_scan(Map<T, BS> a, bool forward, int Tl, T (
     }
 }
 
-// Block inverse of the line kernel: the FP32 path takes the hardware reciprocal
-// approximation (relative error below 2^-22).
-__device__ __forceinline__ float fac_rcp(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-// FP64: the hardware approximation r0 (about 20 bits) and one step of Householder's cubic iteration, r0 (1 + e
-// + e^2) with e = 1 - x r0: three FMAs against a division's ten or so operations on the FP64 pipe that bounds these kernels;
-// the error left is e^3 = 2^-60 and one rounding (measured against 1 / x: at most 1 ulp).
-__device__ __forceinline__ double fac_rcp(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = __fma_rn(-x, r, 1.0);
-    return __fma_rn(r, __fma_rn(e, e, e), r);
-}
+// Block inverse of the line kernel.
 template <typename T, int BS>
 __device__ __forceinline__ void fac_inv(const T (&S)[BS][BS], T (&R)[BS][BS]) {
     if constexpr (BS == 2) {
@@ -1830,10 +2048,24 @@ line_solve_factored_kernel(const LineDesc<T> *__restrict__ descs, const FacGroup
     }
 }
 
+// The records of nlines lines of one simulation and direction (N cells each).  dB: 18 FP64 values a line.
 template <typename T>
-cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, double *ws, int *status, cudaStream_t s) {
+cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, int method, int N, double *dB, int *status,
+                                  cudaStream_t s) {
     if (nlines <= 0) return cudaSuccess;
-    fac_precompute_kernel<T><<<(nlines + 63) / 64, 64, 0, s>>>(d, nlines, ws, status);
+    const int jobs = 2 * nlines;
+    fac_ends_kernel<T><<<(jobs + kFacEndWarps - 1) / kFacEndWarps, 32 * kFacEndWarps, 0, s>>>(d, nlines, dB, status);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const FacGeom g = fac_geom(method, N);
+    // threads per line: a power of two, up to four warps an SM in all (the FP64 pipe's four parts) while a run
+    // is no shorter than half its warm-up (1023 CFD lines of 1024 cells: 267 us)
+    int segs = 1, dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 152;
+    while (segs < 32 && (long long)nlines * segs < 4ll * 32 * sms && g.nb / (2 * segs) >= fac_warm(method) / 2) segs *= 2;
+    const int per = kFacRecThreads / segs;
+    fac_records_kernel<T><<<(nlines + per - 1) / per, kFacRecThreads, 0, s>>>(d, nlines, segs, dB, status);
     return cudaGetLastError();
 }
 
@@ -1880,8 +2112,8 @@ cudaError_t launch_line_solve_factored(const LineDesc<T> *d, const FacGroup *gro
     return cudaErrorInvalidValue;
 }
 
-template cudaError_t launch_fac_precompute<float>(const LineDesc<float> *, int, double *, int *, cudaStream_t);
-template cudaError_t launch_fac_precompute<double>(const LineDesc<double> *, int, double *, int *, cudaStream_t);
+template cudaError_t launch_fac_precompute<float>(const LineDesc<float> *, int, int, int, double *, int *, cudaStream_t);
+template cudaError_t launch_fac_precompute<double>(const LineDesc<double> *, int, int, int, double *, int *, cudaStream_t);
 template cudaError_t launch_line_solve_factored<float>(const LineDesc<float> *, const FacGroup *, int, int, size_t, int,
                                                        int, int, int *, cudaStream_t);
 template cudaError_t launch_line_solve_factored<double>(const LineDesc<double> *, const FacGroup *, int, int, size_t,

@@ -147,10 +147,10 @@ constexpr int kFacVariants = 7;
 int fac_lines_per_cta(int method, int N, size_t esz);
 size_t fac_stage_bytes(int method, int N, int nl, size_t esz);  // shared memory of one stage
 int fac_stages_for(size_t stage_bytes, size_t esz, int method);  // groups in flight that fit: 3, 2, 1 or 0
-size_t fac_ws_doubles();                 // FP64 workspace per line of the precompute
+size_t fac_ws_doubles();                 // FP64 workspace per line of the precompute (its ends' dB)
 // status[0]: set when a line system is singular; status[1]: atomic max of the lines' scan reach
 template <typename T>
-cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, double *ws, int *status,
+cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, int method, int N, double *ws, int *status,
                                   cudaStream_t s);
 // Each group takes the windowed or the full scans by its own kFacOwnFull bit, so a line's
 // arithmetic does not depend on the other lines of the launch.

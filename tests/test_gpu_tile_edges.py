@@ -72,6 +72,27 @@ def test_line_lengths_at_path_changes(adi, method, n, fp64):
     _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, 3, source=src), fp64)
 
 
+@pytest.mark.parametrize("method", [CFD, MFD])
+@pytest.mark.parametrize("cfl", [0.8, 40.0])
+def test_records_of_long_lines(adi, method, cfl):
+    """The factored solver's records of a line are built by several threads, each from a start that forgets what lies
+    before it; with a large time step it does not and the line is done in one run.  Both against the
+    thread-per-line elimination in FP64.  Tolerance: the line systems' condition number grows as cfl^2 (about 10
+    at 0.8, 2e4 at 40 on these media) times a few hundred roundings of 1.1e-16: 1e-12 and 2e-9."""
+    nx, ny = 2000, 40
+    h, dt, c, U, V, W = _case(method, nx, ny, 5, cfl=cfl)
+    out = []
+    for solver in (adi.ADI_SOLVER_FACTORED, adi.ADI_SOLVER_LINE):
+        sim = adi.Sim(method, nx, ny, h, dt, c, U, V, W, precision=adi.ADI_FP64, solver=solver)
+        assert sim.solver == solver
+        sim.step(1)
+        out.append(sim.read())
+        sim.close()
+    tol = 1e-12 if cfl < 1 else 2e-9
+    for a, b in zip(*out):
+        assert np.max(np.abs(a - b)) <= tol * np.max(np.abs(b))
+
+
 def test_fp64_reciprocal():
     """The FP64 line kernels' reciprocal (fac_rcp) against CUDA's correctly rounded 1 / x: at most one unit in the
     last place off, for 2^20 values over the exponents that pivots and determinants take."""
