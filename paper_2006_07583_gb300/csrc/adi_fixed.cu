@@ -5,10 +5,15 @@
 // along every line of its direction until the sum of the Frobenius norms of the two updates
 // is at most eps, or kmax sweeps have run.  Dv, Du are the App. A compact operators
 // (Pbar^{-1} Qbar, P^{-1} Q: a tridiagonal solve per application) or the App. B mimetic
-// stencils (D4, G4).  The norm test runs on the device: every sweep's kernels read a status
-// word and return at once when an earlier sweep has converged, so no host round trip sits
-// between sweeps.  One thread per line (the paper's GPU decomposition); natural (u, v, w)
-// fields in row-major device arrays.
+// stencils (D4, G4).  The norm test runs on the device: every sweep's kernel reads a status
+// word and returns at once when an earlier sweep has converged, so no host round trip sits
+// between sweeps.  Natural (u, v, w) fields in row-major device arrays; one launch per sweep.
+//
+// A block takes up to four lines.  The stencils and updates are spread over its threads; the Thomas
+// recurrences, which are serial along a line and are done in the order of a plain elimination, run on one thread per
+// line out of shared memory, sixteen rows' operands loaded ahead; they bound it.  With everything on one thread per
+// line in global memory (the paper's own decomposition) each row waited for memory several times: 1093 us a sweep for
+// 512 lines of 512 cells, now 36 us.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -27,70 +32,17 @@ namespace {
 template <typename T>
 struct FpTri {
     const T *m, *id, *c;
+    int lo, hi;  // the rows lo .. hi-1 have the factors of row lo (the elimination settles within some 30 rows)
 };
 
 // Device-side convergence state of one stage's iteration.
 struct FpState {
     double sum[2];  // squared Frobenius norms of the two updates of the current sweep
-    int k;          // sweeps done in this stage
+    unsigned arrived;  // blocks of the current sweep that have added theirs
+    int k;          // sweeps done in this stage (its parity picks the current iterate's buffers)
     int done;       // the stage's iteration has stopped
     long long sweeps;  // sweeps over the whole call
 };
-
-// Du along a line of N cells: CFD P^{-1} Q / h on nodes 0..N (N+1 -> N+1); MFD G4 / h
-// (N+2 -> N+1).  x: the pressure line with element stride sx; out: N+1 values, stride so.
-template <typename T>
-__device__ void fp_du(int method, int N, T ih, const T *x, long long sx, T *out, long long so, FpTri<T> P) {
-    double w[6];
-    int c0 = 0;
-    if (method == kCFD) {
-        for (int r = 0; r <= N; ++r) {
-            const int n = cfd_Q_row(N, r, &c0, w);
-            T acc = T(0);
-            for (int i = 0; i < n; ++i) acc += (T)w[i] * x[(long long)(c0 + i) * sx];
-            out[(long long)r * so] = acc * ih;
-        }
-        for (int r = 1; r <= N; ++r) out[(long long)r * so] -= P.m[r] * out[(long long)(r - 1) * so];
-        out[(long long)N * so] *= P.id[N];
-        for (int r = N - 1; r >= 0; --r)
-            out[(long long)r * so] = (out[(long long)r * so] - P.c[r] * out[(long long)(r + 1) * so]) * P.id[r];
-    } else {
-        for (int j = 0; j <= N; ++j) {
-            const int n = mfd_G_row(N, j, &c0, w);
-            T acc = T(0);
-            for (int i = 0; i < n; ++i) acc += (T)w[i] * x[(long long)(c0 + i) * sx];
-            out[(long long)j * so] = acc * ih;
-        }
-    }
-}
-
-// Dv along a line of N cells: CFD Pbar^{-1} Qbar / h (N+1 -> interior nodes 1..N-1); MFD
-// D4 / h (N+1 -> cells 1..N).  Written at the pressure-line indices 1..L-1 of out.
-template <typename T>
-__device__ void fp_dv(int method, int N, T ih, const T *x, long long sx, T *out, long long so, FpTri<T> Pb) {
-    double w[6];
-    int c0 = 0;
-    if (method == kCFD) {
-        for (int j = 1; j <= N - 1; ++j) {
-            const int n = cfd_Qbar_row(N, j, &c0, w);
-            T acc = T(0);
-            for (int i = 0; i < n; ++i) acc += (T)w[i] * x[(long long)(c0 + i) * sx];
-            out[(long long)j * so] = acc * ih;
-        }
-        // Pbar rows j = 1..N-1 are factor rows 0..N-2
-        for (int j = 2; j <= N - 1; ++j) out[(long long)j * so] -= Pb.m[j - 1] * out[(long long)(j - 1) * so];
-        out[(long long)(N - 1) * so] *= Pb.id[N - 2];
-        for (int j = N - 2; j >= 1; --j)
-            out[(long long)j * so] = (out[(long long)j * so] - Pb.c[j - 1] * out[(long long)(j + 1) * so]) * Pb.id[j - 1];
-    } else {
-        for (int r = 0; r < N; ++r) {
-            const int n = mfd_D_row(N, r, &c0, w);
-            T acc = T(0);
-            for (int i = 0; i < n; ++i) acc += (T)w[i] * x[(long long)(c0 + i) * sx];
-            out[(long long)(r + 1) * so] = acc * ih;
-        }
-    }
-}
 
 // Lines of one direction: line l (first .. first + n - 1) of the pressure-like arrays starts
 // at l * lsp with element stride esp, of the velocity arrays at l * lsv with stride esv.
@@ -99,68 +51,229 @@ struct FpLines {
     long long lsp, esp, lsv, esv;
 };
 
+__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fmar(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fmar(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// A block's share: `lines` (1, 2 or 4) lines from line0 on, nl of them in use; threads run along a line in whole
+// warps where its elements are contiguous (unit), else with the lines side by side.
+constexpr int kFpThreads = 256, kFpLines = 4;
+struct FpShare {
+    int lines, nl;
+    long long line0;
+    __device__ FpShare(const FpLines &g, int lines_) : lines(lines_) {
+        const int at = blockIdx.x * lines;
+        nl = min(lines, g.n - at);
+        line0 = (long long)g.first + at;
+    }
+    __device__ int line(bool unit) const { return (unit ? threadIdx.x >> 5 : threadIdx.x) & (lines - 1); }
+    __device__ int first(bool unit) const { return unit ? (threadIdx.x >> 5) / lines * 32 + (threadIdx.x & 31) : threadIdx.x / lines; }
+    __device__ int step() const { return kFpThreads / lines; }
+};
+
+// Thomas solve in place, one thread per line: x[r], r < n, factors f (row r at index r).  The middle rows, whose
+// factors are all the same, go in batches, the next batch's values loaded before this one's recurrence.
+template <typename T>
+__device__ void fp_thomas(T *x, int n, FpTri<T> f) {
+    constexpr int U = 16;
+    T v[U], w[U];
+    T d = x[0];
+    int r = 1;
+    for (; r < f.lo; ++r) { d = fmar(-f.m[r], d, x[r]); x[r] = d; }
+    if (r + U <= f.hi) {
+        const T m = -f.m[r];
+#pragma unroll
+        for (int i = 0; i < U; ++i) v[i] = x[r + i];
+        for (; r + U <= f.hi; r += U) {
+            const bool more = r + 2 * U <= f.hi;
+            if (more)
+#pragma unroll
+                for (int i = 0; i < U; ++i) w[i] = x[r + U + i];
+#pragma unroll
+            for (int i = 0; i < U; ++i) { d = fmar(m, d, v[i]); x[r + i] = d; }
+            if (more)
+#pragma unroll
+                for (int i = 0; i < U; ++i) v[i] = w[i];
+        }
+    }
+    for (; r < n; ++r) { d = fmar(-f.m[r], d, x[r]); x[r] = d; }
+    d = mulr(d, f.id[n - 1]);
+    x[n - 1] = d;
+    for (r = n - 2; r >= f.hi; --r) { d = mulr(fmar(-f.c[r], d, x[r]), f.id[r]); x[r] = d; }
+    if (r - U + 1 >= f.lo) {
+        const T c = -f.c[r], id = f.id[r];
+#pragma unroll
+        for (int i = 0; i < U; ++i) v[i] = x[r - i];
+        for (; r - U + 1 >= f.lo; r -= U) {
+            const bool more = r - 2 * U + 1 >= f.lo;
+            if (more)
+#pragma unroll
+                for (int i = 0; i < U; ++i) w[i] = x[r - U - i];
+#pragma unroll
+            for (int i = 0; i < U; ++i) { d = mulr(fmar(c, d, v[i]), id); x[r - i] = d; }
+            if (more)
+#pragma unroll
+                for (int i = 0; i < U; ++i) v[i] = w[i];
+        }
+    }
+    for (; r >= 0; --r) { d = mulr(fmar(-f.c[r], d, x[r]), f.id[r]); x[r] = d; }
+}
+
+// Du of the share's pressure lines u (global): CFD P^{-1} Q / h on nodes 0..N; MFD G4 / h.  Into x[l * pitch + j].
+template <typename T>
+__device__ void fp_du(int method, int N, T ih, const T *u, long long ls, long long es, const FpShare &sh, T *x, int pitch,
+                      FpTri<T> P) {
+    const int l = sh.line(es == 1);
+    const T *ul = u + (sh.line0 + l) * ls;
+    for (int j = sh.first(es == 1); j <= N && l < sh.nl; j += sh.step()) {
+        T acc = T(0);
+        if (method == kCFD && j > 0 && j < N) {
+            acc = fmar(T(3), ul[(j + 1) * es], mulr(T(-3), ul[(j - 1) * es]));
+        } else if (method != kCFD && j > 1 && j < N - 1) {
+            acc = mulr((T)mim_w(0), ul[(j - 1) * es]);
+#pragma unroll
+            for (int i = 1; i < 4; ++i) acc = fmar((T)mim_w(i), ul[(j - 1 + i) * es], acc);
+        } else {
+            double w[6];
+            int c0 = 0;
+            const int n = method == kCFD ? cfd_Q_row(N, j, &c0, w) : mfd_G_row(N, j, &c0, w);
+            for (int i = 0; i < n; ++i) acc = fmar((T)w[i], ul[(c0 + i) * es], acc);
+        }
+        x[l * pitch + j] = mulr(acc, ih);
+    }
+    __syncthreads();
+    if (method == kCFD) {
+        if ((int)threadIdx.x < sh.nl) fp_thomas<T>(x + threadIdx.x * pitch, N + 1, P);
+        __syncthreads();
+    }
+}
+
+// Dv of the share's velocity lines v: CFD Pbar^{-1} Qbar / h at nodes 1..N-1; MFD D4 / h at cells 1..N.  Into x[l *
+// pitch + k], k the pressure index.
+template <typename T>
+__device__ void fp_dv(int method, int N, T ih, const T *v, long long ls, long long es, const FpShare &sh, T *x, int pitch,
+                      FpTri<T> Pb) {
+    const int l = sh.line(es == 1), last = method == kCFD ? N - 1 : N;
+    const T *vl = v + (sh.line0 + l) * ls;
+    for (int k = 1 + sh.first(es == 1); k <= last && l < sh.nl; k += sh.step()) {
+        T acc = T(0);
+        if (method == kCFD && k > 1 && k < N - 1) {
+            acc = fmar(T(3), vl[(k + 1) * es], mulr(T(-3), vl[(k - 1) * es]));
+        } else if (method != kCFD && k > 1 && k < N) {
+            acc = mulr((T)mim_w(0), vl[(k - 2) * es]);
+#pragma unroll
+            for (int i = 1; i < 4; ++i) acc = fmar((T)mim_w(i), vl[(k - 2 + i) * es], acc);
+        } else {
+            double w[6];
+            int c0 = 0;
+            const int n = method == kCFD ? cfd_Qbar_row(N, k, &c0, w) : mfd_D_row(N, k - 1, &c0, w);
+            for (int i = 0; i < n; ++i) acc = fmar((T)w[i], vl[(c0 + i) * es], acc);
+        }
+        x[l * pitch + k] = mulr(acc, ih);
+    }
+    __syncthreads();
+    if (method == kCFD) {  // Pbar's rows 0 .. N-2 are the nodes 1 .. N-1
+        if ((int)threadIdx.x < sh.nl) fp_thomas<T>(x + threadIdx.x * pitch + 1, N - 1, Pb);
+        __syncthreads();
+    }
+}
+__host__ __device__ inline int fp_pitch(int N) { return (N + 2) | 1; }
+
 // Explicit right-hand side of a stage along its explicit direction:
 //   ov = vl - beta Du(ul)   (all N+1 velocities),   oa = ul - alpha Dv(vl)   (interior)
-template <typename T>
-__global__ void fp_rhs_kernel(int method, FpLines g, T ih, T beta, const T *__restrict__ ul, const T *__restrict__ vl,
-                              const T *__restrict__ alpha, T *ov, T *oa, FpTri<T> P, FpTri<T> Pb) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= g.n) return;
-    const long long l = g.first + t;
-    const T *u = ul + l * g.lsp, *v = vl + l * g.lsv, *al = alpha + l * g.lsp;
-    T *o_v = ov + l * g.lsv, *o_a = oa + l * g.lsp;
-    fp_du<T>(method, g.N, ih, u, g.esp, o_v, g.esv, P);
-    for (int k = 0; k <= g.N; ++k) o_v[k * g.esv] = v[k * g.esv] - beta * o_v[k * g.esv];
-    fp_dv<T>(method, g.N, ih, v, g.esv, o_a, g.esp, Pb);
-    for (int k = 1; k < g.L; ++k) o_a[k * g.esp] = u[k * g.esp] - al[k * g.esp] * o_a[k * g.esp];
-}
-
-// One sweep of Eq. 9 along the implicit direction:
-//   oa = a - alpha Dv(vk)   (interior; oa's end values are the Dirichlet data),
-//   ov = vb - beta Du(oa).
-template <typename T>
-__global__ void fp_sweep_kernel(int method, FpLines g, T ih, T beta, const T *__restrict__ a, const T *__restrict__ vk,
-                                const T *__restrict__ vb, const T *__restrict__ alpha, T *oa, T *ov, FpTri<T> P,
-                                FpTri<T> Pb, const FpState *st) {
-    if (st->done) return;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= g.n) return;
-    const long long l = g.first + t;
-    const T *av = a + l * g.lsp, *v = vk + l * g.lsv, *b = vb + l * g.lsv, *al = alpha + l * g.lsp;
-    T *o_a = oa + l * g.lsp, *o_v = ov + l * g.lsv;
-    fp_dv<T>(method, g.N, ih, v, g.esv, o_a, g.esp, Pb);
-    for (int k = 1; k < g.L; ++k) o_a[k * g.esp] = av[k * g.esp] - al[k * g.esp] * o_a[k * g.esp];
-    fp_du<T>(method, g.N, ih, o_a, g.esp, o_v, g.esv, P);
-    for (int k = 0; k <= g.N; ++k) o_v[k * g.esv] = b[k * g.esv] - beta * o_v[k * g.esv];
-}
-
-// Squared norm of x - y into *sum (FP64 accumulation).
-template <typename T>
-__global__ void fp_diff_kernel(const T *__restrict__ x, const T *__restrict__ y, size_t n, double *sum, const FpState *st) {
-    if (st->done) return;
-    double acc = 0.0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const double d = (double)x[i] - (double)y[i];
-        acc += d * d;
+// ul0 / ul1 (and vl0 / vl1): the iterate's buffers, picked by the parity of st->k (st may be null).
+// FAR: a line's rows do not fit shared memory and go through the block's part of far_rows instead.
+template <typename T, bool FAR>
+__global__ void __launch_bounds__(kFpThreads) fp_rhs_kernel(int method, FpLines g, T ih, T beta, const T *ul0, const T *ul1,
+                                                            const T *vl0, const T *vl1, const T *__restrict__ alpha, T *ov,
+                                                            T *oa, FpTri<T> P, FpTri<T> Pb, const FpState *st, int lines,
+                                                            T *far_rows) {
+    extern __shared__ __align__(16) unsigned char fp_smem[];
+    T *x = FAR ? far_rows + (size_t)blockIdx.x * lines * fp_pitch(g.N) : (T *)fp_smem;
+    const bool odd = st && (st->k & 1);
+    const T *ul = odd ? ul1 : ul0, *vl = odd ? vl1 : vl0;
+    const FpShare sh(g, lines);
+    const int pitch = fp_pitch(g.N), l = sh.line(g.esv == 1);
+    fp_du<T>(method, g.N, ih, ul, g.lsp, g.esp, sh, x, pitch, P);
+    for (int k = sh.first(g.esv == 1); k <= g.N && l < sh.nl; k += sh.step()) {
+        const long long o = (sh.line0 + l) * g.lsv + k * g.esv;
+        ov[o] = fmar(-beta, x[l * pitch + k], vl[o]);
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    __shared__ double part[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) part[warp] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
-        atomicAdd(sum, s);
+    fp_dv<T>(method, g.N, ih, vl, g.lsv, g.esv, sh, x, pitch, Pb);
+    for (int k = 1 + sh.first(g.esp == 1); k < g.L && l < sh.nl; k += sh.step()) {
+        const long long o = (sh.line0 + l) * g.lsp + k * g.esp;
+        oa[o] = fmar(-alpha[o], x[l * pitch + k], ul[o]);
     }
 }
 
-// End of a sweep: the test of the paper (sum of the two Frobenius norms) against eps and the
-// sweep limit; later sweeps of the stage return at once once it has stopped.
-__global__ void fp_finish_kernel(FpState *st, double eps, int kmax) {
+// x - y exactly as FP64 gives it, with one FP64 conversion where FP32 already holds it (two values within a factor of
+// two of each other; Knuth's two-sum finds what is left otherwise): the FP64 pipe is far slower than FP32's.
+__device__ __forceinline__ double fp_diff(double x, double y) { return x - y; }
+__device__ __forceinline__ double fp_diff(float x, float y) {
+    const float d = __fsub_rn(x, y), yv = __fsub_rn(x, d), xv = __fadd_rn(d, yv);
+    const float rest = __fadd_rn(__fsub_rn(x, xv), __fsub_rn(yv, y));
+    double e = (double)d;
+    if (rest != 0.f) e += (double)rest;
+    return e;
+}
+
+// One sweep of Eq. 9 along the implicit direction, from the iterate (u_k, v_k) of the parity of st->k
+// to the other buffers:
+//   u_{k+1} = a - alpha Dv(v_k)   (interior; the end values are the Dirichlet data, in both buffers),
+//   v_{k+1} = vb - beta Du(u_{k+1}),
+// with the squared norms of the two updates; the last block to finish does the stopping test (the
+// paper's: the sum of the two Frobenius norms against eps, or kmax sweeps).
+template <typename T, bool FAR>
+__global__ void __launch_bounds__(kFpThreads) fp_sweep_kernel(int method, FpLines g, T ih, T beta, const T *__restrict__ a,
+                                                              T *u0, T *u1, T *v0, T *v1, const T *__restrict__ vb,
+                                                              const T *__restrict__ alpha, FpTri<T> P, FpTri<T> Pb,
+                                                              FpState *st, double eps, int kmax, int lines, T *far_rows) {
     if (st->done) return;
-    const double test = sqrt(st->sum[0]) + sqrt(st->sum[1]);
+    extern __shared__ __align__(16) unsigned char fp_smem[];
+    T *x = FAR ? far_rows + (size_t)blockIdx.x * lines * fp_pitch(g.N) : (T *)fp_smem;
+    const bool odd = st->k & 1;
+    const T *uk = odd ? u1 : u0, *vk = odd ? v1 : v0;
+    T *un = odd ? u0 : u1, *vn = odd ? v0 : v1;
+    const FpShare sh(g, lines);
+    const int pitch = fp_pitch(g.N), l = sh.line(g.esv == 1);
+    double du2 = 0.0, dv2 = 0.0;
+    fp_dv<T>(method, g.N, ih, vk, g.lsv, g.esv, sh, x, pitch, Pb);
+    for (int k = 1 + sh.first(g.esp == 1); k < g.L && l < sh.nl; k += sh.step()) {
+        const long long o = (sh.line0 + l) * g.lsp + k * g.esp;
+        const T val = fmar(-alpha[o], x[l * pitch + k], a[o]);
+        const double e = fp_diff(val, uk[o]);
+        du2 += e * e;
+        un[o] = val;
+    }
+    __syncthreads();  // u_{k+1} of the share's lines is read back by its other threads
+    fp_du<T>(method, g.N, ih, un, g.lsp, g.esp, sh, x, pitch, P);
+    for (int k = sh.first(g.esv == 1); k <= g.N && l < sh.nl; k += sh.step()) {
+        const long long o = (sh.line0 + l) * g.lsv + k * g.esv;
+        const T val = fmar(-beta, x[l * pitch + k], vb[o]);
+        const double e = fp_diff(val, vk[o]);
+        dv2 += e * e;
+        vn[o] = val;
+    }
+    __shared__ double part[2][kFpThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) {
+        du2 += __shfl_xor_sync(0xffffffffu, du2, o);
+        dv2 += __shfl_xor_sync(0xffffffffu, dv2, o);
+    }
+    if ((threadIdx.x & 31) == 0) { part[0][threadIdx.x >> 5] = du2; part[1][threadIdx.x >> 5] = dv2; }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    du2 = dv2 = 0.0;
+    for (int w = 0; w < kFpThreads / 32; ++w) { du2 += part[0][w]; dv2 += part[1][w]; }
+    atomicAdd(&st->sum[0], du2);
+    atomicAdd(&st->sum[1], dv2);
+    __threadfence();
+    if (atomicAdd(&st->arrived, 1u) + 1 != gridDim.x) return;
+    __threadfence();
+    const double test = sqrt(__ldcg(&st->sum[0])) + sqrt(__ldcg(&st->sum[1]));
     st->sum[0] = st->sum[1] = 0.0;
+    st->arrived = 0;
     st->k += 1;
     st->sweeps += 1;
     if (test <= eps || st->k >= kmax) st->done = 1;
@@ -168,13 +281,15 @@ __global__ void fp_finish_kernel(FpState *st, double eps, int kmax) {
 
 __global__ void fp_reset_kernel(FpState *st) {
     st->sum[0] = st->sum[1] = 0.0;
+    st->arrived = 0;
     st->k = 0;
     st->done = 0;
 }
 
+// dst <- src0, or src1 where st (if given) ended a stage at an odd number of sweeps.
 template <typename T>
-__global__ void fp_copy_kernel(T *dst, const T *__restrict__ src, size_t n, const FpState *st) {
-    if (st && st->done) return;
+__global__ void fp_copy_kernel(T *dst, const T *src0, const T *src1, size_t n, const FpState *st) {
+    const T *src = st && (st->k & 1) ? src1 : src0;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         dst[i] = src[i];
 }
@@ -269,6 +384,12 @@ int run_fixed(int method, int nx, int ny, double h, double dt, const double *c_f
                 ++slot;
             }
             t.m = ptr[0]; t.id = ptr[1]; t.c = ptr[2];
+            // the run of equal factors around the middle row, in the precision that the kernels use
+            const int n = (int)m.size();
+            auto same = [&](int r, int k) { return (T)m[r] == (T)m[k] && (T)id[r] == (T)id[k] && (T)c[r] == (T)c[k]; };
+            t.lo = t.hi = n / 2;
+            while (t.hi < n - 1 && same(t.hi, n / 2)) ++t.hi;
+            while (t.lo > 1 && same(t.lo - 1, n / 2)) --t.lo;
             return t;
         };
         Px = make(nx, false); Pbx = make(nx, true); Py = make(ny, false); Pby = make(ny, true);
@@ -279,11 +400,33 @@ int run_fixed(int method, int nx, int ny, double h, double dt, const double *c_f
     FpLines rows{1, piy, nx, cfd ? nx : nx + 1, (long long)cu, 1, (long long)cv, 1};
     FpLines cols{1, pix, ny, cfd ? ny : ny + 1, 1, (long long)cu, 1, (long long)cw};
     const T ih = (T)(1.0 / h), beta = (T)(0.5 * dt);
-    const int tb = 128;
-    auto blocks = [&](int n) { return (n + tb - 1) / tb; };
+    // lines per block: four, fewer where their rows would not fit shared memory (beside the norms' 128 bytes); lines that
+    // do not fit alone keep their rows in global memory
+    constexpr size_t kSmem = 226 * 1024;
+    auto far = [&](const FpLines &g) { return fp_pitch(g.N) * sizeof(T) > kSmem; };
+    auto lines_of = [&](const FpLines &g) {
+        int n = kFpLines;
+        while (!far(g) && n > 1 && (size_t)n * fp_pitch(g.N) * sizeof(T) > kSmem) n /= 2;
+        return n;
+    };
+    auto smem = [&](const FpLines &g) { return far(g) ? 0 : (size_t)lines_of(g) * fp_pitch(g.N) * sizeof(T); };
+    auto grid = [&](const FpLines &g) { return (unsigned)((g.n + lines_of(g) - 1) / lines_of(g)); };
+    auto rhs = [&](const FpLines &g) { return far(g) ? fp_rhs_kernel<T, true> : fp_rhs_kernel<T, false>; };
+    auto sweep = [&](const FpLines &g) { return far(g) ? fp_sweep_kernel<T, true> : fp_sweep_kernel<T, false>; };
+    DevArr far_mem;
+    size_t far_n = 0;
+    for (const FpLines *g : {&rows, &cols})
+        if (far(*g)) far_n = std::max(far_n, (size_t)grid(*g) * lines_of(*g) * fp_pitch(g->N));
+    if (far_n && cudaMalloc(&far_mem.p, far_n * sizeof(T)) != cudaSuccess) { (void)cudaGetLastError(); return ADI_ENOMEM; }
+    T *far_rows = (T *)far_mem.p;
+    const int most = (int)std::max(smem(rows), smem(cols));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_rhs_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fp_sweep_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e != cudaSuccess) { (void)cudaGetLastError(); return ADI_ECUDA; }
     FpState *st = (FpState *)state.p;
-    auto copy = [&](int dst, int src, size_t n, const FpState *guard) {
-        fp_copy_kernel<T><<<152 * 4, 256>>>(P(dst), P(src), n, guard);
+    auto copy = [&](int dst, int src0, int src1, size_t n, const FpState *s) {
+        fp_copy_kernel<T><<<152 * 4, 256>>>(P(dst), P(src0), P(src1), n, s);
     };
     const double sscale = 0.5 * dt / (h * h);
     const long long sp = src ? (long long)src[0] * cu + (long long)src[1] : 0;
@@ -294,45 +437,39 @@ int run_fixed(int method, int nx, int ny, double h, double dt, const double *c_f
     cudaEventRecord(e0);
     for (int m = 0; m < nsteps; ++m) {
         const double t = t0 + m * dt;
-        // ---- stage 1: w* and a explicit along y (columns), then x-line sweeps ----
-        copy(dWs, dW, nW, nullptr);
-        copy(dUs, dU, nU, nullptr);
-        copy(dVs, dV, nV, nullptr);
-        fp_rhs_kernel<T><<<blocks(pix), tb>>>(method, cols, ih, beta, P(dU), P(dW), P(dAl), P(dWs), P(dA), Py, Pby);
+        // ---- stage 1: w* and a explicit along y (columns), then x-line sweeps; u* and v* alternate
+        // between (Us, Vs) and (Uk, Vk), starting from u^m, v^m in the latter pair ----
+        copy(dWs, dW, dW, nW, nullptr);
+        copy(dUs, dU, dU, nU, nullptr);
+        copy(dVs, dV, dV, nV, nullptr);
+        copy(dUk, dU, dU, nU, nullptr);
+        copy(dVk, dV, dV, nV, nullptr);
+        rhs(cols)<<<grid(cols), kFpThreads, smem(cols)>>>(method, cols, ih, beta, P(dU), P(dU), P(dW), P(dW), P(dAl),
+                                                                 P(dWs), P(dA), Py, Pby, nullptr, lines_of(cols), far_rows);
         if (src) fp_source_kernel<T><<<1, 1>>>(P(dA), sp, sscale, src[2], src[3], src[4], t);
-        copy(dUk, dU, nU, nullptr);
-        copy(dVk, dV, nV, nullptr);
         fp_reset_kernel<<<1, 1>>>(st);
-        for (int k = 0; k < kmax; ++k) {
-            fp_sweep_kernel<T><<<blocks(piy), tb>>>(method, rows, ih, beta, P(dA), P(dVk), P(dV), P(dAl), P(dUs),
-                                                    P(dVs), Px, Pbx, st);
-            fp_diff_kernel<T><<<152 * 2, 256>>>(P(dUs), P(dUk), nU, &st->sum[0], st);
-            fp_diff_kernel<T><<<152 * 2, 256>>>(P(dVs), P(dVk), nV, &st->sum[1], st);
-            fp_finish_kernel<<<1, 1>>>(st, eps, kmax);
-            copy(dUk, dUs, nU, st);
-            copy(dVk, dVs, nV, st);
-        }
-        // ---- stage 2: v^{m+1} and C explicit along x (rows), then y-line sweeps ----
-        copy(dVn, dVs, nV, nullptr);
-        fp_rhs_kernel<T><<<blocks(piy), tb>>>(method, rows, ih, beta, P(dUs), P(dVs), P(dAl), P(dVn), P(dA), Px, Pbx);
+        for (int k = 0; k < kmax; ++k)
+            sweep(rows)<<<grid(rows), kFpThreads, smem(rows)>>>(method, rows, ih, beta, P(dA), P(dUk), P(dUs), P(dVk),
+                                                                       P(dVs), P(dV), P(dAl), Px, Pbx, st, eps, kmax,
+                                                                       lines_of(rows), far_rows);
+        // ---- stage 2: v^{m+1} and C explicit along x (rows), then y-line sweeps from u* and w^m,
+        // alternating between (Uk, Wk) and (Un, Wn) ----
+        copy(dVn, dVk, dVs, nV, st);
+        copy(dUn, dUk, dUs, nU, st);
+        rhs(rows)<<<grid(rows), kFpThreads, smem(rows)>>>(method, rows, ih, beta, P(dUk), P(dUs), P(dVk), P(dVs),
+                                                                 P(dAl), P(dVn), P(dA), Px, Pbx, st, lines_of(rows), far_rows);
         if (src) fp_source_kernel<T><<<1, 1>>>(P(dA), sp, sscale, src[2], src[3], src[4], t + dt);
-        copy(dWn, dWs, nW, nullptr);
-        copy(dUn, dUs, nU, nullptr);
-        copy(dUk, dUs, nU, nullptr);
-        copy(dWk, dW, nW, nullptr);
+        copy(dUk, dUn, dUn, nU, nullptr);
+        copy(dWn, dWs, dWs, nW, nullptr);
+        copy(dWk, dW, dW, nW, nullptr);
         fp_reset_kernel<<<1, 1>>>(st);
-        for (int k = 0; k < kmax; ++k) {
-            fp_sweep_kernel<T><<<blocks(pix), tb>>>(method, cols, ih, beta, P(dA), P(dWk), P(dWs), P(dAl), P(dUn),
-                                                    P(dWn), Py, Pby, st);
-            fp_diff_kernel<T><<<152 * 2, 256>>>(P(dUn), P(dUk), nU, &st->sum[0], st);
-            fp_diff_kernel<T><<<152 * 2, 256>>>(P(dWn), P(dWk), nW, &st->sum[1], st);
-            fp_finish_kernel<<<1, 1>>>(st, eps, kmax);
-            copy(dUk, dUn, nU, st);
-            copy(dWk, dWn, nW, st);
-        }
-        copy(dU, dUn, nU, nullptr);
-        copy(dV, dVn, nV, nullptr);
-        copy(dW, dWn, nW, nullptr);
+        for (int k = 0; k < kmax; ++k)
+            sweep(cols)<<<grid(cols), kFpThreads, smem(cols)>>>(method, cols, ih, beta, P(dA), P(dUk), P(dUn), P(dWk),
+                                                                       P(dWn), P(dWs), P(dAl), Py, Pby, st, eps, kmax,
+                                                                       lines_of(cols), far_rows);
+        copy(dU, dUk, dUn, nU, st);
+        copy(dV, dVn, dVn, nV, nullptr);
+        copy(dW, dWk, dWn, nW, st);
     }
     cudaEventRecord(e1);
     e = cudaEventSynchronize(e1);

@@ -72,6 +72,22 @@ def test_line_lengths_at_path_changes(adi, method, n, fp64):
     _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, 3, source=src), fp64)
 
 
+# line counts around a block's four lines; lines so long that a block takes two (FP64 above 7260 cells, FP32 above
+# 14520) or one (FP64 above 14520), or keeps its rows in global memory (FP64 above 28900, FP32 above 57800); the
+# recurrences go sixteen rows at a time
+@pytest.mark.parametrize("method,nx,ny,fp64", [(CFD, 16, 17, True), (CFD, 17, 18, False), (MFD, 18, 19, True),
+                                               (CFD, 23, 24, True), (CFD, 25, 320, False), (CFD, 7300, 16, True),
+                                               (CFD, 16, 14600, True), (MFD, 15000, 16, False),
+                                               (CFD, 29000, 16, True), (MFD, 16, 58000, False)])
+def test_fixed_point_blocks(adi, method, nx, ny, fp64):
+    h, dt, c, U, V, W = _case(method, nx, ny, 21, cfl=0.6)
+    src = (ny // 2, nx // 3, 0.01, 15.0, 0.0)
+    *G, sweeps, _ = adi.fixed_point(method, nx, ny, h, dt, c, U, V, W, 2, source=src, kmax=3, eps=0.0,
+                                    precision=adi.ADI_FP64 if fp64 else adi.ADI_FP32)
+    assert sweeps == 2 * 2 * 3
+    _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, 2, source=src, kmax=3, eps=0.0), fp64)
+
+
 @pytest.mark.parametrize("method", [CFD, MFD])
 @pytest.mark.parametrize("cfl", [0.8, 40.0])
 def test_records_of_long_lines(adi, method, cfl):
