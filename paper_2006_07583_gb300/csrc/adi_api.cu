@@ -205,9 +205,7 @@ struct Plan {
         SpongeRec rec[2];         // the natural fields to damp (v: the copy stage 1 wrote)
         const void *ydesc[2];     // y-line descriptors of the next step's parity
         int nlines = 0, N = 0, method = 0;
-        void *scr = nullptr;      // prologue scratch, then (CFD) the Thomas factors
-        const void *fac = nullptr;
-        long long st = 1;
+        const void *fac = nullptr;  // CFD: the prologue's Thomas factors
         void *A3 = nullptr, *A0 = nullptr;
         int rows_u = 0, ldu = 0, ldc = 0, lda = 0;
         int harm = -1;            // index of the member's harmonic record, or -1
@@ -270,8 +268,8 @@ struct adi_sim {
     double h = 0, dt = 0;
     size_t esz = 4;
     DevBuf A[4], V[2], W[2], alpha, alphaT, Uo, Wo, tab, sep, cold_all, clock, status;
-    // host <-> device staging of the natural fields (FP64) and the prologue's scratch with the
-    // Thomas factors after it: allocated by the first adi_set_fields / adi_read_fields /
+    // host <-> device staging of the natural fields (FP64) and the prologue's Thomas factors
+    // (CFD): allocated by the first adi_set_fields / adi_read_fields /
     // adi_set_source after creation and kept until adi_destroy (adi_create frees its own)
     DevBuf xfer, pro;
     int parity = 0;                           // which V/W copy is current
@@ -299,11 +297,11 @@ struct adi_sim {
     double h_omega = 0, h_phb = 0, h_phf = 0;
     DevBuf h_edges, h_frow, h_fcol, h_self;
     // absorbing layers (adi_set_sponge): width in cells and strength; the y-line descriptors
-    // of both parities and the prologue's scratch (with the CFD Thomas factors) kept on the
-    // device for the per-step rebuild of the carried state
+    // of both parities and the prologue's Thomas factors (CFD) kept on the device for the
+    // per-step rebuild of the carried state
     bool sp_on = false;
     double sp_width = 0, sp_a = 0;
-    DevBuf sp_desc[2], sp_scr;
+    DevBuf sp_desc[2], sp_fac;
 };
 
 struct adi_batch_t {
@@ -851,9 +849,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
             sp.ydesc[q] = s->sp_desc[1 - pm].p;
         }
         sp.nlines = s->nlines[1]; sp.N = g.ny; sp.method = g.method;
-        sp.st = std::max(1, s->nlines[1]);
-        sp.scr = s->sp_scr.p;
-        sp.fac = g.method == ADI_CFD ? (const void *)((unsigned char *)s->sp_scr.p + (size_t)(2 * g.ny + 2) * sp.st * s->esz) : nullptr;
+        sp.fac = s->sp_fac.p;
         sp.A3 = s->A[3].p; sp.A0 = s->A[0].p;
         sp.rows_u = g.rows_u; sp.ldu = g.ldu; sp.ldc = g.ldc; sp.lda = g.lda;
         sp.harm = my_h;
@@ -921,7 +917,7 @@ cudaError_t enqueue_stage(const Plan &p, int q, int dir, int natural, cudaStream
             e = launch_sponge<T>(sp.rec[q], stream);
             if (e == cudaSuccess)
                 e = launch_prologue_lines<T>((const LineDesc<T> *)sp.ydesc[q], sp.nlines, sp.N, sp.method,
-                                             (const T *)sp.fac, (T *)sp.scr, sp.st, stream);
+                                             (const T *)sp.fac, stream);
             if (e == cudaSuccess) {  // the prologue wrote a column-major (A[3]); a row-major copy
                 dim3 grid((unsigned)((sp.rows_u + 31) / 32), (unsigned)((sp.ldu + 31) / 32)), block(32, 8);
                 transpose_kernel<T><<<grid, block, 0, stream>>>((const T *)sp.A3, sp.ldu, sp.rows_u, sp.ldc,
@@ -997,26 +993,21 @@ int upload_sim_descs(adi_sim *s) {
 template <typename T>
 int run_prologue_t(adi_sim *s) {
     const LineDesc<T> *cols = (const LineDesc<T> *)((unsigned char *)s->cold_all.p + s->h_desc[s->parity][0].size());
-    const long long st = std::max(1, s->nlines[1]);
     const int N = s->g.ny;
-    const size_t scr = (size_t)(2 * N + 2) * st, nfac = s->g.method == ADI_CFD ? prologue_factor_count(N) : 0;
-    const size_t bytes = (scr + nfac) * sizeof(T);
+    const size_t bytes = s->g.method == ADI_CFD ? prologue_factor_count(N) * sizeof(T) : 0;
     cudaError_t e = cudaSuccess;
-    if (s->pro.bytes != bytes) {  // first use: scratch plus the CFD Thomas factors of P, Pbar
+    if (s->pro.bytes != bytes) {  // first use: the CFD Thomas factors of P, Pbar
         dev_free(s->pro);
         int rc = dev_alloc(s->pro, bytes);
         if (rc) return rc;
-        if (nfac) {
-            std::vector<double> f;
-            prologue_factors(N, f);
-            std::vector<T> ft(f.begin(), f.end());
-            e = cudaMemcpyAsync((T *)s->pro.p + scr, ft.data(), ft.size() * sizeof(T), cudaMemcpyHostToDevice, s->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // ft leaves scope
-        }
+        std::vector<double> f;
+        prologue_factors(N, f);
+        std::vector<T> ft(f.begin(), f.end());
+        e = cudaMemcpyAsync(s->pro.p, ft.data(), ft.size() * sizeof(T), cudaMemcpyHostToDevice, s->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // ft leaves scope
     }
     if (e == cudaSuccess)
-        e = launch_prologue_lines<T>(cols, s->nlines[1], N, s->g.method, nfac ? (const T *)s->pro.p + scr : nullptr,
-                                     (T *)s->pro.p, st, s->stream);
+        e = launch_prologue_lines<T>(cols, s->nlines[1], N, s->g.method, (const T *)s->pro.p, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     // the prologue wrote a column-major (A[3]), like a stage-2 launch
@@ -1619,35 +1610,26 @@ int adi_set_sponge(adi_handle s, double width, double a) {
     if (width == 0 || a == 0) {
         if (!s->sp_on) return ADI_OK;
         s->sp_on = false;
-        dev_free(s->sp_desc[0]); dev_free(s->sp_desc[1]); dev_free(s->sp_scr);
+        dev_free(s->sp_desc[0]); dev_free(s->sp_desc[1]); dev_free(s->sp_fac);
     } else {
         const Geometry &g = s->g;
-        const long long st = std::max(1, s->nlines[1]);
         const int N = g.ny;
-        const size_t scr = (size_t)(2 * N + 2) * st, nfac = g.method == ADI_CFD ? prologue_factor_count(N) : 0;
+        const size_t nfac = g.method == ADI_CFD ? prologue_factor_count(N) : 0;
         const size_t dbytes = s->h_desc[0][1].size();
         if (s->sp_desc[0].bytes != dbytes) {
             dev_free(s->sp_desc[0]); dev_free(s->sp_desc[1]);
             rc = dev_alloc(s->sp_desc[0], dbytes);
             if (!rc) rc = dev_alloc(s->sp_desc[1], dbytes);
         }
-        if (!rc && s->sp_scr.bytes != (scr + nfac) * s->esz) {
-            dev_free(s->sp_scr);
-            rc = dev_alloc(s->sp_scr, (scr + nfac) * s->esz);
-            if (!rc && nfac) {
-                std::vector<double> f;
-                prologue_factors(N, f);
-                if (s->precision == ADI_FP64) {
-                    rc = cuda_status(cudaMemcpyAsync((double *)s->sp_scr.p + scr, f.data(), f.size() * sizeof(double),
-                                                     cudaMemcpyHostToDevice, s->stream));
-                    if (!rc) rc = cuda_status(cudaStreamSynchronize(s->stream));
-                } else {
-                    std::vector<float> ff(f.begin(), f.end());
-                    rc = cuda_status(cudaMemcpyAsync((float *)s->sp_scr.p + scr, ff.data(), ff.size() * sizeof(float),
-                                                     cudaMemcpyHostToDevice, s->stream));
-                    if (!rc) rc = cuda_status(cudaStreamSynchronize(s->stream));  // ff leaves scope
-                }
-            }
+        if (!rc && s->sp_fac.bytes != nfac * s->esz) {
+            dev_free(s->sp_fac);
+            rc = dev_alloc(s->sp_fac, nfac * s->esz);
+            std::vector<double> f;
+            prologue_factors(N, f);
+            const std::vector<float> ff(f.begin(), f.end());
+            const void *src = s->precision == ADI_FP64 ? (const void *)f.data() : (const void *)ff.data();
+            if (!rc) rc = cuda_status(cudaMemcpyAsync(s->sp_fac.p, src, nfac * s->esz, cudaMemcpyHostToDevice, s->stream));
+            if (!rc) rc = cuda_status(cudaStreamSynchronize(s->stream));  // the factors leave scope
         }
         if (!rc) { s->sp_on = true; s->sp_width = width; s->sp_a = a; }
     }
@@ -1682,7 +1664,7 @@ int adi_set_source(adi_handle s, int is, int js, double amp, double f0, double t
     if (!rc) rc = plan_build(s->plan, std::vector<adi_sim *>{s}, s->stream);
     s->plan_base = s->parity;
     if (!rc) rc = prologue(s);  // a picks up dt/2 f(t_now) at the source point
-    dev_free(s->pro);           // a one-off: the prologue's scratch is not kept
+    dev_free(s->pro);           // a one-off: the prologue's factors are not kept
     if (rc) s->sticky = rc;
     return rc;
 }
@@ -1857,7 +1839,7 @@ int adi_destroy(adi_handle s) {
     DevBuf *bufs[] = {&s->A[0], &s->A[1], &s->A[2], &s->A[3], &s->V[0], &s->V[1], &s->W[0], &s->W[1], &s->alpha,
                       &s->alphaT, &s->Uo, &s->Wo, &s->tab, &s->sep, &s->cold_all, &s->clock, &s->status,
                       &s->xfer, &s->pro, &s->h_edges, &s->h_frow, &s->h_fcol, &s->h_self,
-                      &s->sp_desc[0], &s->sp_desc[1], &s->sp_scr};
+                      &s->sp_desc[0], &s->sp_desc[1], &s->sp_fac};
     for (DevBuf *b : bufs) dev_free(*b);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     (void)cudaGetLastError();

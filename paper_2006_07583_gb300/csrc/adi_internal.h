@@ -61,12 +61,11 @@ cudaError_t launch_prologue(const LineDesc<T> *col_lines, int nlines, const T *f
 // chunked solves (prologue_factor_count(N) values in all)
 void prologue_factors(int N, std::vector<double> &out);
 size_t prologue_factor_count(int N);
-// The prologue over the y-lines of one simulation (N cells each) with one thread per line
-// element for the stencils (and, for CFD, one per line for the Thomas solves with fac).
-// scratch: 2N elements per line (element k at k * st + line).
+// The prologue over the y-lines of one simulation (N cells each), spread over the lines' elements;
+// fac: the Thomas factors of prologue_factors() in T (CFD; nullptr for MFD).
 template <typename T>
 cudaError_t launch_prologue_lines(const LineDesc<T> *col_lines, int nlines, int N, int method, const T *fac,
-                                  T *scratch, long long st, cudaStream_t s);
+                                  cudaStream_t s);
 template <typename T>
 cudaError_t launch_finite_check(const T *x, size_t n, int *flag, cudaStream_t s);
 

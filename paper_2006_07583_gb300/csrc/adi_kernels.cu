@@ -378,29 +378,19 @@ __global__ void prologue_kernel(const LineDesc<T> *__restrict__ descs, int nline
 }
 
 // ---------------------------------------------------------------------------------------
-// The same prologue spread over the lines' elements.  prologue_stencil_kernel: block (32
-// lines, 8 elements); for CFD it leaves (Q u)_j / h (j = 0..N) and (Qbar w)_j / h (j = 1..N-1)
-// in the scratch (element k of a line at k * st + line), for MFD it writes w* and a directly.
-// prologue_solve_win_kernel (CFD): the two Thomas solves with the precomputed factors, one
-// thread per chunk of a line (below).
+// The same prologue spread over the lines' elements.  prologue_mfd_kernel: MFD, block (32 lines, 8
+// elements).  prologue_cfd_kernel: CFD, the two Thomas solves with the precomputed factors, one thread
+// per chunk of a line, the right-hand sides formed as the sweeps need them.
 // ---------------------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T prologue_src(const LineDesc<T> &d) {
     return (T)(d.src_scale * ricker(d.src_amp, d.src_f0, d.src_tdelay, (double)(*d.clock) * d.dt));
 }
 
-// Interior rows of the explicit operators (CFD Q and Qbar: -3, 0, 3; MFD D4 and G4: the
-// fourth-order staggered stencil), with the weights as compile-time constants of T; the same
+// Interior rows of MFD's explicit operators (D4 and G4: the fourth-order staggered stencil), with the
+// weights as compile-time constants of T; the same
 // terms in the same order as the row functions give them, so the sums are the same.  p points
 // at the row's first point, s is the stride along the line.
-template <typename T>
-__device__ __forceinline__ T cfd_interior_dot(const T *p, long long s) {
-    T acc = T(0);
-    acc += T(-3.0) * p[0];
-    acc += T(0.0) * p[s];
-    acc += T(3.0) * p[2 * s];
-    return acc;
-}
 template <typename T>
 __device__ __forceinline__ T mfd_interior_dot(const T *p, long long s) {
     T acc = T(0);
@@ -412,11 +402,10 @@ __device__ __forceinline__ T mfd_interior_dot(const T *p, long long s) {
 }
 
 template <typename T>
-__global__ void prologue_stencil_kernel(const LineDesc<T> *__restrict__ descs, int nlines, int N, int method,
-                                        T *scratch, long long st) {
+__global__ void prologue_mfd_kernel(const LineDesc<T> *__restrict__ descs, int nlines, int N) {
     // block (32 lines, 8): elements j0 .. j0 + 31 of 32 consecutive lines; lane = line reads the
-    // row-major natural fields coalesced.  MFD writes w* and a, which are contiguous along each
-    // line, through shared memory, along each line in turn.
+    // row-major natural fields coalesced; w* and a, which are contiguous along each line, are written
+    // through shared memory, along each line in turn.
     __shared__ T tv[32][33], tp[32][33], tu[32][33];
     // the block's 32 descriptors, copied once with 16-byte loads (each thread would otherwise
     // read its own descriptor's fields, 32 scattered sectors per load)
@@ -444,54 +433,30 @@ __global__ void prologue_stencil_kernel(const LineDesc<T> *__restrict__ descs, i
         for (int jj = y; jj < 32; jj += 8) {
             const int j = j0 + jj;
             if (j > N + 1) break;
-            if (method == kCFD) {
-                if (j <= N) {
-                    T acc = T(0);
-                    if (j >= 1 && j <= N - 1) {
-                        acc = cfd_interior_dot(un + (long long)(j - 1) * snp, snp);
-                    } else {
-                        const int n = cfd_Q_row(N, j, &c0, w);
-                        for (int t = 0; t < n; ++t) acc += (T)w[t] * un[(c0 + t) * snp];
-                    }
-                    scratch[(long long)j * st + line] = acc * ih;
+            if (j <= N) {
+                T acc = T(0);
+                if (j >= 2 && j <= N - 2) {
+                    acc = mfd_interior_dot(un + (long long)(j - 1) * snp, snp);
+                } else {
+                    const int n = mfd_G_row(N, j, &c0, w);
+                    for (int t = 0; t < n; ++t) acc += (T)w[t] * un[(c0 + t) * snp];
                 }
-                if (j >= 1 && j <= N - 1) {
-                    T acc = T(0);
-                    if (j >= 2 && j <= N - 2) {
-                        acc = cfd_interior_dot(wn + (long long)(j - 1) * snv, snv);
-                    } else {
-                        const int n = cfd_Qbar_row(N, j, &c0, w);
-                        for (int t = 0; t < n; ++t) acc += (T)w[t] * wn[(c0 + t) * snv];
-                    }
-                    scratch[(long long)(N + j) * st + line] = acc * ih;
+                tv[jj][x] = wn[j * snv] - beta * acc * ih;
+            }
+            tu[jj][x] = un[j * snp];
+            if (j >= 1 && j <= N) {
+                // a = u - alpha (D w)/h (+ source), formed below along the line
+                T acc = T(0);
+                if (j >= 2 && j <= N - 1) {
+                    acc = mfd_interior_dot(wn + (long long)(j - 2) * snv, snv);
+                } else {
+                    const int n = mfd_D_row(N, j - 1, &c0, w);
+                    for (int t = 0; t < n; ++t) acc += (T)w[t] * wn[(c0 + t) * snv];
                 }
-            } else {
-                if (j <= N) {
-                    T acc = T(0);
-                    if (j >= 2 && j <= N - 2) {
-                        acc = mfd_interior_dot(un + (long long)(j - 1) * snp, snp);
-                    } else {
-                        const int n = mfd_G_row(N, j, &c0, w);
-                        for (int t = 0; t < n; ++t) acc += (T)w[t] * un[(c0 + t) * snp];
-                    }
-                    tv[jj][x] = wn[j * snv] - beta * acc * ih;
-                }
-                tu[jj][x] = un[j * snp];
-                if (j >= 1 && j <= N) {
-                    // a = u - alpha (D w)/h (+ source), formed below along the line
-                    T acc = T(0);
-                    if (j >= 2 && j <= N - 1) {
-                        acc = mfd_interior_dot(wn + (long long)(j - 2) * snv, snv);
-                    } else {
-                        const int n = mfd_D_row(N, j - 1, &c0, w);
-                        for (int t = 0; t < n; ++t) acc += (T)w[t] * wn[(c0 + t) * snv];
-                    }
-                    tp[jj][x] = acc;
-                }
+                tp[jj][x] = acc;
             }
         }
     }
-    if (method == kCFD) return;  // uniform over the block
     __syncthreads();
     // lane = element: 8 lines at a time, 32 consecutive elements each
     for (int l = y; l < 32 && line0 + l < nlines; l += 8) {
@@ -508,7 +473,7 @@ __global__ void prologue_stencil_kernel(const LineDesc<T> *__restrict__ descs, i
     }
 }
 
-// The same two Thomas solves spread over chunks of kProR rows of every line, one thread per
+// The two Thomas solves spread over chunks of kProR rows of every line, one thread per
 // (line, chunk): a line of 4097 rows gives 65 threads instead of one, so the solve is no longer a
 // chain of thousands of dependent steps per thread.  Each thread solves the rows of its chunk
 // plus a halo of kProH rows on each side that are not at a line end, with the values beyond the
@@ -559,46 +524,100 @@ __host__ __device__ __forceinline__ void prologue_win_solve(int n, int r0, int r
     }
 }
 
-// grid.y: the chunks of P (N+1 rows) first, then those of Pbar (N-1 rows).  A block is one warp
-// of 32 consecutive lines.  The lines' natural fields are row-major, so lane = line reads them
-// coalesced; the outputs (w*, a) and alpha are contiguous along each line, so they go through
-// shared memory and move along each line in turn, lane = row.  (Loading the window's right-hand
-// sides and natural values into shared memory first measured slower: 508-536 against 406 us at
-// 4096 lines of 4097 rows.)
+// A warp takes 32 consecutive lines and one chunk of P (N+1 rows) or Pbar (N-1 rows); grid.y times the
+// block's warps: the chunks of P first, then those of Pbar.  The lines' natural fields are row-major, so
+// lane = line reads them coalesced, and the right-hand sides Q u / h and Qbar w / h are formed row by row
+// from them (two reads, one of them still in the L1 from the row before, instead of a pass of its own
+// that wrote them and a read of that), without a branch, so that the rows' loads run ahead of the recurrence: the
+// two boundary rows' values are formed beforehand.  The outputs (w*, a) and alpha are contiguous along each
+// line, so they go through shared memory and move along each line in turn, lane = row, eight lines' loads at
+// a time (one line after the other made a warp wait for alpha 64 times).  Every value is rounded as the two-pass
+// form rounded it.  4096 lines of 4097 rows: 531 -> 305 us with the stencil pass that this replaces; 640 lines of 641 rows 46
+// -> 25 us.
 template <typename T>
-__global__ void __launch_bounds__(32) prologue_solve_win_kernel(const LineDesc<T> *__restrict__ descs, int nlines,
-                                                                int N, const T *scratch, long long st,
-                                                                const T *__restrict__ fac) {
-    __shared__ T tile[kProR][33];  // per line: the forward values, then the chunk's outputs
-    __shared__ T tu[kProR][33];    // Pbar chunks: u at the chunk's nodes
-    const int lane = threadIdx.x;
-    const int line0 = blockIdx.x * 32, line = line0 + lane;
+constexpr int kProWarps = sizeof(T) == 4 ? 2 : 1;
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_of(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_of(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+template <typename T>
+__global__ void __launch_bounds__(32 * kProWarps<T>) prologue_cfd_kernel(const LineDesc<T> *__restrict__ descs, int nlines,
+                                                                         int N, const T *__restrict__ fac) {
+    __shared__ T stile[kProWarps<T>][kProR][33];  // per line: the forward values, then the chunk's outputs
+    __shared__ T stu[kProWarps<T>][kProR][33];    // Pbar chunks: u at the chunk's nodes
+    __shared__ __align__(16) unsigned char sdesc[32 * sizeof(LineDesc<T>)];
+    static_assert(sizeof(LineDesc<T>) % 16 == 0, "descriptor size");
+    const int lane = threadIdx.x, warp = threadIdx.y;
+    const int line0 = blockIdx.x * 32, nl = min(32, nlines - line0);
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(descs + line0);
+        uint4 *dst = reinterpret_cast<uint4 *>(sdesc);
+        const int nvec = nl * (int)(sizeof(LineDesc<T>) / 16);
+        for (int k = warp * 32 + lane; k < nvec; k += 32 * kProWarps<T>) dst[k] = src[k];
+    }
+    __syncthreads();
+    const LineDesc<T> *sd = reinterpret_cast<const LineDesc<T> *>(sdesc);
+    T (*tile)[33] = stile[warp], (*tu)[33] = stu[warp];
     const int nP = N + 1, nB = N - 1;
-    const int chP = (nP + kProR - 1) / kProR;
-    const bool isP = (int)blockIdx.y < chP;
-    const int c = isP ? (int)blockIdx.y : (int)blockIdx.y - chP;
+    const int chP = (nP + kProR - 1) / kProR, chB = (nB + kProR - 1) / kProR;
+    const int ch = blockIdx.y * kProWarps<T> + warp;
+    if (ch >= chP + chB) return;
+    const bool isP = ch < chP;
+    const int c = isP ? ch : ch - chP;
     const int r0 = c * kProR, r1 = min(isP ? nP : nB, r0 + kProR), nr = r1 - r0;
     const T *su_id = fac + 3 * (N + 1) + 3 * (N - 1);
-    if (line < nlines) {
-        const LineDesc<T> &d = descs[line];
-        const T beta = (T)d.beta;
-        const T *un = d.u_out, *wn = d.w_out;
+    if (lane < nl) {
+        const LineDesc<T> &d = sd[lane];
+        const T beta = (T)d.beta, ih = (T)d.inv_h;
+        const T *__restrict__ un = d.u_out, *__restrict__ wn = d.w_out;
         const long long snp = d.snp, snv = d.snv;
-        const T *__restrict__ q = scratch + (isP ? 0 : (long long)(N + 1) * st) + line;
-        auto qf = [&](int r) -> T { return q[(long long)r * st]; };
+        double w[8];
+        int c0;
+        auto row_dot = [&](const T *x, long long st, int n) {
+            T acc = T(0);
+            for (int t = 0; t < n; ++t) acc += (T)w[t] * x[(c0 + t) * st];
+            return mul_rn(acc, ih);
+        };
+        // rows r0 - kProH .. r1 + kProH - 1 at most: inside the line (no boundary row, no clamped address) or not
+        const bool inner = r0 - kProH >= 1 && r1 + kProH <= (isP ? N : N - 2);
         if (isP) {
             // P g = (Q u)/h over rows 0..N; w*_r = w_r - beta g_r
             const T *lo = fac, *cu = fac + (N + 1), *id = fac + 2 * (N + 1);
-            prologue_win_solve<T>(nP, r0, r1, qf, lo, cu, id, su_id, &tile[0][lane], 33,
-                                  [&](int r, T g) { tile[r - r0][lane] = wn[(long long)r * snv] - beta * g; }, r0);
+            auto qi = [&](int lo_r, int hi_r) -> T {
+                return mul_rn(fma_of(T(3), un[hi_r * snp], mul_rn(T(-3), un[lo_r * snp])), ih);
+            };
+            auto out = [&](int r, T g) { tile[r - r0][lane] = wn[r * snv] - beta * g; };
+            if (inner) {
+                prologue_win_solve<T>(nP, r0, r1, [&](int r) -> T { return qi(r - 1, r + 1); }, lo, cu, id, su_id, &tile[0][lane],
+                                      33, out, r0);
+            } else {
+                const T first = row_dot(un, snp, cfd_Q_row(N, 0, &c0, w)), last = row_dot(un, snp, cfd_Q_row(N, N, &c0, w));
+                prologue_win_solve<T>(nP, r0, r1, [&](int r) -> T {
+                    const T q = qi(max(r - 1, 0), min(r + 1, N));
+                    return r == 0 ? first : r == N ? last : q;
+                }, lo, cu, id, su_id, &tile[0][lane], 33, out, r0);
+            }
         } else {
             // Pbar e = (Qbar w)/h over nodes 1..N-1 (rows 0..N-2); a_j = u_j - alpha_j e_j (+ source)
             const T *fb = fac + 3 * (N + 1);
             const T *lo = fb, *cu = fb + (N - 1), *id = fb + 2 * (N - 1);
-            prologue_win_solve<T>(nB, r0, r1, qf, lo, cu, id, su_id, &tile[0][lane], 33, [&](int r, T e) {
+            auto qi = [&](int r) -> T {
+                return mul_rn(fma_of(T(3), wn[(r + 2) * snv], mul_rn(T(-3), wn[r * snv])), ih);
+            };
+            auto out = [&](int r, T e) {
                 tile[r - r0][lane] = e;
-                tu[r - r0][lane] = un[(long long)(r + 1) * snp];
-            }, r0);
+                tu[r - r0][lane] = un[(r + 1) * snp];
+            };
+            if (inner) {
+                prologue_win_solve<T>(nB, r0, r1, qi, lo, cu, id, su_id, &tile[0][lane], 33, out, r0);
+            } else {
+                const T first = row_dot(wn, snv, cfd_Qbar_row(N, 1, &c0, w)), last = row_dot(wn, snv, cfd_Qbar_row(N, N - 1, &c0, w));
+                prologue_win_solve<T>(nB, r0, r1, [&](int r) -> T {
+                    const T q = qi(r);
+                    return r == 0 ? first : r == N - 2 ? last : q;
+                }, lo, cu, id, su_id, &tile[0][lane], 33, out, r0);
+            }
             if (c == 0) {
                 d.po[0] = un[0];
                 d.po[(long long)N * d.spo] = un[(long long)N * snp];
@@ -606,19 +625,27 @@ __global__ void __launch_bounds__(32) prologue_solve_win_kernel(const LineDesc<T
         }
     }
     __syncwarp();
-    for (int l = 0; l < 32 && line0 + l < nlines; ++l) {
-        const LineDesc<T> &dl = descs[line0 + l];
-        if (isP) {
-            for (int k = lane; k < nr; k += 32) dl.v[(long long)(r0 + k) * dl.sv] = tile[k][l];
-        } else {
-            for (int k = lane; k < nr; k += 32) {
+    for (int k = lane; k < nr; k += 32)
+        for (int l0 = 0; l0 < nl; l0 += 8) {
+            if (isP) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (l0 + i < nl) sd[l0 + i].v[(r0 + k) * sd[l0 + i].sv] = tile[k][l0 + i];
+            } else {
                 const long long j = r0 + k + 1;
-                T val = tu[k][l] - dl.alpha[j * dl.sp] * tile[k][l];
-                if (j == dl.src_k) val += prologue_src(dl);
-                dl.po[j * dl.spo] = val;
+                T al[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) al[i] = l0 + i < nl ? sd[l0 + i].alpha[j * sd[l0 + i].sp] : T(0);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (l0 + i >= nl) break;
+                    const LineDesc<T> &dl = sd[l0 + i];
+                    T val = tu[k][l0 + i] - al[i] * tile[k][l0 + i];
+                    if (j == dl.src_k) val += prologue_src(dl);
+                    dl.po[j * dl.spo] = val;
+                }
             }
         }
-    }
 }
 
 // Sets *flag if any x[i] is NaN or infinite: 16-byte loads over the aligned body of x (when x
@@ -677,15 +704,14 @@ cudaError_t launch_prologue(const LineDesc<T> *d, int nlines, const T *fac, T *s
 }
 
 template <typename T>
-cudaError_t launch_prologue_lines(const LineDesc<T> *d, int nlines, int N, int method, const T *fac, T *scratch,
-                                  long long st, cudaStream_t s) {
+cudaError_t launch_prologue_lines(const LineDesc<T> *d, int nlines, int N, int method, const T *fac, cudaStream_t s) {
     if (nlines <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((nlines + 31) / 32), (unsigned)((N + 2 + 31) / 32));
-    prologue_stencil_kernel<T><<<grid, dim3(32, 8), 0, s>>>(d, nlines, N, method, scratch, st);
+    const unsigned gx = (unsigned)((nlines + 31) / 32);
     if (method == kCFD) {
-        const unsigned chunks = (unsigned)((N + 1 + kProR - 1) / kProR + (N - 1 + kProR - 1) / kProR);
-        prologue_solve_win_kernel<T><<<dim3((unsigned)((nlines + 31) / 32), chunks), 32, 0, s>>>(d, nlines, N,
-                                                                                              scratch, st, fac);
+        const int chunks = (N + 1 + kProR - 1) / kProR + (N - 1 + kProR - 1) / kProR, w = kProWarps<T>;
+        prologue_cfd_kernel<T><<<dim3(gx, (unsigned)((chunks + w - 1) / w)), dim3(32, w), 0, s>>>(d, nlines, N, fac);
+    } else {
+        prologue_mfd_kernel<T><<<dim3(gx, (unsigned)((N + 2 + 31) / 32)), dim3(32, 8), 0, s>>>(d, nlines, N);
     }
     return cudaGetLastError();
 }
@@ -741,8 +767,7 @@ cudaError_t launch_finite_check(const T *x, size_t n, int *flag, cudaStream_t s)
                                                  int, cudaStream_t);                         \
     template cudaError_t launch_prologue<T>(const LineDesc<T> *, int, const T *, T *, long long,  \
                                             cudaStream_t);                                         \
-    template cudaError_t launch_prologue_lines<T>(const LineDesc<T> *, int, int, int, const T *, T *, \
-                                                  long long, cudaStream_t);                                   \
+    template cudaError_t launch_prologue_lines<T>(const LineDesc<T> *, int, int, int, const T *, cudaStream_t); \
     template cudaError_t launch_finite_check<T>(const T *, size_t, int *, cudaStream_t);
 ADI_INST(float)
 ADI_INST(double)
