@@ -436,6 +436,46 @@ __global__ void transpose_kernel(const T *__restrict__ src, int rows, int cols, 
     }
 }
 
+// The entries of the carried arrays that no line writes, from the natural fields: the outer rows and columns
+// of the pressure arrays (the Dirichlet data), the first and last columns of both w* copies and the first and
+// last rows of the v copy that the next step writes.  Everything else of these arrays is written before
+// it is read (A[1] and A[2] by stage 1, A[3] and the current w* by the prologue, the other w* and v copies by
+// the step), so loading new fields copies edges only: at 4096^2 four transposes and three copies of whole
+// fields (300 us) became one launch of 5 us.
+template <typename T>
+struct EdgeRec {
+    const T *u, *w, *v;     // natural u (rows_u x ldu), w (rows_w x ldw); the current v (leading dimension ldvp)
+    T *a1, *a2, *a3;        // A[1] (column-major, ldc), A[2] (row-major, lda), A[3] (as A[1])
+    T *w0, *w1, *vo;        // both w* copies (column-major, ldwc), the other v copy
+    int rows_u, ldu, rows_w, ldw, rows_v, ldv, lda, ldc, ldwc, ldvp;
+};
+template <typename T>
+__global__ void edges_kernel(EdgeRec<T> r) {
+    const size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const size_t lr = r.rows_u - 1, lc = r.ldu - 1, wc = r.ldw - 1, vr = r.rows_v - 1;
+    if (k <= lc) {  // first and last rows of u
+        const T a = r.u[k], b = r.u[lr * r.ldu + k];
+        r.a2[k] = a; r.a2[lr * r.lda + k] = b;
+        r.a1[k * r.ldc] = a; r.a1[k * r.ldc + lr] = b;
+        r.a3[k * r.ldc] = a; r.a3[k * r.ldc + lr] = b;
+    }
+    if (k <= lr) {  // first and last columns
+        const T a = r.u[k * r.ldu], b = r.u[k * r.ldu + lc];
+        r.a2[k * r.lda] = a; r.a2[k * r.lda + lc] = b;
+        r.a1[k] = a; r.a1[lc * r.ldc + k] = b;
+        r.a3[k] = a; r.a3[lc * r.ldc + k] = b;
+    }
+    if (k < (size_t)r.rows_w) {
+        const T a = r.w[k * r.ldw], b = r.w[k * r.ldw + wc];
+        r.w0[k] = a; r.w0[wc * r.ldwc + k] = b;
+        r.w1[k] = a; r.w1[wc * r.ldwc + k] = b;
+    }
+    if (k < (size_t)r.ldv) {
+        r.vo[k] = r.v[k];
+        r.vo[vr * r.ldvp + k] = r.v[vr * r.ldvp + k];
+    }
+}
+
 // One array of a batched transpose: dst[c * ld_dst + r] = src[r * ld_src + c] for r < rows,
 // c < cols.
 struct TDesc {
@@ -876,6 +916,20 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
     return rc;
 }
 
+// The carried pressure of every member into the layout of the next stage's lines.
+template <typename T>
+cudaError_t enqueue_transposes(const Plan &p, int dir, cudaStream_t stream) {
+    if (!p.tcount[dir]) return cudaSuccess;
+    if (sizeof(T) == 4) {
+        dim3 grid((unsigned)((p.tcols[dir] + 63) / 64), (unsigned)((p.trows[dir] + 63) / 64), (unsigned)p.tcount[dir]);
+        transpose_batch64_kernel<<<grid, dim3(16, 16), 0, stream>>>((const TDesc *)p.tdesc[dir].p);
+        return cudaGetLastError();
+    }
+    dim3 grid((unsigned)((p.tcols[dir] + 31) / 32), (unsigned)((p.trows[dir] + 31) / 32), (unsigned)p.tcount[dir]);
+    transpose_batch_kernel<T><<<grid, dim3(32, 8), 0, stream>>>((const TDesc *)p.tdesc[dir].p);
+    return cudaGetLastError();
+}
+
 // One stage (dir 0: stage 1 over x-lines, dir 1: stage 2 over y-lines) of a plan at plan
 // parity q.
 template <typename T>
@@ -907,16 +961,7 @@ cudaError_t enqueue_stage(const Plan &p, int q, int dir, int natural, cudaStream
         naturalize_kernel<T><<<grid, dim3(32, 8), 0, stream>>>((const NatDesc *)p.ndesc[q].p);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && p.tcount[dir]) {
-        if (sizeof(T) == 4) {
-            dim3 grid((unsigned)((p.tcols[dir] + 63) / 64), (unsigned)((p.trows[dir] + 63) / 64), (unsigned)p.tcount[dir]);
-            transpose_batch64_kernel<<<grid, dim3(16, 16), 0, stream>>>((const TDesc *)p.tdesc[dir].p);
-        } else {
-            dim3 grid((unsigned)((p.tcols[dir] + 31) / 32), (unsigned)((p.trows[dir] + 31) / 32), (unsigned)p.tcount[dir]);
-            transpose_batch_kernel<T><<<grid, dim3(32, 8), 0, stream>>>((const TDesc *)p.tdesc[dir].p);
-        }
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = enqueue_transposes<T>(p, dir, stream);
     // time-harmonic walls and forcing, in the layout the next stage reads
     if (e == cudaSuccess && p.hcount)
         e = launch_harmonic<T>((const HarmDesc *)p.hdesc.p, p.hcount, p.hmax, dir, stream);
@@ -1018,13 +1063,10 @@ int run_prologue_t(adi_sim *s) {
     }
     if (e == cudaSuccess)
         e = launch_prologue_lines<T>(cols, s->nlines[1], N, s->g.method, (const T *)s->pro.p, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_status(e);
     // the prologue wrote a column-major (A[3]), like a stage-2 launch
-    const Geometry &g = s->g;
-    int rc = transpose(s, s->A[3].p, g.ldu, g.rows_u, g.ldc, s->A[0].p, g.lda);
-    if (!rc) rc = cuda_status(cudaStreamSynchronize(s->stream));
-    return rc;
+    if (e == cudaSuccess) e = enqueue_transposes<T>(s->plan, 1, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    return cuda_status(e);
 }
 
 // One launch of the harmonic kernel for this simulation alone (mode 2 or 3).
@@ -1175,29 +1217,35 @@ int load_field(adi_sim *s, const void *staged, bool f32, void *dst, size_t rows,
     return cuda_status(cudaGetLastError());
 }
 
+template <typename T>
+int set_edges(adi_sim *s) {
+    const Geometry &g = s->g;
+    const int cur = s->parity;
+    EdgeRec<T> r;
+    r.u = (const T *)s->Uo.p; r.w = (const T *)s->Wo.p; r.v = (const T *)s->V[cur].p;
+    r.a1 = (T *)s->A[1].p; r.a2 = (T *)s->A[2].p; r.a3 = (T *)s->A[3].p;
+    r.w0 = (T *)s->W[0].p; r.w1 = (T *)s->W[1].p; r.vo = (T *)s->V[1 - cur].p;
+    r.rows_u = g.rows_u; r.ldu = g.ldu; r.rows_w = g.rows_w; r.ldw = g.ldw; r.rows_v = g.rows_v; r.ldv = g.ldv;
+    r.lda = g.lda; r.ldc = g.ldc; r.ldwc = g.ldwc; r.ldvp = g.ldvp;
+    const int n = std::max(std::max(g.rows_u, g.ldu), std::max(g.rows_w, g.ldv));
+    edges_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, s->stream>>>(r);
+    return cuda_status(cudaGetLastError());
+}
+
 // Loads natural fields (staged device copies from stage_fields; nullptr keeps the current
-// natural value, or zeros without keep_missing) into both ping-pong copies and rebuilds the
+// natural value, or zeros without keep_missing) and rebuilds the
 // carried state at the current parity with the prologue (so a member of a batch stays
 // consistent with the batch's plan).
 int load_state(adi_sim *s, const void *const staged[3], bool f32, bool keep_missing) {
     const Geometry &g = s->g;
-    const size_t esz = s->esz;
     const int cur = s->parity;
     int rc = ADI_OK;
     if (staged[1] || !keep_missing) rc = load_field(s, staged[1], f32, s->V[cur].p, g.rows_v, g.ldv, g.ldvp);
-    if (!rc) rc = cuda_status(cudaMemcpyAsync(s->V[1 - cur].p, s->V[cur].p, g.nVp() * esz, cudaMemcpyDeviceToDevice, s->stream));
     if (!rc && (staged[0] || !keep_missing)) rc = load_field(s, staged[0], f32, s->Uo.p, g.rows_u, g.ldu, g.ldu);
     if (!rc && (staged[2] || !keep_missing)) rc = load_field(s, staged[2], f32, s->Wo.p, g.rows_w, g.ldw, g.ldw);
     // with time-harmonic walls, u's walls are the harmonic data at the current time
     if (!rc) rc = harm_self(s, 2);
-    // all four carried-pressure arrays start from u (their outer rows/columns stay the
-    // Dirichlet data: line kernels write interior lines only)
-    for (int k = 0; k <= 2 && !rc; k += 2)
-        rc = cuda_status(cudaMemcpy2DAsync(s->A[k].p, g.lda * esz, s->Uo.p, g.ldu * esz, g.ldu * esz, g.rows_u,
-                                           cudaMemcpyDeviceToDevice, s->stream));
-    for (int k = 1; k <= 3 && !rc; k += 2) rc = transpose(s, s->Uo.p, g.rows_u, g.ldu, g.ldu, s->A[k].p, g.ldc);
-    for (int k = 0; k < 2 && !rc; ++k) rc = transpose(s, s->Wo.p, g.rows_w, g.ldw, g.ldw, s->W[k].p, g.ldwc);
-    if (!rc) rc = cuda_status(cudaStreamSynchronize(s->stream));
+    if (!rc) rc = s->precision == ADI_FP64 ? set_edges<double>(s) : set_edges<float>(s);
     if (!rc) rc = upload_sim_descs(s);  // descriptors of the current parity
     if (!rc) rc = prologue(s);
     return rc;

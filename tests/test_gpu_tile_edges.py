@@ -72,6 +72,27 @@ def test_line_lengths_at_path_changes(adi, method, n, fp64):
     _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, 3, source=src), fp64)
 
 
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("method,nx,ny", [(CFD, 33, 31), (CFD, 40, 32), (CFD, 31, 33), (CFD, 65, 64), (CFD, 34, 95),
+                                          (CFD, 31, 97), (CFD, 33, 130), (MFD, 33, 31), (MFD, 64, 66)])
+def test_loading_fields_mid_run(adi, method, nx, ny, fp64):
+    """New fields loaded into a simulation that has stepped an odd number of steps: the carried state is rebuilt
+    from them (chunks of 32 rows of every line) and nothing of the old fields is left in the arrays."""
+    h, dt, c, U, V, W = _case(method, nx, ny, 7)
+    U2, V2, W2 = _case(method, nx, ny, 8)[3:]
+    sim = adi.Sim(method, nx, ny, h, dt, c, U, V, W, precision=adi.ADI_FP64 if fp64 else adi.ADI_FP32)
+    sim.step(3)
+    if fp64:
+        sim.set_fields(U2, V2, W2)
+    else:
+        sim.set_fields_f32(*[np.ascontiguousarray(a, dtype=np.float32) for a in (U2, V2, W2)])
+    _check(sim.read(), (U2, V2, W2), fp64)
+    sim.step(2)
+    G = sim.read()
+    sim.close()
+    _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U2, V2, W2, 2), fp64)
+
+
 # line counts around a block's four lines; lines so long that a block takes two (FP64 above 7260 cells, FP32 above
 # 14520) or one (FP64 above 14520), or keeps its rows in global memory (FP64 above 28900, FP32 above 57800); the
 # recurrences go sixteen rows at a time
