@@ -380,42 +380,58 @@ struct NatDesc {
     double dt, src_amp, src_f0, src_td, src_scale;
 };
 
-// blockIdx.z: the member; a 32 x 32 tile of (row k, column j) per block.  The carried arrays are
-// read along their columns (lane = row) and the natural ones written along their rows (lane =
-// column), through shared memory, so both sides are coalesced.
+// blockIdx.z: the member; a tile of 64 rows k and 32 columns j per block.  The carried arrays are
+// read along their columns in 16-byte loads (leading dimensions are multiples of 32 elements, so a load
+// that starts inside a column's leading dimension stays there) and the natural ones written along their
+// rows (lane = column), through shared memory, so both sides are coalesced.  Bound by memory: every
+// thread has 8 (FP32) or 16 (FP64) such loads in flight; with 32 x 32 tiles of single elements 4096^2 took 231
+// us, now 64 us (403 MB).
+constexpr int kNatRows = 64;
 template <typename T>
-__global__ void naturalize_kernel(const NatDesc *__restrict__ nd) {
-    __shared__ T tu[32][33], tw[32][33];
-    const NatDesc d = nd[blockIdx.z];
-    const int k0 = blockIdx.y * 32, jb = blockIdx.x * 32;
-    if (k0 >= max(d.ku1, d.kw1) || jb >= d.j1) return;  // uniform over the block
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const T *a = (const T *)d.a, *c = (const T *)d.c, *wn = (const T *)d.wn, *wi = (const T *)d.wi;
-    T src = T(0);
-    if (d.src_j >= 0)
-        src = (T)(d.src_scale *
-                  ricker(d.src_amp, d.src_f0, d.src_td, (double)(*d.clock + d.clock_ahead) * d.dt));
-    for (int jj = ty; jj < 32; jj += 8) {
-        const int j = jb + jj, k = k0 + tx;
-        if (j < 1 || j >= d.j1) continue;
-        if (k >= d.ku0 && k < d.ku1) {
-            const long long o = (long long)j * d.ldc + k;
-            T u = T(0.5) * (a[o] + c[o]);
-            if (k == d.src_i && j == d.src_j) u -= T(0.5) * src;
-            tu[jj][tx] = u;
+__global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restrict__ nd) {
+    constexpr int V = 16 / sizeof(T), KV = kNatRows / V;
+    struct alignas(16) Vec { T x[V]; };
+    __shared__ T tu[32][kNatRows + 1], tw[32][kNatRows + 1];
+    const NatDesc &d = nd[blockIdx.z];
+    const int k0 = blockIdx.y * kNatRows, jb = blockIdx.x * 32, j1 = d.j1, ku1 = d.ku1, kw1 = d.kw1;
+    if (k0 >= max(ku1, kw1) || jb >= j1) return;  // uniform over the block
+    const T *__restrict__ a = (const T *)d.a, *__restrict__ c = (const T *)d.c;
+    const T *__restrict__ wn = (const T *)d.wn, *__restrict__ wi = (const T *)d.wi;
+    const long long ldc = d.ldc, ldwc = d.ldwc;
+#pragma unroll
+    for (int q = threadIdx.x; q < 32 * KV; q += 256) {
+        const int jj = q / KV, kv = (q % KV) * V, j = jb + jj, k = k0 + kv;
+        if (j < 1 || j >= j1) continue;
+        Vec va{}, vc{}, vn{}, vi{};
+        if (k < ku1) {
+            va = *reinterpret_cast<const Vec *>(a + j * ldc + k);
+            vc = *reinterpret_cast<const Vec *>(c + j * ldc + k);
         }
-        if (k < d.kw1) {
-            const long long o = (long long)j * d.ldwc + k;
-            tw[jj][tx] = T(0.5) * (wn[o] + wi[o]);
+        if (k < kw1) {
+            vn = *reinterpret_cast<const Vec *>(wn + j * ldwc + k);
+            vi = *reinterpret_cast<const Vec *>(wi + j * ldwc + k);
+        }
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            tu[jj][kv + i] = T(0.5) * (va.x[i] + vc.x[i]);
+            tw[jj][kv + i] = T(0.5) * (vn.x[i] + vi.x[i]);
         }
     }
     __syncthreads();
     T *uo = (T *)d.uo, *wo = (T *)d.wo;
-    for (int kk = ty; kk < 32; kk += 8) {
-        const int k = k0 + kk, j = jb + tx;
-        if (j < 1 || j >= d.j1) continue;
-        if (k >= d.ku0 && k < d.ku1) uo[(long long)k * d.ldu + j] = tu[tx][kk];
-        if (k < d.kw1) wo[(long long)k * d.ldw + j] = tw[tx][kk];
+    const int j = jb + (threadIdx.x & 31), ku0 = d.ku0, ldu = d.ldu, ldw = d.ldw, src_i = j == d.src_j ? d.src_i : -1;
+    if (j < 1 || j >= j1) return;
+#pragma unroll
+    for (int kk = threadIdx.x >> 5; kk < kNatRows; kk += 8) {
+        const int k = k0 + kk;
+        if (k >= ku0 && k < ku1) {
+            T u = tu[threadIdx.x & 31][kk];
+            if (k == src_i)  // the point source's dt/2 f is not part of u
+                u -= T(0.5) * (T)(d.src_scale * ricker(d.src_amp, d.src_f0, d.src_td,
+                                                       (double)(*d.clock + d.clock_ahead) * d.dt));
+            uo[(long long)k * ldu + j] = u;
+        }
+        if (k < kw1) wo[(long long)k * ldw + j] = tw[threadIdx.x & 31][kk];
     }
 }
 
@@ -957,8 +973,8 @@ cudaError_t enqueue_stage(const Plan &p, int q, int dir, int natural, cudaStream
     if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, stream);
     // natural u and w from the carried state, before anything moves or changes it
     if (e == cudaSuccess && nat && p.ncount) {
-        dim3 grid((unsigned)((p.ncols + 31) / 32), (unsigned)((p.nrows + 31) / 32), (unsigned)p.ncount);
-        naturalize_kernel<T><<<grid, dim3(32, 8), 0, stream>>>((const NatDesc *)p.ndesc[q].p);
+        dim3 grid((unsigned)((p.ncols + 31) / 32), (unsigned)((p.nrows + kNatRows - 1) / kNatRows), (unsigned)p.ncount);
+        naturalize_kernel<T><<<grid, 256, 0, stream>>>((const NatDesc *)p.ndesc[q].p);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = enqueue_transposes<T>(p, dir, stream);
