@@ -365,53 +365,6 @@ __device__ bool fac_rhs_coeffs(const LineDesc<TS> &d, int i, int op, int ov, int
     return ok;
 }
 
-// Gauss-Jordan inverse with partial pivoting of an n x n matrix (n <= 13, destroyed) by one warp: lane
-// j holds column j of [A | R] (R starts as the identity); the same operations in the same order as
-// small_inverse.
-__device__ inline bool warp_inverse(double *A, int n, double *R, int lane) {
-    double scale = 0.0;
-    for (int i = lane; i < n * n; i += 32) {
-        R[i] = (i / n == i % n) ? 1.0 : 0.0;
-        scale = fmax(scale, fabs(A[i]));
-    }
-    for (int o = 16; o > 0; o >>= 1) scale = fmax(scale, __shfl_xor_sync(0xffffffffu, scale, o));
-    __syncwarp();
-    double *col = lane < n ? A + lane : R + (lane - n);  // this lane's column, stride n
-    const bool mine = lane < 2 * n;
-    for (int c = 0; c < n; ++c) {
-        double f[13];
-        int p = c;
-        double best = fabs(A[c * n + c]);
-#pragma unroll
-        for (int i = 0; i < 13; ++i) {
-            f[i] = i < n ? A[i * n + c] : 0.0;
-            if (i > c && i < n && fabs(f[i]) > best) { best = fabs(f[i]); p = i; }
-        }
-        if (!(best > 1e-13 * scale)) return false;  // uniform over the warp
-        __syncwarp();  // column c has been read
-        if (mine) {
-            const double ap = col[p * n], ac = col[c * n];
-            double fp = 0.0, fc = 0.0;
-#pragma unroll
-            for (int i = 0; i < 13; ++i) {
-                if (i == p) fp = f[i];
-                if (i == c) fc = f[i];
-            }
-            const double row = ap * (1.0 / fp);
-            if (p != c) col[p * n] = ac;
-            col[c * n] = row;
-#pragma unroll
-            for (int i = 0; i < 13; ++i) {
-                if (i >= n || i == c) continue;
-                const double fi = i == p ? fc : f[i];  // rows p and c are swapped
-                if (fi != 0.0) col[i * n] -= fi * row;
-            }
-        }
-        __syncwarp();
-    }
-    return true;
-}
-
 // Dense elimination of one end region (end 0: head, 1: tail) into its table by one warp, in its
 // shared workspace ws (kFacWs doubles); dB of the end (bs x bs, row-major) is also returned in FP64
 // in dBo (global memory).  False if the region is singular.

@@ -52,14 +52,14 @@ cudaError_t launch_precompute(const LineDesc<T> *d, int nlines, T *tab_out_base,
 template <typename T>
 cudaError_t launch_line_solve_v1(const LineDesc<T> *d, int nlines, T *scratch,
                                  long long scratch_stride, int write_natural, cudaStream_t s);
-// fac: the Thomas factors of prologue_factors() in T, or nullptr (formed on the fly; the
-// scratch then holds two vectors per line)
+// The same lines with one warp each (lines of at most kV1ShortCells cells, all of one method and N).
+constexpr int kV1ShortCells = 128;
 template <typename T>
-cudaError_t launch_prologue(const LineDesc<T> *col_lines, int nlines, const T *fac, T *scratch,
-                            long long scratch_stride, cudaStream_t s);
+cudaError_t launch_line_solve_short(const LineDesc<T> *d, int nlines, int method, int N, int write_natural, cudaStream_t s);
 // CFD: 3 (N+1) + 3 (N-1) Thomas factors of P and Pbar, then the start-up factors of the
 // chunked solves (prologue_factor_count(N) values in all)
 void prologue_factors(int N, std::vector<double> &out);
+void prologue_factors(int N, double *out);
 size_t prologue_factor_count(int N);
 // The prologue over the y-lines of one simulation (N cells each), spread over the lines' elements;
 // fac: the Thomas factors of prologue_factors() in T (CFD; nullptr for MFD).

@@ -23,65 +23,63 @@
 
 namespace adi {
 
-// One thread per line: head and tail elimination tables.
+// Head and tail elimination tables, one warp per (line, end): the entries of the eliminated rows, their
+// inverse and the products spread over the lanes.  (One thread per line took 221 us for the 126 lines of a
+// 64 x 64 grid, a chain of some 150 evaluated entries and two 5 x 5 inversions each; this 14 us.)
+constexpr int kTabWarps = 4;
 template <typename T>
-__global__ void precompute_kernel(const LineDesc<T> *__restrict__ descs, int nlines,
-                                  T *tab_out_base, int *status) {
-    int line = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32 * kTabWarps) precompute_kernel(const LineDesc<T> *__restrict__ descs, int nlines,
+                                                                    T *tab_out_base, int *status) {
+    __shared__ double ws[kTabWarps][4 * 36];
+    const int lane = threadIdx.x & 31, job = blockIdx.x * kTabWarps + (threadIdx.x >> 5), line = job >> 1, end = job & 1;
     if (line >= nlines) return;
-    const LineDesc<T> d = descs[line];
+    const LineDesc<T> &d = descs[line];
     const LineShape s = line_shape(d.method, d.N);
-    T *tab = tab_out_base + (size_t)line * kTabLine;
+    T *t = tab_out_base + (size_t)line * kTabLine + end * kTabEnd;
     const int bs = s.bs;
-    for (int end = 0; end < 2; ++end) {
-        const int m = end == 0 ? s.hu : s.tu;
-        // index ranges: region R (the m eliminated unknowns), adjacent block J (bs)
-        const int r0 = end == 0 ? 0 : s.nunk - s.tu;
-        const int j0 = end == 0 ? s.hu : s.nunk - s.tu - bs;
-        double H[36], Hi[36], E[18], F[18];
-        for (int i = 0; i < m; ++i)
-            for (int j = 0; j < m; ++j) H[i * m + j] = line_entry(d, r0 + i, r0 + j);
-        for (int i = 0; i < m; ++i)
-            for (int j = 0; j < bs; ++j) E[i * bs + j] = line_entry(d, r0 + i, j0 + j);
-        for (int i = 0; i < bs; ++i)
-            for (int j = 0; j < m; ++j) F[i * m + j] = line_entry(d, j0 + i, r0 + j);
-        if (!small_inverse(H, m, Hi)) { atomicExch(status, 1); return; }
-        T *t = tab + end * kTabEnd;
-        for (int i = 0; i < m * m; ++i) t[kTabHinv + i] = (T)Hi[i];
-        double HiE[18];
-        for (int i = 0; i < m; ++i)
-            for (int j = 0; j < bs; ++j) {
-                double acc = 0.0;
-                for (int k = 0; k < m; ++k) acc += Hi[i * m + k] * E[k * bs + j];
-                HiE[i * bs + j] = acc;
-                t[kTabHinvE + i * bs + j] = (T)acc;
-            }
-        for (int i = 0; i < bs; ++i)
-            for (int j = 0; j < m; ++j) {
-                double acc = 0.0;
-                for (int k = 0; k < m; ++k) acc += F[i * m + k] * Hi[k * m + j];
-                t[kTabK + i * m + j] = (T)acc;
-            }
-        for (int i = 0; i < bs; ++i)
-            for (int j = 0; j < bs; ++j) {
-                double acc = 0.0;
-                for (int k = 0; k < m; ++k) acc += F[i * m + k] * HiE[k * bs + j];
-                t[kTabDB + i * bs + j] = (T)acc;
-            }
+    const int m = end == 0 ? s.hu : s.tu;
+    // index ranges: region R (the m eliminated unknowns), adjacent block J (bs)
+    const int r0 = end == 0 ? 0 : s.nunk - s.tu;
+    const int j0 = end == 0 ? s.hu : s.nunk - s.tu - bs;
+    double *H = ws[threadIdx.x >> 5], *Hi = H + 36, *E = Hi + 36, *F = E + 18, *HiE = F + 18;
+    for (int i = lane; i < m * m; i += 32) H[i] = line_entry(d, r0 + i / m, r0 + i % m);
+    for (int i = lane; i < m * bs; i += 32) E[i] = line_entry(d, r0 + i / bs, j0 + i % bs);
+    for (int i = lane; i < bs * m; i += 32) F[i] = line_entry(d, j0 + i / m, r0 + i % m);
+    __syncwarp();
+    if (!warp_inverse(H, m, Hi, lane)) {
+        if (lane == 0) atomicExch(status, 1);
+        return;
+    }
+    for (int i = lane; i < m * m; i += 32) t[kTabHinv + i] = (T)Hi[i];
+    for (int i = lane; i < m * bs; i += 32) {
+        double acc = 0.0;
+        for (int k = 0; k < m; ++k) acc += Hi[(i / bs) * m + k] * E[k * bs + i % bs];
+        HiE[i] = acc;
+        t[kTabHinvE + i] = (T)acc;
+    }
+    for (int i = lane; i < bs * m; i += 32) {
+        double acc = 0.0;
+        for (int k = 0; k < m; ++k) acc += F[(i / m) * m + k] * Hi[k * m + i % m];
+        t[kTabK + i] = (T)acc;
+    }
+    __syncwarp();
+    for (int i = lane; i < bs * bs; i += 32) {
+        double acc = 0.0;
+        for (int k = 0; k < m; ++k) acc += F[(i / bs) * m + k] * HiE[k * bs + i % bs];
+        t[kTabDB + i] = (T)acc;
     }
 }
 
 // ---------------------------------------------------------------------------------------
 // Thread-per-line solver.
 // ---------------------------------------------------------------------------------------
-size_t v1_scratch_words(int method, int N) {
-    LineShape s = line_shape(method, N);
-    return (size_t)s.nunk + (size_t)s.nb * (s.bs * s.bs + s.bs);
-}
+__host__ __device__ inline int v1_words(const LineShape &s) { return s.nunk + s.nb * (s.bs * s.bs + s.bs); }
+size_t v1_scratch_words(int method, int N) { return (size_t)v1_words(line_shape(method, N)); }
 
-template <typename T, int BS>
-__device__ void solve_line_v1(const LineDesc<T> &d, T *scr, long long st, int write_natural) {
-    const Line<T> L(d);
+// LANES = 1: one thread, its scratch in global memory with stride st.  LANES = 32: one warp whose line is staged
+// in shared memory (L), with unit stride; the two sweeps are lane 0's, everything else is spread over the lanes.
+template <typename T, int BS, int LANES>
+__device__ void solve_line_v1(const LineDesc<T> &d, const Line<T> &L, T *scr, long long st, int lane, int write_natural) {
     const LineShape s = line_shape(d.method, d.N);
     const int N = d.N, hu = s.hu, tu = s.tu, nb = s.nb, nunk = s.nunk;
     auto X = [&](int k) -> T & { return scr[(long long)k * st]; };
@@ -89,10 +87,19 @@ __device__ void solve_line_v1(const LineDesc<T> &d, T *scr, long long st, int wr
     auto Y = [&](int b, int i) -> T & { return scr[(long long)(nunk + nb * BS * BS + b * BS + i) * st]; };
     const T *th = d.tab, *tt = d.tab + kTabEnd;
 
-    T rH[6], rT[6];
-    for (int i = 0; i < hu; ++i) rH[i] = rhs_row(L, i);
-    for (int i = 0; i < tu; ++i) rT[i] = rhs_row(L, nunk - tu + i);
+    // right-hand sides of the two end regions
+    T reg[LANES == 1 ? 12 : 1];
+    T *rH = LANES == 1 ? reg : scr + v1_words(s), *rT = rH + 6;
+    if constexpr (LANES == 1) {
+        for (int i = 0; i < hu; ++i) rH[i] = rhs_row(L, i);
+        for (int i = 0; i < tu; ++i) rT[i] = rhs_row(L, nunk - tu + i);
+    } else {
+        if (lane < hu) rH[lane] = rhs_row(L, lane);
+        if (lane >= 16 && lane - 16 < tu) rT[lane - 16] = rhs_row(L, nunk - tu + lane - 16);
+        __syncwarp();
+    }
 
+    if (lane == 0) {
     // forward sweep
     T Gp[BS][BS], yp[BS];
 #pragma unroll
@@ -170,20 +177,24 @@ __device__ void solve_line_v1(const LineDesc<T> &d, T *scr, long long st, int wr
 #pragma unroll
         for (int i = 0; i < BS; ++i) { xn[i] = x[i]; X(hu + b * BS + i) = x[i]; }
     }
+    }
+    if constexpr (LANES > 1) __syncwarp();
     // eliminated head/tail unknowns
-    for (int i = 0; i < hu; ++i) {
+    for (int i = lane; i < hu; i += LANES) {
         T acc = T(0);
         for (int k = 0; k < hu; ++k) acc += th[kTabHinv + i * hu + k] * rH[k];
         for (int k = 0; k < BS; ++k) acc -= th[kTabHinvE + i * BS + k] * X(hu + k);
         X(i) = acc;
     }
     const int lb = hu + (nb - 1) * BS;
-    for (int i = 0; i < tu; ++i) {
+    for (int i = lane; i < tu; i += LANES) {
         T acc = T(0);
         for (int k = 0; k < tu; ++k) acc += tt[kTabHinv + i * tu + k] * rT[k];
         for (int k = 0; k < BS; ++k) acc -= tt[kTabHinvE + i * BS + k] * X(lb + k);
         X(nunk - tu + i) = acc;
     }
+
+    if constexpr (LANES > 1) __syncwarp();
 
     // source term dt/2 f(t_{m+1}) at the source point of this line
     T src = T(0);
@@ -191,21 +202,22 @@ __device__ void solve_line_v1(const LineDesc<T> &d, T *scr, long long st, int wr
         long long m = *d.clock;
         double t1 = (double)(m + 1) * d.dt;
         src = (T)(d.src_scale * ricker(d.src_amp, d.src_f0, d.src_tdelay, t1));
-        if (d.advance_clock) *d.clock = m + 1;
+        if constexpr (LANES > 1) __syncwarp();  // every lane has read the clock
+        if (d.advance_clock && lane == 0) *d.clock = m + 1;
     }
 
     // epilogue: carried outputs (and natural outputs on request)
     const T beta = (T)d.beta;
     if (d.method == kCFD) {
-        for (int j = 0; j <= N; ++j) {
+        for (int j = lane; j <= N; j += LANES) {
             T g = X(cfd_idx_g(N, j));
-            T vin = d.v[j * d.sv];
+            T vin = L.v(j);
             d.vo[j * d.svo] = vin - T(2) * beta * g;
             if (write_natural && d.w_out) d.w_out[j * d.snv] = vin - beta * g;
         }
-        for (int j = 1; j <= N - 1; ++j) {
+        for (int j = 1 + lane; j <= N - 1; j += LANES) {
             T e = X(cfd_idx_e(j));
-            T pin = d.p[j * d.sp];
+            T pin = L.p(j);
             T ae = L.al(j) * e;
             d.po[j * d.spo] = pin - T(2) * ae + (j == d.src_k ? src : T(0));
             if (write_natural && d.u_out) d.u_out[j * d.snp] = pin - ae;
@@ -213,7 +225,7 @@ __device__ void solve_line_v1(const LineDesc<T> &d, T *scr, long long st, int wr
     } else {
         const T ih = (T)d.inv_h;
         const T p0 = L.p(0), pl = L.p(N + 1);
-        for (int j = 0; j <= N; ++j) {
+        for (int j = lane; j <= N; j += LANES) {
             double gw[8];
             int g0;
             int ng = mfd_G_row(N, j, &g0, gw);
@@ -224,13 +236,13 @@ __device__ void solve_line_v1(const LineDesc<T> &d, T *scr, long long st, int wr
                 acc += (T)gw[t] * uk;
             }
             T gu = acc * ih;
-            T vin = d.v[j * d.sv];
+            T vin = L.v(j);
             d.vo[j * d.svo] = vin - T(2) * beta * gu;
             if (write_natural && d.w_out) d.w_out[j * d.snv] = vin - beta * gu;
         }
-        for (int c = 1; c <= N; ++c) {
+        for (int c = 1 + lane; c <= N; c += LANES) {
             T u = X(c - 1);
-            T pin = d.p[c * d.sp];
+            T pin = L.p(c);
             d.po[c * d.spo] = T(2) * u - pin + (c == d.src_k ? src : T(0));
             if (write_natural && d.u_out) d.u_out[c * d.snp] = u;
         }
@@ -245,14 +257,37 @@ __global__ void __launch_bounds__(128) line_solve_v1_kernel(const LineDesc<T> *_
     if (line >= nlines) return;
     const LineDesc<T> d = descs[line];
     T *scr = scratch + line;
+    const Line<T> L(d);
     if (d.method == kCFD)
-        solve_line_v1<T, 2>(d, scr, st, write_natural);
+        solve_line_v1<T, 2, 1>(d, L, scr, st, 0, write_natural);
     else
-        solve_line_v1<T, 3>(d, scr, st, write_natural);
+        solve_line_v1<T, 3, 1>(d, L, scr, st, 0, write_natural);
+}
+
+// Short lines (at most kV1ShortCells cells): one warp per line, the line and the factors in shared memory.  So few
+// lines leave the GPU idle and each is a chain of dependent steps; with a thread per line every step of
+// the chain waits for global memory (64 lines of 64 cells 71 us, this 14 us).
+template <typename T>
+__global__ void __launch_bounds__(32) line_solve_short_kernel(const LineDesc<T> *__restrict__ descs, int write_natural) {
+    extern __shared__ __align__(16) unsigned char v1_smem[];
+    const LineDesc<T> &d = descs[blockIdx.x];
+    const int lane = threadIdx.x, N = d.N, np = p_last(d.method, N) + 1;
+    T *P = (T *)v1_smem, *Al = P + np, *V = Al + np, *scr = V + N + 1;
+    for (int k = lane; k < np; k += 32) {
+        P[k] = d.p[k * d.sp];
+        Al[k] = d.alpha[k * d.sp];
+    }
+    for (int k = lane; k <= N; k += 32) V[k] = d.v[k * d.sv];
+    __syncwarp();
+    const Line<T> L(d, P, V, Al);
+    if (d.method == kCFD)
+        solve_line_v1<T, 2, 32>(d, L, scr, 1, lane, write_natural);
+    else
+        solve_line_v1<T, 3, 32>(d, L, scr, 1, lane, write_natural);
 }
 
 // ---------------------------------------------------------------------------------------
-// Prologue: carried state from natural fields, one thread per stage-2 (y) line.
+// Prologue: carried state from natural fields, along the stage-2 (y) lines.
 //   a_k  = u_k - alpha_k (Dv w)_k + dt/2 f(t_m)   (interior pressure points) -> d.po
 //   w*_j = w_j - beta (Du u)_j                      (all velocity points)     -> d.v
 // (d.po of a stage-2 line is the stage-1 input buffer; d.v is the stage-2 input; the
@@ -260,125 +295,7 @@ __global__ void __launch_bounds__(128) line_solve_v1_kernel(const LineDesc<T> *_
 // CFD derivatives solve Pbar e = Qbar w and P g = Q u by the Thomas algorithm, with the
 // factors of the two constant matrices precomputed (fac: P's sub-diagonal, eliminated
 // super-diagonal and inverse pivots, N+1 each, then Pbar's, N-1 each).
-// ---------------------------------------------------------------------------------------
-template <typename T>
-__device__ void thomas_apply(int n, T *rhs, long long st, const T *__restrict__ lo, const T *__restrict__ cu,
-                             const T *__restrict__ id) {
-    // Solves the n-row system in place: forward d_r = (rhs_r - lo_r d_{r-1}) / den_r, then
-    // x_r = d_r - c_r x_{r+1}; the running value stays in a register.
-    T d = rhs[0] * id[0];
-    rhs[0] = d;
-    for (int r = 1; r < n; ++r) {
-        d = (rhs[(long long)r * st] - lo[r] * d) * id[r];
-        rhs[(long long)r * st] = d;
-    }
-    T x = d;
-    for (int r = n - 2; r >= 0; --r) {
-        x = rhs[(long long)r * st] - cu[r] * x;
-        rhs[(long long)r * st] = x;
-    }
-}
-
-// Without precomputed factors (fac == nullptr): the same elimination with each row's factors
-// formed on the fly, the eliminated super-diagonal kept in cs (stride st).
-template <typename T>
-__device__ void thomas_rows(int N, bool reduced, T *rhs, T *cs, long long st) {
-    const int n = reduced ? N - 1 : N + 1;
-    double w[8];
-    int c0;
-    T cprev = T(0), d = T(0);
-    for (int r = 0; r < n; ++r) {
-        if (reduced) cfd_Pbar_row(N, r + 1, &c0, w); else cfd_P_row(N, r, &c0, w);
-        T lo = T(0), di, up = T(0);
-        if (r == 0) { di = (T)w[0]; up = (T)w[1]; }
-        else if (r == n - 1) { lo = (T)w[0]; di = (T)w[1]; }
-        else { lo = (T)w[0]; di = (T)w[1]; up = (T)w[2]; }
-        const T den = di - lo * cprev;
-        cprev = up / den;
-        d = (rhs[(long long)r * st] - lo * d) / den;
-        cs[(long long)r * st] = cprev;
-        rhs[(long long)r * st] = d;
-    }
-    T x = d;
-    for (int r = n - 2; r >= 0; --r) {
-        x = rhs[(long long)r * st] - cs[(long long)r * st] * x;
-        rhs[(long long)r * st] = x;
-    }
-}
-
-template <typename T>
-__global__ void prologue_kernel(const LineDesc<T> *__restrict__ descs, int nlines, T *scratch,
-                                long long st, const T *__restrict__ fac) {
-    int line = blockIdx.x * blockDim.x + threadIdx.x;
-    if (line >= nlines) return;
-    const LineDesc<T> d = descs[line];
-    const int N = d.N;
-    const T ih = (T)d.inv_h, beta = (T)d.beta;
-    T *scr = scratch + line;
-    auto S = [&](int k) -> T & { return scr[(long long)k * st]; };
-    const T *un = d.u_out;  // natural u along the line (same indexing as p)
-    const T *wn = d.w_out;  // natural w along the line (same indexing as v)
-    double w[8];
-    int c0;
-    T src = T(0);
-    if (d.src_k >= 0) {
-        double t = (double)(*d.clock) * d.dt;
-        src = (T)(d.src_scale * ricker(d.src_amp, d.src_f0, d.src_tdelay, t));
-    }
-    const long long snp = d.snp, snv = d.snv, spo = d.spo;
-    if (d.method == kCFD) {
-        // g = P^{-1} Q u  (slots 0..N), then w* = w - beta g
-        for (int j = 0; j <= N; ++j) {
-            int n = cfd_Q_row(N, j, &c0, w);
-            T acc = T(0);
-            for (int t = 0; t < n; ++t) acc += (T)w[t] * un[(c0 + t) * snp];
-            S(j) = acc * ih;
-        }
-        if (fac) thomas_apply<T>(N + 1, scr, st, fac, fac + (N + 1), fac + 2 * (N + 1));
-        else thomas_rows<T>(N, false, scr, scr + (long long)(N + 1) * st, st);
-        for (int j = 0; j <= N; ++j) d.v[j * d.sv] = wn[j * snv] - beta * S(j);
-        // e = Pbar^{-1} Qbar w  (slots 0..N-2 for nodes 1..N-1), then a = u - alpha e
-        for (int j = 1; j <= N - 1; ++j) {
-            int n = cfd_Qbar_row(N, j, &c0, w);
-            T acc = T(0);
-            for (int t = 0; t < n; ++t) acc += (T)w[t] * wn[(c0 + t) * snv];
-            S(j - 1) = acc * ih;
-        }
-        if (fac) {
-            const T *fb = fac + 3 * (N + 1);
-            thomas_apply<T>(N - 1, scr, st, fb, fb + (N - 1), fb + 2 * (N - 1));
-        } else {
-            thomas_rows<T>(N, true, scr, scr + (long long)(N + 1) * st, st);
-        }
-        for (int j = 1; j <= N - 1; ++j) {
-            T val = un[j * snp] - d.alpha[j * d.sp] * S(j - 1);
-            if (j == d.src_k) val += src;
-            d.po[j * spo] = val;
-        }
-        d.po[0] = un[0];
-        d.po[(long long)N * spo] = un[(long long)N * snp];
-    } else {
-        for (int j = 0; j <= N; ++j) {
-            int n = mfd_G_row(N, j, &c0, w);
-            T acc = T(0);
-            for (int t = 0; t < n; ++t) acc += (T)w[t] * un[(c0 + t) * snp];
-            d.v[j * d.sv] = wn[j * snv] - beta * acc * ih;
-        }
-        for (int c = 1; c <= N; ++c) {
-            int n = mfd_D_row(N, c - 1, &c0, w);
-            T acc = T(0);
-            for (int t = 0; t < n; ++t) acc += (T)w[t] * wn[(c0 + t) * snv];
-            T val = un[c * snp] - d.alpha[c * d.sp] * acc * ih;
-            if (c == d.src_k) val += src;
-            d.po[c * spo] = val;
-        }
-        d.po[0] = un[0];
-        d.po[(long long)(N + 1) * spo] = un[(long long)(N + 1) * snp];
-    }
-}
-
-// ---------------------------------------------------------------------------------------
-// The same prologue spread over the lines' elements.  prologue_mfd_kernel: MFD, block (32 lines, 8
+// Spread over the lines' elements: prologue_mfd_kernel: MFD, block (32 lines, 8
 // elements).  prologue_cfd_kernel: CFD, the two Thomas solves with the precomputed factors, one thread
 // per chunk of a line, the right-hand sides formed as the sweeps need them.
 // ---------------------------------------------------------------------------------------
@@ -681,8 +598,8 @@ template <typename T>
 cudaError_t launch_precompute(const LineDesc<T> *d, int nlines, T *tab, int *status,
                               cudaStream_t s) {
     if (nlines <= 0) return cudaSuccess;
-    int tpb = 64;
-    precompute_kernel<T><<<(nlines + tpb - 1) / tpb, tpb, 0, s>>>(d, nlines, tab, status);
+    const int jobs = 2 * nlines;
+    precompute_kernel<T><<<(jobs + kTabWarps - 1) / kTabWarps, 32 * kTabWarps, 0, s>>>(d, nlines, tab, status);
     return cudaGetLastError();
 }
 template <typename T>
@@ -695,11 +612,11 @@ cudaError_t launch_line_solve_v1(const LineDesc<T> *d, int nlines, T *scratch, l
     return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_prologue(const LineDesc<T> *d, int nlines, const T *fac, T *scratch, long long st,
-                            cudaStream_t s) {
+cudaError_t launch_line_solve_short(const LineDesc<T> *d, int nlines, int method, int N, int write_natural, cudaStream_t s) {
     if (nlines <= 0) return cudaSuccess;
-    int tpb = 128;
-    prologue_kernel<T><<<(nlines + tpb - 1) / tpb, tpb, 0, s>>>(d, nlines, scratch, st, fac);
+    if (N > kV1ShortCells) return cudaErrorInvalidValue;
+    const size_t words = 2 * (p_last(method, N) + 1) + N + 1 + v1_scratch_words(method, N) + 12;
+    line_solve_short_kernel<T><<<nlines, 32, words * sizeof(T), s>>>(d, write_natural);
     return cudaGetLastError();
 }
 
@@ -722,10 +639,13 @@ cudaError_t launch_prologue_lines(const LineDesc<T> *d, int nlines, int N, int m
 size_t prologue_factor_count(int N) { return (size_t)3 * (N + 1) + 3 * (N - 1) + kProH; }
 void prologue_factors(int N, std::vector<double> &out) {
     out.assign(prologue_factor_count(N), 0.0);
+    prologue_factors(N, out.data());
+}
+void prologue_factors(int N, double *out) {
     // start-up factors of a window that begins on an interior row (no predecessor): 1 / den_k with
     // den_0 = 4, den_k = 4 - 1 / den_{k-1}
     {
-        double *su = out.data() + 3 * (N + 1) + 3 * (N - 1), den = 4.0;
+        double *su = out + 3 * (N + 1) + 3 * (N - 1), den = 4.0;
         for (int k = 0; k < kProH; ++k) {
             su[k] = 1.0 / den;
             den = 4.0 - su[k];
@@ -733,7 +653,7 @@ void prologue_factors(int N, std::vector<double> &out) {
     }
     for (int bar = 0; bar < 2; ++bar) {
         const int n = bar ? N - 1 : N + 1;
-        double *lo = out.data() + (bar ? 3 * (N + 1) : 0), *cu = lo + n, *id = cu + n;
+        double *lo = out + (bar ? 3 * (N + 1) : 0), *cu = lo + n, *id = cu + n;
         double cprev = 0.0;
         for (int r = 0; r < n; ++r) {
             double w[8];
@@ -765,8 +685,7 @@ cudaError_t launch_finite_check(const T *x, size_t n, int *flag, cudaStream_t s)
                                               cudaStream_t);                                 \
     template cudaError_t launch_line_solve_v1<T>(const LineDesc<T> *, int, T *, long long,   \
                                                  int, cudaStream_t);                         \
-    template cudaError_t launch_prologue<T>(const LineDesc<T> *, int, const T *, T *, long long,  \
-                                            cudaStream_t);                                         \
+    template cudaError_t launch_line_solve_short<T>(const LineDesc<T> *, int, int, int, int, cudaStream_t); \
     template cudaError_t launch_prologue_lines<T>(const LineDesc<T> *, int, int, int, const T *, cudaStream_t); \
     template cudaError_t launch_finite_check<T>(const T *, size_t, int *, cudaStream_t);
 ADI_INST(float)

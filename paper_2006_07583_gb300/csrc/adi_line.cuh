@@ -239,30 +239,48 @@ __device__ inline double line_entry(const LineDesc<T> &d, int row, int col) {
     return acc;
 }
 
-// Gauss-Jordan inverse with partial pivoting of an n x n matrix (A is destroyed).
-__device__ inline bool small_inverse(double *A, int n, double *R) {
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) R[i * n + j] = (i == j) ? 1.0 : 0.0;
+// Gauss-Jordan inverse with partial pivoting of an n x n matrix (n <= 13, destroyed) by one warp: lane
+// j holds column j of [A | R] (R starts as the identity).
+__device__ inline bool warp_inverse(double *A, int n, double *R, int lane) {
     double scale = 0.0;
-    for (int i = 0; i < n * n; ++i) scale = fmax(scale, fabs(A[i]));
+    for (int i = lane; i < n * n; i += 32) {
+        R[i] = (i / n == i % n) ? 1.0 : 0.0;
+        scale = fmax(scale, fabs(A[i]));
+    }
+    for (int o = 16; o > 0; o >>= 1) scale = fmax(scale, __shfl_xor_sync(0xffffffffu, scale, o));
+    __syncwarp();
+    double *col = lane < n ? A + lane : R + (lane - n);  // this lane's column, stride n
+    const bool mine = lane < 2 * n;
     for (int c = 0; c < n; ++c) {
+        double f[13];
         int p = c;
-        for (int i = c + 1; i < n; ++i)
-            if (fabs(A[i * n + c]) > fabs(A[p * n + c])) p = i;
-        if (!(fabs(A[p * n + c]) > 1e-13 * scale)) return false;
-        if (p != c)
-            for (int j = 0; j < n; ++j) {
-                double t = A[c * n + j]; A[c * n + j] = A[p * n + j]; A[p * n + j] = t;
-                t = R[c * n + j]; R[c * n + j] = R[p * n + j]; R[p * n + j] = t;
-            }
-        double ip = 1.0 / A[c * n + c];
-        for (int j = 0; j < n; ++j) { A[c * n + j] *= ip; R[c * n + j] *= ip; }
-        for (int i = 0; i < n; ++i) {
-            if (i == c) continue;
-            double f = A[i * n + c];
-            if (f == 0.0) continue;
-            for (int j = 0; j < n; ++j) { A[i * n + j] -= f * A[c * n + j]; R[i * n + j] -= f * R[c * n + j]; }
+        double best = fabs(A[c * n + c]);
+#pragma unroll
+        for (int i = 0; i < 13; ++i) {
+            f[i] = i < n ? A[i * n + c] : 0.0;
+            if (i > c && i < n && fabs(f[i]) > best) { best = fabs(f[i]); p = i; }
         }
+        if (!(best > 1e-13 * scale)) return false;  // uniform over the warp
+        __syncwarp();  // column c has been read
+        if (mine) {
+            const double ap = col[p * n], ac = col[c * n];
+            double fp = 0.0, fc = 0.0;
+#pragma unroll
+            for (int i = 0; i < 13; ++i) {
+                if (i == p) fp = f[i];
+                if (i == c) fc = f[i];
+            }
+            const double row = ap * (1.0 / fp);
+            if (p != c) col[p * n] = ac;
+            col[c * n] = row;
+#pragma unroll
+            for (int i = 0; i < 13; ++i) {
+                if (i >= n || i == c) continue;
+                const double fi = i == p ? fc : f[i];  // rows p and c are swapped
+                if (fi != 0.0) col[i * n] -= fi * row;
+            }
+        }
+        __syncwarp();
     }
     return true;
 }

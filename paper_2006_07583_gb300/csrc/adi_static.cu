@@ -2,8 +2,8 @@
 // caller keeps in device memory, with every temporary of the library placed in one
 // fixed-size device array compiled into libadi.  Nothing is allocated on the device or the
 // host heap: the array's address is looked up once per device (cudaGetSymbolAddress) and
-// handed to the same kernels the handle path launches with the thread-per-line solver
-// (head/tail tables, carried-state prologue, x-line and y-line solves).
+// handed to the kernels of the handle path's plain solver (head/tail tables, carried-state
+// prologue, x-line and y-line solves with one warp per line).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -78,8 +78,7 @@ Shape shape_of(int method, int nx, int ny) {
 
 // Byte offsets of the temporaries inside the scratch array (each 256-byte aligned).
 struct Layout {
-    size_t desc, status, alpha, A, C, W0, W1, tab, scr, end;
-    long long st;  // word stride of the per-line solver scratch (lines side by side)
+    size_t desc, fac, status, alpha, A, C, W0, W1, tab, end;
 };
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -94,6 +93,7 @@ Layout layout_of(int method, int nx, int ny, const Shape &g, size_t esz) {
     };
     const size_t nl = (size_t)g.pix + g.piy;
     L.desc = take(nl * sizeof(LineDesc<double>));  // LineDesc<float> has the same size
+    L.fac = take(method == ADI_CFD ? prologue_factor_count(ny) * esz : 0);  // copied with the descriptors
     L.status = take(sizeof(int));
     L.alpha = take(g.nU * esz);
     L.A = take(g.nU * esz);
@@ -101,19 +101,19 @@ Layout layout_of(int method, int nx, int ny, const Shape &g, size_t esz) {
     L.W0 = take(g.nW * esz);
     L.W1 = take(g.nW * esz);
     L.tab = take(nl * kTabLine * esz);
-    L.st = std::max(g.pix, g.piy);
-    size_t words = std::max(v1_scratch_words(method, nx), v1_scratch_words(method, ny));
-    words = std::max(words, (size_t)(2 * ny + 4));  // the prologue's column solves
-    L.scr = take(words * (size_t)L.st * esz);
     L.end = off;
     return L;
 }
 
 static_assert(sizeof(LineDesc<float>) == sizeof(LineDesc<double>), "descriptor sizes differ");
+static_assert(ADI_STATIC_MAX_CELLS <= kV1ShortCells, "the short-line solver takes every accepted line");
 
-// Host staging of the descriptors: static storage, sized for the largest accepted grid.
+// Host staging of the descriptors and the prologue's Thomas factors: static storage, sized for the
+// largest accepted grid.
 constexpr int kMaxLines = 2 * ADI_STATIC_MAX_CELLS;
-alignas(64) unsigned char g_host_descs[kMaxLines * sizeof(LineDesc<double>)];
+constexpr size_t kMaxFactors = 6 * ADI_STATIC_MAX_CELLS + 64;
+alignas(64) unsigned char g_host_descs[kMaxLines * sizeof(LineDesc<double>) + 256 + kMaxFactors * sizeof(double)];
+double g_host_factors[kMaxFactors];
 
 template <typename T>
 void fill_descs(int method, int nx, int ny, double h, double dt, const Shape &g,
@@ -185,10 +185,18 @@ int step_static(int method, int nx, int ny, double h, double dt, const T *c, con
     LineDesc<T> *dd = (LineDesc<T> *)(base + L.desc);
     int *status = (int *)(base + L.status);
     T *alpha = (T *)(base + L.alpha), *A = (T *)(base + L.A), *C = (T *)(base + L.C);
-    T *tab = (T *)(base + L.tab), *scr = (T *)(base + L.scr);
+    T *tab = (T *)(base + L.tab);
     const size_t esz = sizeof(T);
+    size_t nfac = 0;
+    if (method == ADI_CFD) {
+        nfac = prologue_factor_count(ny);
+        if (nfac > kMaxFactors) return ADI_ENOMEM;
+        prologue_factors(ny, g_host_factors);
+        T *hf = (T *)(g_host_descs + (L.fac - L.desc));
+        for (size_t k = 0; k < nfac; ++k) hf[k] = (T)g_host_factors[k];
+    }
 
-    cudaError_t e = cudaMemcpyAsync(dd, hd, (size_t)nl * sizeof(LineDesc<T>), cudaMemcpyHostToDevice, s);
+    cudaError_t e = cudaMemcpyAsync(dd, hd, L.fac - L.desc + nfac * esz, cudaMemcpyHostToDevice, s);
     // the singular-pivot flag is the one temporary read before it is written
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, sizeof(int), s);
     if (e == cudaSuccess) {
@@ -204,9 +212,9 @@ int step_static(int method, int nx, int ny, double h, double dt, const T *c, con
     if (e == cudaSuccess) e = cudaMemcpyAsync(w_out, w, g.nW * esz, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = launch_precompute<T>(dd, nl, tab, status, s);
     // carried state a, w* from the natural fields (read through the y-lines' u_out/w_out)
-    if (e == cudaSuccess) e = launch_prologue<T>(dd + g.piy, g.pix, nullptr, scr, L.st, s);
-    if (e == cudaSuccess) e = launch_line_solve_v1<T>(dd, g.piy, scr, L.st, 0, s);
-    if (e == cudaSuccess) e = launch_line_solve_v1<T>(dd + g.piy, g.pix, scr, L.st, 1, s);
+    if (e == cudaSuccess) e = launch_prologue_lines<T>(dd + g.piy, g.pix, ny, method, (const T *)(base + L.fac), s);
+    if (e == cudaSuccess) e = launch_line_solve_short<T>(dd, g.piy, method, nx, 0, s);
+    if (e == cudaSuccess) e = launch_line_solve_short<T>(dd + g.piy, g.pix, method, ny, 1, s);
     int singular = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&singular, status, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
