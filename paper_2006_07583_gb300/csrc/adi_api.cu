@@ -195,7 +195,9 @@ struct Plan {
     // natural fields after a stage 2 that writes them: one record per member, per plan parity
     DevBuf ndesc[2];
     int ncount = 0, nrows = 0, ncols = 0;
-    DevBuf fault;                            // set by a factored launch whose wait ran out
+    // [0] set by a factored launch whose wait ran out, [1] by the finite check of fields to load: side by
+    // side, so that one small copy brings both to the host
+    DevBuf fault;
     // time-harmonic walls and forcing of the members that have them (after each stage)
     DevBuf hdesc;
     int hcount = 0;
@@ -268,6 +270,7 @@ struct adi_sim {
     double h = 0, dt = 0;
     size_t esz = 4;
     DevBuf A[4], V[2], W[2], alpha, alphaT, Uo, Wo, tab, sep, cold_all, clock, status;
+    int cold_parity = -1;  // parity of the descriptors in cold_all (-1: none, or out of date)
     // host <-> device staging of the natural fields (FP64) and the prologue's Thomas factors
     // (CFD): allocated by the first adi_set_fields / adi_read_fields /
     // adi_set_source after creation and kept until adi_destroy (adi_create frees its own)
@@ -337,14 +340,6 @@ __global__ void convert_from_double(const double *src, T *dst, size_t rows, size
         const double x = src[r * cols + c];
         dst[r * ld + c] = (T)(square ? scale * x * x : scale * x);
     }
-}
-// Rows with leading dimension ld in T -> compact row-major double.
-template <typename T>
-__global__ void convert_to_double(const T *src, double *dst, size_t rows, size_t cols, size_t ld) {
-    const size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (c >= cols) return;
-#pragma unroll 4
-    for (size_t r = blockIdx.y; r < rows; r += gridDim.y) dst[r * cols + c] = (double)src[r * ld + c];
 }
 // Compact row-major S (rows x cols) -> rows with leading dimension ld in T.
 template <typename S, typename T>
@@ -661,6 +656,7 @@ void build_host_descs(adi_sim *s) {
         s->h_desc[par][0].assign((unsigned char *)rows.data(), (unsigned char *)(rows.data() + rows.size()));
         s->h_desc[par][1].assign((unsigned char *)cols.data(), (unsigned char *)(cols.data() + cols.size()));
     }
+    s->cold_parity = -1;
 }
 
 // The harmonic record of a simulation with time-harmonic walls (and forcing).
@@ -921,8 +917,8 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
         sp.harm = my_h;
         p.sponges.push_back(sp);
     }
-    if (!rc) rc = dev_alloc(p.fault, sizeof(int));
-    if (!rc) rc = cuda_status(cudaMemsetAsync(p.fault.p, 0, sizeof(int), stream));
+    if (!rc) rc = dev_alloc(p.fault, 2 * sizeof(int));
+    if (!rc) rc = cuda_status(cudaMemsetAsync(p.fault.p, 0, 2 * sizeof(int), stream));
     if (!rc && (p.v1n[0] || p.v1n[1])) {
         p.scratch_stride = std::max(p.v1n[0], p.v1n[1]);
         rc = dev_alloc(p.scratch, words * (size_t)p.scratch_stride * esz);
@@ -1046,6 +1042,7 @@ cudaError_t run_graph(Plan &p, int q0, int nsteps, cudaStream_t stream) {
 // Uploads the sim's descriptors of its current parity (x-lines then y-lines) for the
 // prologue and the precomputes.
 int upload_sim_descs(adi_sim *s) {
+    if (s->cold_parity == s->parity) return ADI_OK;  // they are there
     const std::vector<unsigned char> &hx = s->h_desc[s->parity][0], &hy = s->h_desc[s->parity][1];
     size_t bytes = hx.size() + hy.size();
     if (s->cold_all.bytes < bytes) {
@@ -1057,8 +1054,8 @@ int upload_sim_descs(adi_sim *s) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync((unsigned char *)s->cold_all.p + hx.size(), hy.data(), hy.size(),
                             cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    return cuda_status(e);
+    if (e == cudaSuccess) s->cold_parity = s->parity;
+    return cuda_status(e);  // the copies' host sources live with the simulation
 }
 
 template <typename T>
@@ -1191,7 +1188,8 @@ int xfer_buffer(adi_sim *s) {
 
 // Copies host fields (FP64, or FP32 with f32) into their slots of the staging buffer and checks
 // them there, before any of the simulation's state changes (ADI_EINVAL on NaN/Inf).  staged[k]
-// receives the slot of field k, or nullptr for a field not given.
+// receives the slot of field k, or nullptr for a field not given.  The one wait covers everything on
+// the stream before it as adi_sync does: an error of that work is made sticky.
 int stage_fields(adi_sim *s, const void *const f[3], bool f32, const void *staged[3]) {
     int rc = xfer_buffer(s);
     if (rc) return rc;
@@ -1200,22 +1198,24 @@ int stage_fields(adi_sim *s, const void *const f[3], bool f32, const void *stage
     xfer_slots(g, off);
     const size_t n[3] = {g.nU(), g.nV(), g.nW()};
     const size_t hsz = f32 ? sizeof(float) : sizeof(double);
-    cudaError_t e = cudaMemsetAsync(s->status.p, 0, sizeof(int), s->stream);
+    int *bad = (int *)s->plan.fault.p + 1;
+    cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), s->stream);
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
         staged[k] = nullptr;
         if (!f[k]) continue;
         void *slot = (unsigned char *)s->xfer.p + off[k];
         e = cudaMemcpyAsync(slot, f[k], n[k] * hsz, cudaMemcpyHostToDevice, s->stream);
         if (e == cudaSuccess)
-            e = f32 ? launch_finite_check<float>((const float *)slot, n[k], (int *)s->status.p, s->stream)
-                    : launch_finite_check<double>((const double *)slot, n[k], (int *)s->status.p, s->stream);
+            e = f32 ? launch_finite_check<float>((const float *)slot, n[k], bad, s->stream)
+                    : launch_finite_check<double>((const double *)slot, n[k], bad, s->stream);
         staged[k] = slot;
     }
-    int flag = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, s->status.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+    int flags[2] = {0, 0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(flags, s->plan.fault.p, sizeof(flags), cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_status(e);
-    return flag ? ADI_EINVAL : ADI_OK;
+    if (e != cudaSuccess) return s->sticky = cuda_status(e);
+    if (flags[0]) return s->sticky = ADI_ETIMEOUT;
+    return flags[1] ? ADI_EINVAL : ADI_OK;
 }
 
 // One staged field (compact rows x cols of FP64, or FP32 with f32) into a device array of the
@@ -1777,40 +1777,59 @@ int adi_sync(adi_handle s) {
     return s->sticky;
 }
 
-int adi_read_fields(adi_handle s, double *u, double *v, double *w) {
+namespace {
+// adi_read_fields / adi_read_fields_f32.  A field whose host type or row length differs from the device
+// array's is first converted or packed into its slot of the staging buffer (a pitched device-to-host
+// copy runs at about half the speed of a contiguous one).  One wait covers the work before and all copies; the
+// fault word comes with them.
+int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
     if (!s) return ADI_EINVAL;
     if (s->in_batch && s->batch_stream) {
         cudaError_t be = cudaStreamSynchronize(s->batch_stream);
         if (be != cudaSuccess) return s->sticky = cuda_status(be);
     }
-    int rc = adi_sync(s);
-    if (rc) return rc;
+    if (s->sticky) return s->sticky;
     const Geometry &g = s->g;
-    struct { const void *src; double *dst; size_t rows, cols, ld; } parts[3] = {
+    struct { const void *src; void *dst; size_t rows, cols, ld; } parts[3] = {
         {s->Uo.p, u, (size_t)g.rows_u, (size_t)g.ldu, (size_t)g.ldu},
         {s->V[s->parity].p, v, (size_t)g.rows_v, (size_t)g.ldv, (size_t)g.ldvp},
         {s->Wo.p, w, (size_t)g.rows_w, (size_t)g.ldw, (size_t)g.ldw}};
-    rc = xfer_buffer(s);
-    if (rc) return rc;
-    DevBuf &tmp = s->xfer;
-    for (auto &pt : parts) {
+    const bool dev32 = s->precision == ADI_FP32;
+    size_t off[4];
+    xfer_slots(g, off);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+        auto &pt = parts[k];
         if (!pt.dst) continue;
-        const size_t n = pt.rows * pt.cols;
-        const dim3 grid = conv_grid(pt.rows, pt.cols);
-        if (s->precision == ADI_FP64)
-            convert_to_double<double><<<grid, 256, 0, s->stream>>>((const double *)pt.src, (double *)tmp.p, pt.rows, pt.cols, pt.ld);
-        else
-            convert_to_double<float><<<grid, 256, 0, s->stream>>>((const float *)pt.src, (double *)tmp.p, pt.rows, pt.cols, pt.ld);
-        cudaError_t e = cudaGetLastError();
+        const void *src = pt.src;
+        if (dev32 != f32 || pt.ld != pt.cols) {
+            int rc = xfer_buffer(s);
+            if (rc) return rc;
+            void *slot = (unsigned char *)s->xfer.p + off[k];
+            const dim3 grid = conv_grid(pt.rows, pt.cols);
+            if (dev32 && f32)
+                convert_out<float, float><<<grid, 256, 0, s->stream>>>((const float *)src, (float *)slot, pt.rows, pt.cols, pt.ld);
+            else if (dev32)
+                convert_out<float, double><<<grid, 256, 0, s->stream>>>((const float *)src, (double *)slot, pt.rows, pt.cols, pt.ld);
+            else if (f32)
+                convert_out<double, float><<<grid, 256, 0, s->stream>>>((const double *)src, (float *)slot, pt.rows, pt.cols, pt.ld);
+            else
+                convert_out<double, double><<<grid, 256, 0, s->stream>>>((const double *)src, (double *)slot, pt.rows, pt.cols, pt.ld);
+            e = cudaGetLastError();
+            src = slot;
+        }
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(pt.dst, tmp.p, n * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-        if (e != cudaSuccess) return s->sticky = cuda_status(e);
+            e = cudaMemcpyAsync(pt.dst, src, pt.rows * pt.cols * (f32 ? sizeof(float) : sizeof(double)), cudaMemcpyDeviceToHost,
+                                s->stream);
     }
-    return ADI_OK;
+    int fault = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&fault, s->plan.fault.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return s->sticky = cuda_status(e);
+    if (fault) s->sticky = ADI_ETIMEOUT;
+    return s->sticky;
 }
 
-namespace {
 // adi_set_fields / adi_set_fields_f32: stage and check every given field, then load them.
 int set_fields_any(adi_handle s, const void *u, const void *v, const void *w, bool f32) {
     if (!s) return ADI_EINVAL;
@@ -1818,10 +1837,9 @@ int set_fields_any(adi_handle s, const void *u, const void *v, const void *w, bo
         cudaError_t be = cudaStreamSynchronize(s->batch_stream);
         if (be != cudaSuccess) return s->sticky = cuda_status(be);
     }
-    int rc = adi_sync(s);
-    if (rc) return rc;
+    if (s->sticky) return s->sticky;
     const void *f[3] = {u, v, w}, *staged[3];
-    rc = stage_fields(s, f, f32, staged);
+    int rc = stage_fields(s, f, f32, staged);
     if (rc == ADI_EINVAL) return rc;
     if (rc) return s->sticky = rc;
     rc = load_state(s, staged, f32, true);
@@ -1829,6 +1847,10 @@ int set_fields_any(adi_handle s, const void *u, const void *v, const void *w, bo
     return rc;
 }
 }  // namespace
+
+int adi_read_fields(adi_handle s, double *u, double *v, double *w) {
+    return read_fields_any(s, u, v, w, false);
+}
 
 int adi_set_fields(adi_handle s, const double *u, const double *v, const double *w) {
     return set_fields_any(s, u, v, w, false);
@@ -1839,52 +1861,7 @@ int adi_set_fields_f32(adi_handle s, const float *u, const float *v, const float
 }
 
 int adi_read_fields_f32(adi_handle s, float *u, float *v, float *w) {
-    if (!s) return ADI_EINVAL;
-    if (s->in_batch && s->batch_stream) {
-        cudaError_t be = cudaStreamSynchronize(s->batch_stream);
-        if (be != cudaSuccess) return s->sticky = cuda_status(be);
-    }
-    int rc = adi_sync(s);
-    if (rc) return rc;
-    const Geometry &g = s->g;
-    struct { const void *src; float *dst; size_t rows, cols, ld; } parts[3] = {
-        {s->Uo.p, u, (size_t)g.rows_u, (size_t)g.ldu, (size_t)g.ldu},
-        {s->V[s->parity].p, v, (size_t)g.rows_v, (size_t)g.ldv, (size_t)g.ldvp},
-        {s->Wo.p, w, (size_t)g.rows_w, (size_t)g.ldw, (size_t)g.ldw}};
-    // FP64 fields are converted through the staging buffer; an FP32 field whose rows are padded
-    // (v) is first packed there on the device, since a pitched device-to-host copy runs at about
-    // half the speed of a contiguous one
-    bool need_xfer = s->precision == ADI_FP64;
-    for (auto &pt : parts) need_xfer |= pt.dst && pt.ld != pt.cols;
-    if (need_xfer) {
-        rc = xfer_buffer(s);
-        if (rc) return rc;
-    }
-    cudaError_t e = cudaSuccess;
-    for (auto &pt : parts) {
-        if (!pt.dst || e != cudaSuccess) continue;
-        if (s->precision == ADI_FP32 && pt.ld == pt.cols) {  // straight from the device array
-            e = cudaMemcpyAsync(pt.dst, pt.src, pt.rows * pt.cols * sizeof(float), cudaMemcpyDeviceToHost, s->stream);
-        } else if (s->precision == ADI_FP32) {
-            convert_out<float, float><<<conv_grid(pt.rows, pt.cols), 256, 0, s->stream>>>(
-                (const float *)pt.src, (float *)s->xfer.p, pt.rows, pt.cols, pt.ld);
-            e = cudaGetLastError();
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(pt.dst, s->xfer.p, pt.rows * pt.cols * sizeof(float), cudaMemcpyDeviceToHost, s->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // the staging is reused
-        } else {
-            const size_t n = pt.rows * pt.cols;
-            convert_out<double, float><<<conv_grid(pt.rows, pt.cols), 256, 0, s->stream>>>((const double *)pt.src,
-                                                                                           (float *)s->xfer.p, pt.rows,
-                                                                                           pt.cols, pt.ld);
-            e = cudaGetLastError();
-            if (e == cudaSuccess) e = cudaMemcpyAsync(pt.dst, s->xfer.p, n * sizeof(float), cudaMemcpyDeviceToHost, s->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // the staging is reused
-        }
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return s->sticky = cuda_status(e);
-    return ADI_OK;
+    return read_fields_any(s, u, v, w, true);
 }
 
 int adi_check_finite(adi_handle s) {
