@@ -688,6 +688,19 @@ SpongeRec sponge_rec_of(const adi_sim *s) {
     return r;
 }
 
+// The addresses of a group's lines (from line `line` of the simulation and direction on), for plan parities 0
+// and 1.  Descriptors of both precisions have one layout.
+void set_group_lines(FacGroup &fg, const adi_sim *s, int dir, int line) {
+    const Geometry &g = s->g;
+    const LineDesc<float> *d[2];
+    for (int q = 0; q < 2; ++q) d[q] = (const LineDesc<float> *)s->h_desc[s->parity ^ q][dir].data() + line;
+    fg.gp = d[0]->p; fg.ga = d[0]->alpha; fg.gs = d[0]->sep;
+    fg.gv[0] = d[0]->v; fg.gv[1] = d[1]->v;
+    fg.dp = dir == 0 ? g.lda : g.ldc;
+    fg.dv = dir == 0 ? g.ldvp : g.ldwc;
+    fg.dr = (int)fac_words(g.method, dir == 0 ? g.nx : g.ny);
+}
+
 // Builds an execution plan for members (all of one precision).  Plan parity q uses each
 // member's descriptors of parity (member's current parity) ^ q.
 int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stream) {
@@ -738,6 +751,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
                         const int k = fac_split_groups(s->g.method, N, first + st, std::max(1, s->fac_reach),
                                                        1.0 / s->h, 0.5 * s->dt, esz, sub, &sb);
                         if (k == 0) return ADI_ENOTSUP;
+                        for (int i = 0; i < k; ++i) set_group_lines(sub[i], s, dir, st);
                         fgr[dir][v].insert(fgr[dir][v].end(), sub, sub + k);
                         p.fstage[dir][v] = std::max(p.fstage[dir][v], sb);
                     }
@@ -749,6 +763,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
                         FacGroup fg = fac_group_of(s->g.method, N, first + st, cnt, 1.0 / s->h, 0.5 * s->dt);
                         // the scans this simulation's lines need, whatever else shares the launch
                         if (s->fac_reach > kFacMaxReach) fg.own |= kFacOwnFull;
+                        set_group_lines(fg, s, dir, st);
                         fgr[dir][v].push_back(fg);
                         p.fstage[dir][v] = std::max(p.fstage[dir][v], fac_stage_bytes(s->g.method, N, cnt, esz));
                         st += cnt;
@@ -959,7 +974,7 @@ cudaError_t enqueue_stage(const Plan &p, int q, int dir, int natural, cudaStream
         if (p.nfgroups[dir][v])
             e = launch_line_solve_factored<T>((const LineDesc<T> *)p.fd[q][dir].p,
                                               (const FacGroup *)p.fgroups[dir][v].p, p.nfgroups[dir][v], v,
-                                              p.fstage[dir][v], p.fstages[dir][v], p.fgrid[dir][v], 0,
+                                              p.fstage[dir][v], p.fstages[dir][v], p.fgrid[dir][v], 0, q,
                                               (int *)p.fault.p, stream);
     for (int m = 0; m < 2 && e == cudaSuccess; ++m)
         if (p.ngroups[dir][m])

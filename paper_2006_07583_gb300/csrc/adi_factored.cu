@@ -168,8 +168,8 @@ constexpr size_t kDescBytes = sizeof(LineDesc<float>);
 static_assert(sizeof(LineDesc<float>) == sizeof(LineDesc<double>), "descriptor sizes differ");
 static_assert(kDescBytes % 16 == 0, "descriptor size");
 __host__ __device__ inline size_t fac_desc_area(int nl) { return ((size_t)nl * kDescBytes + 127) & ~(size_t)127; }
-// A stage: the group (128 bytes), the descriptors, then the lines.
-constexpr size_t kFacGroupBytes = 128;
+// A stage: the group (192 bytes), the descriptors, then the lines.
+constexpr size_t kFacGroupBytes = 192;
 static_assert(sizeof(FacGroup) % 16 == 0 && sizeof(FacGroup) <= kFacGroupBytes, "group header");
 __host__ __device__ inline size_t fac_head_bytes(int nl) { return kFacGroupBytes + fac_desc_area(nl); }
 
@@ -1018,8 +1018,7 @@ __device__ void fac_store_outputs(const unsigned char *stage, int lane) {
 // The staging warp: stage one line group (descriptors, then per line the pressure, velocity
 // and alpha lines and the record) into shared memory.  Lane 0 announces the group's bytes on the
 // stage's "full" barrier (its only arrival) and copies the header and the descriptors; lane k
-// reads the descriptors of lines k, k + 32, ... from global memory and issues their copies, so
-// that a group of many short lines costs one round trip for its descriptors, not one per line.
+// issues the copies of lines k, k + 32, ..., whose addresses follow from the group's header alone.
 // A sub-line of a split line stages its span of the three lines and, of the record, its chunks'
 // S, F and H parts, the end tables it holds and the reach.  Every source starts on a 16-byte
 // boundary (padded leading dimensions; spans start at multiples of four elements; record parts
@@ -1027,7 +1026,7 @@ __device__ void fac_store_outputs(const unsigned char *stage, int lane) {
 // copies, rounded up to 16 bytes, stay inside the padded line or the record.
 template <typename T, int BS, bool SPLIT>
 __device__ void fac_issue(const LineDesc<T> *__restrict__ descs, const FacGroup *gp, unsigned char *stage,
-                          unsigned long long *bar, int lane) {
+                          unsigned long long *bar, int lane, int q) {
     const FacGroup &gr = *gp;
     const int Lp = gr.lp, lo = SPLIT ? gr.lo : 0;
     const unsigned bp = round16((unsigned)gr.pn * (unsigned)sizeof(T));
@@ -1042,14 +1041,15 @@ __device__ void fac_issue(const LineDesc<T> *__restrict__ descs, const FacGroup 
     }
     __syncwarp();  // the group's bytes are announced before any line copy is issued
     T *base = (T *)(stage + fac_head_bytes(gr.nl));
+    const T *gp_ = (const T *)gr.gp, *gv_ = (const T *)gr.gv[q], *ga_ = (const T *)gr.ga, *gs_ = (const T *)gr.gs;
     for (int l = lane; l < gr.nl; l += 32) {
-        const LineDesc<T> &d = descs[gr.first + l];
         T *ln = base + (size_t)l * gr.ls;
-        bulk_to_smem(ln, d.p + lo, bp, bar);
-        bulk_to_smem(ln + Lp, d.v + lo, bv, bar);
-        bulk_to_smem(ln + 2 * Lp, d.alpha + lo, bp, bar);
+        const T *sep = gs_ + (size_t)l * gr.dr;
+        bulk_to_smem(ln, gp_ + (size_t)l * gr.dp + lo, bp, bar);
+        bulk_to_smem(ln + Lp, gv_ + (size_t)l * gr.dv + lo, bv, bar);
+        bulk_to_smem(ln + 2 * Lp, ga_ + (size_t)l * gr.dp + lo, bp, bar);
         if constexpr (!SPLIT) {
-            bulk_to_smem(ln + 3 * Lp, d.sep, br, bar);
+            bulk_to_smem(ln + 3 * Lp, sep, br, bar);
         } else {
             const FacGeom g = fac_geom(BS == 2 ? kCFD : kMFD, gr.N);
             const int pg = fac_part(g), es = fac_e_stride(g);
@@ -1057,7 +1057,7 @@ __device__ void fac_issue(const LineDesc<T> *__restrict__ descs, const FacGroup 
             const unsigned bpart = (unsigned)gr.part * (unsigned)sizeof(T);
             const unsigned be = (unsigned)es * (unsigned)sizeof(T);
             T *rec = ln + 3 * Lp;
-            const T *src = d.sep;
+            const T *src = sep;
             bulk_to_smem(rec, src + cs, bpart, bar);
             bulk_to_smem(rec + gr.part, src + pg + cs, bpart, bar);
             bulk_to_smem(rec + 2 * gr.part, src + 2 * pg + cs, bpart, bar);
@@ -1942,7 +1942,7 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
 template <typename T, int BS, int MM, bool SPLIT, int NT>
 __global__ void __launch_bounds__(NT, 1)
 line_solve_factored_kernel(const LineDesc<T> *__restrict__ descs, const FacGroup *__restrict__ groups, int ngroups,
-                           int natural, unsigned stage_bytes, int stages, int *fault) {
+                           int natural, unsigned stage_bytes, int stages, int q, int *fault) {
     extern __shared__ __align__(128) unsigned char fac_smem[];
     __shared__ ScanSmem<T, BS> ssm;
     __shared__ __align__(8) unsigned long long full[kFacMaxStages], empty[kFacMaxStages];
@@ -1975,7 +1975,7 @@ line_solve_factored_kernel(const LineDesc<T> *__restrict__ descs, const FacGroup
                 fac_store_outputs<T>(stage, lane);
                 __syncwarp();  // every lane's output copies have read the stage
             }
-            fac_issue<T, BS, SPLIT>(descs, groups + gi, stage, &full[st], lane);
+            fac_issue<T, BS, SPLIT>(descs, groups + gi, stage, &full[st], lane, q);
             last[st] = use;
             if (++st == stages) { st = 0; ++use; }
         }
@@ -2024,7 +2024,7 @@ cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, int method, 
 
 template <typename T, int BS, int MM, bool SPLIT, int NT>
 cudaError_t launch_fac_inst(const LineDesc<T> *d, const FacGroup *groups, int ngroups, size_t stage_bytes, int stages,
-                            int grid, int natural, int *fault, cudaStream_t s) {
+                            int grid, int natural, int q, int *fault, cudaStream_t s) {
     auto kern = line_solve_factored_kernel<T, BS, MM, SPLIT, NT>;
     // the host sizes the ring with fac_static_smem, an upper bound of the kernel's own static
     // shared memory: check it against the compiled kernel once
@@ -2036,30 +2036,30 @@ cudaError_t launch_fac_inst(const LineDesc<T> *d, const FacGroup *groups, int ng
     const size_t dyn = (size_t)stages * stage_bytes;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     if (e != cudaSuccess) return e;
-    kern<<<grid, NT, dyn, s>>>(d, groups, ngroups, natural, (unsigned)stage_bytes, stages, fault);
+    kern<<<grid, NT, dyn, s>>>(d, groups, ngroups, natural, (unsigned)stage_bytes, stages, q, fault);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_line_solve_factored(const LineDesc<T> *d, const FacGroup *groups, int ngroups, int variant,
-                                       size_t stage_bytes, int stages, int grid, int natural, int *fault,
+                                       size_t stage_bytes, int stages, int grid, int natural, int q, int *fault,
                                        cudaStream_t s) {
     if (ngroups <= 0) return cudaSuccess;
     if (grid > ngroups) grid = ngroups;
     if (stages < 1 || stages > kFacMaxStages) return cudaErrorInvalidValue;
     constexpr int W = kFacThreads;
     switch (variant) {
-    case 0: return launch_fac_inst<T, 2, 9, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 1: return launch_fac_inst<T, 3, 2, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 2: return launch_fac_inst<T, 3, 3, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 3: return launch_fac_inst<T, 2, 9, true, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-    case 4: return launch_fac_inst<T, 3, 3, true, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+    case 0: return launch_fac_inst<T, 2, 9, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
+    case 1: return launch_fac_inst<T, 3, 2, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
+    case 2: return launch_fac_inst<T, 3, 3, false, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
+    case 3: return launch_fac_inst<T, 2, 9, true, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
+    case 4: return launch_fac_inst<T, 3, 3, true, W>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
     }
     if constexpr (sizeof(T) == 8) {
         constexpr int NR = kFacNarrow;
         switch (variant) {
-        case 5: return launch_fac_inst<T, 3, 2, false, NR>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
-        case 6: return launch_fac_inst<T, 3, 3, false, NR>(d, groups, ngroups, stage_bytes, stages, grid, natural, fault, s);
+        case 5: return launch_fac_inst<T, 3, 2, false, NR>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
+        case 6: return launch_fac_inst<T, 3, 3, false, NR>(d, groups, ngroups, stage_bytes, stages, grid, natural, q, fault, s);
         }
     }
     return cudaErrorInvalidValue;
@@ -2068,9 +2068,9 @@ cudaError_t launch_line_solve_factored(const LineDesc<T> *d, const FacGroup *gro
 template cudaError_t launch_fac_precompute<float>(const LineDesc<float> *, int, int, int, double *, int *, cudaStream_t);
 template cudaError_t launch_fac_precompute<double>(const LineDesc<double> *, int, int, int, double *, int *, cudaStream_t);
 template cudaError_t launch_line_solve_factored<float>(const LineDesc<float> *, const FacGroup *, int, int, size_t, int,
-                                                       int, int, int *, cudaStream_t);
+                                                       int, int, int, int *, cudaStream_t);
 template cudaError_t launch_line_solve_factored<double>(const LineDesc<double> *, const FacGroup *, int, int, size_t,
-                                                        int, int, int, int *, cudaStream_t);
+                                                        int, int, int, int, int *, cudaStream_t);
 
 // The bounded wait's failure path, run on purpose: one thread waits on an mbarrier that
 // nothing arrives at, with `polls` polls at most, and records whether the wait gave up (and

@@ -127,6 +127,12 @@ struct alignas(16) FacGroup {
                              // bit 18 holds the head region, bit 19 the tail region, bit 20 a split line
     int sp0, sp1, sv0, sv1;  // pressure / velocity outputs stored by bulk copies ([sp0, sp1)); the
                              // group's other owned outputs are stored by the threads that compute them
+    // what the staging warp copies: the first line's pressure, velocity (per plan parity), alpha and record, and
+    // the distances to the next line's in elements.  Without them its lanes read the line descriptors first, one
+    // more round trip to memory before any line is on its way: half a microsecond of the 8 to 16 that a launch over
+    // small and middle grids takes.
+    const void *gp, *gv[2], *ga, *gs;
+    int dp, dv, dr, pad;
 };
 constexpr int kFacOwnHead = 1 << 18, kFacOwnTail = 1 << 19, kFacOwnSplit = 1 << 20;
 constexpr int kFacOwnFull = 1 << 21;     // the group's lines reach beyond the scan window: full scans
@@ -159,7 +165,7 @@ cudaError_t launch_fac_precompute(const LineDesc<T> *d, int nlines, int method, 
 template <typename T>
 cudaError_t launch_line_solve_factored(const LineDesc<T> *d, const FacGroup *groups, int ngroups,
                                        int variant, size_t stage_bytes, int stages, int grid,
-                                       int natural, int *fault, cudaStream_t s);
+                                       int natural, int q, int *fault, cudaStream_t s);
 
 // Chunked solver (adi_chunked.cu).
 int chunk_M(int method);                 // chunk length in blocks used by the kernel
