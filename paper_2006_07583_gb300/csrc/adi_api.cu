@@ -364,10 +364,11 @@ __global__ void convert_out(const T *src, D *dst, size_t rows, size_t cols, size
 // MFD: cells 1..N; w on 0..N; columns 1..pix).  One record per member and plan parity.
 struct NatDesc {
     const void *a, *c;        // A[3] (a) and A[1] (C), column-major: column j at j * ldc
+    const void *a_row;        // a in A[0] instead (row-major, lda) where stage 2 stores it there, else nullptr
     const void *wn, *wi;      // w*' (the stage's output) and w* (its input), column j at j * ldwc
     void *uo, *wo;            // natural u (row-major, ldu) and w (row-major, ldw)
     const long long *clock;   // the member's step clock (for the point source)
-    int ldc, ldwc, ldu, ldw;
+    int ldc, ldwc, ldu, ldw, lda;
     int j1;                   // columns 1 .. j1 - 1
     int ku0, ku1, kw1;        // u rows [ku0, ku1), w rows [0, kw1)
     int src_i, src_j;         // the point source's row and column, or -1
@@ -391,7 +392,7 @@ __global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restri
     const int k0 = blockIdx.y * kNatRows, jb = blockIdx.x * 32, j1 = d.j1, ku1 = d.ku1, kw1 = d.kw1;
     if (k0 >= max(ku1, kw1) || jb >= j1) return;  // uniform over the block
     const T *__restrict__ a = (const T *)d.a, *__restrict__ c = (const T *)d.c;
-    const T *__restrict__ wn = (const T *)d.wn, *__restrict__ wi = (const T *)d.wi;
+    const T *__restrict__ wn = (const T *)d.wn, *__restrict__ wi = (const T *)d.wi, *__restrict__ a_row = (const T *)d.a_row;
     const long long ldc = d.ldc, ldwc = d.ldwc;
 #pragma unroll
     for (int q = threadIdx.x; q < 32 * KV; q += 256) {
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restri
         if (j < 1 || j >= j1) continue;
         Vec va{}, vc{}, vn{}, vi{};
         if (k < ku1) {
-            va = *reinterpret_cast<const Vec *>(a + j * ldc + k);
+            if (!a_row) va = *reinterpret_cast<const Vec *>(a + j * ldc + k);
             vc = *reinterpret_cast<const Vec *>(c + j * ldc + k);
         }
         if (k < kw1) {
@@ -421,6 +422,7 @@ __global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restri
         const int k = k0 + kk;
         if (k >= ku0 && k < ku1) {
             T u = tu[threadIdx.x & 31][kk];
+            if (a_row) u += T(0.5) * a_row[(long long)k * d.lda + j];  // halves are exact: the same sum
             if (k == src_i)  // the point source's dt/2 f is not part of u
                 u -= T(0.5) * (T)(d.src_scale * ricker(d.src_amp, d.src_f0, d.src_td,
                                                        (double)(*d.clock + d.clock_ahead) * d.dt));
@@ -701,6 +703,20 @@ void set_group_lines(FacGroup &fg, const adi_sim *s, int dir, int line) {
     fg.dr = (int)fac_words(g.method, dir == 0 ? g.nx : g.ny);
 }
 
+// The n line descriptors at h (a plan's copies): the pressure output straight into the layout of the other stage's
+// lines, C into A[1], a into A[0].
+template <typename T>
+void set_direct(unsigned char *h, int n, const adi_sim *s, int dir) {
+    LineDesc<T> *d = reinterpret_cast<LineDesc<T> *>(h);
+    const Geometry &g = s->g;
+    const T *staged = (const T *)s->A[dir == 0 ? 2 : 3].p;
+    const int ld = dir == 0 ? g.lda : g.ldc;
+    for (int k = 0; k < n; ++k) {
+        d[k].po = (T *)s->A[dir == 0 ? 1 : 0].p + (d[k].po - staged) / ld;
+        d[k].spo = dir == 0 ? g.ldc : g.lda;
+    }
+}
+
 // Builds an execution plan for members (all of one precision).  Plan parity q uses each
 // member's descriptors of parity (member's current parity) ^ q.
 int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stream) {
@@ -731,6 +747,16 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
         }
     for (int dir = 0; dir < 2; ++dir)
         for (int v = 0; v < kFacVariants; ++v) frounds[dir][v] = (fmin[dir][v] + sms - 1) / sms;
+    // Lines that store their outputs from the threads that compute them (those within a warp) store the carried
+    // pressure in the next stage's layout at once where the launch is one round of groups: it is then bound by latency,
+    // and the transposing launch with the gap before it goes (one 100^2 member 20.5 -> 16.5 us a step, 16 of 128^2 26.2 ->
+    // 22.0).  A launch of several rounds is bound by its work, and scattered 4-byte stores show: 24 members of
+    // 128-1024 cells took 4860 instead of 4592 us for 16 steps with every line within a warp stored so.
+    auto direct = [&](const adi_sim *s, int dir) {
+        const int N = dir == 0 ? s->g.nx : s->g.ny;
+        return s->solver == ADI_SOLVER_FACTORED && fac_direct(s->g.method, N) &&
+               frounds[dir][fac_variant(s->g.method, N, esz)] == 1;
+    };
     for (adi_sim *s : members) {
         for (int dir = 0; dir < 2; ++dir) {
             if (s->solver == ADI_SOLVER_LINE) {
@@ -774,6 +800,9 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
                 for (int q = 0; q < 2; ++q) {
                     const std::vector<unsigned char> &h = s->h_desc[s->parity ^ q][dir];
                     fdv[q][dir].insert(fdv[q][dir].end(), h.begin(), h.end());
+                    if (!direct(s, dir)) continue;
+                    unsigned char *own = fdv[q][dir].data() + (size_t)first * dsz;
+                    if (prec == ADI_FP64) set_direct<double>(own, n, s, dir); else set_direct<float>(own, n, s, dir);
                 }
             } else {
                 int first = (int)(cd[0][dir].size() / dsz);
@@ -845,6 +874,8 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
         std::vector<TDesc> td;
         for (adi_sim *s : members) {
             const Geometry &g = s->g;
+            // not for lines that store into the other layout, nor for a that the absorbing layers rebuild
+            if (direct(s, dir) || (dir == 1 && s->sp_on)) continue;
             TDesc t;
             if (dir == 0) {  // C row-major (A[2]) -> column-major (A[1])
                 t.src = s->A[2].p; t.dst = s->A[1].p;
@@ -858,6 +889,7 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
             td.push_back(t);
         }
         p.tcount[dir] = (int)td.size();
+        if (td.empty()) continue;
         rc = dev_alloc(p.tdesc[dir], td.size() * sizeof(TDesc));
         if (!rc) rc = cuda_status(cudaMemcpyAsync(p.tdesc[dir].p, td.data(), td.size() * sizeof(TDesc),
                                                   cudaMemcpyHostToDevice, stream));
@@ -871,6 +903,8 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
             NatDesc d;
             std::memset(&d, 0, sizeof(d));
             d.a = s->A[3].p; d.c = s->A[1].p;
+            d.a_row = direct(s, 1) ? s->A[0].p : nullptr;
+            d.lda = g.lda;
             d.wn = s->W[1 - pm].p; d.wi = s->W[pm].p;
             d.uo = s->Uo.p; d.wo = s->Wo.p;
             d.clock = (const long long *)s->clock.p;
@@ -1091,8 +1125,13 @@ int run_prologue_t(adi_sim *s) {
     }
     if (e == cudaSuccess)
         e = launch_prologue_lines<T>(cols, s->nlines[1], N, s->g.method, (const T *)s->pro.p, s->stream);
-    // the prologue wrote a column-major (A[3]), like a stage-2 launch
-    if (e == cudaSuccess) e = enqueue_transposes<T>(s->plan, 1, s->stream);
+    // the prologue wrote a column-major (A[3]); the row-major copy that stage 1 reads
+    if (e == cudaSuccess && s->plan.tcount[1]) {
+        e = enqueue_transposes<T>(s->plan, 1, s->stream);
+    } else if (e == cudaSuccess) {  // no transposes in a plan whose lines store a there at once
+        const int rc = transpose(s, s->A[3].p, s->g.ldu, s->g.rows_u, s->g.ldc, s->A[0].p, s->g.lda);
+        if (rc) return rc;
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     return cuda_status(e);
 }

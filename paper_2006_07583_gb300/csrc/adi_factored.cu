@@ -205,6 +205,7 @@ bool fac_supported(int method, int N, size_t esz) {
 }
 size_t fac_words(int method, int N) { return (size_t)fac_rec(fac_geom(method, N)); }
 int fac_chunks(int method, int N) { return fac_geom(method, N).T; }
+bool fac_direct(int method, int N) { return fac_geom(method, N).T < 32; }
 int fac_variant(int method, int N, size_t esz) {
     const int v = fac_variant_of(method, N);
     return fac_narrow(method, fac_geom(method, N).T, esz) ? v + 4 : v;

@@ -153,6 +153,8 @@ int fac_variant(int method, int N, size_t esz);
 int fac_variant_method(int v);
 constexpr int kFacVariants = 7;
 int fac_lines_per_cta(int method, int N, size_t esz);
+// lines of N cells lie within a warp and store their outputs element by element (any stride)
+bool fac_direct(int method, int N);
 size_t fac_stage_bytes(int method, int N, int nl, size_t esz);  // shared memory of one stage
 int fac_stages_for(size_t stage_bytes, size_t esz, int method);  // groups in flight that fit: 3, 2, 1 or 0
 size_t fac_ws_doubles();                 // FP64 workspace per line of the precompute (its ends' dB)

@@ -93,6 +93,41 @@ def test_loading_fields_mid_run(adi, method, nx, ny, fp64):
     _check(G, oracle.run(method, nx, ny, h, dt, c ** 2, U2, V2, W2, 2), fp64)
 
 
+@pytest.mark.parametrize("fp64", [True, False])
+@pytest.mark.parametrize("method,nx,ny,layers", [(CFD, 40, 33, 0), (MFD, 33, 143, 0), (MFD, 144, 30, 0), (CFD, 143, 31, 4),
+                                                 (CFD, 31, 300, 0)])
+def test_short_lines_alone_and_in_a_wide_batch(adi, method, nx, ny, layers, fp64):
+    """Lines of up to 15 chunks store the carried pressure in the next stage's layout at once when their launch is one
+    round of groups, as for the simulation alone, and in their own layout beside members that make it two (CFD and
+    MFD of 1030 cells, whose solves also run on two streams): the steps before, in and after such a batch."""
+    h, dt, c, U, V, W = _case(method, nx, ny, 31)
+    prec = adi.ADI_FP64 if fp64 else adi.ADI_FP32
+    src = (ny // 2, nx // 3, 0.01, 15.0, 0.0)
+    sims = [adi.Sim(method, nx, ny, h, dt, c, U, V, W, precision=prec)]
+    sims[0].set_source(*src)
+    if layers:
+        sims[0].set_sponge(layers, 0.1)
+    for m in (CFD, MFD):
+        bh, bdt, bc, bU, bV, bW = _case(m, 1030, 1030, 32)
+        sims.append(adi.Sim(m, 1030, 1030, bh, bdt, bc, bU, bV, bW, precision=prec))
+    sims[0].step(1)
+    b = adi.Batch(sims)
+    b.step(3)
+    b.sync()
+    b.close()
+    mid = sims[0].read()
+    sims[0].step(2)
+    end = sims[0].read()
+    for s in sims:
+        s.close()
+    for got, n in ((mid, 4), (end, 6)):
+        if layers:
+            want = oracle.run_sponge(method, nx, ny, h, dt, c ** 2, U, V, W, n, layers, 0.1, source=src)
+        else:
+            want = oracle.run(method, nx, ny, h, dt, c ** 2, U, V, W, n, source=src)
+        _check(got, want, fp64)
+
+
 # line counts around a block's four lines; lines so long that a block takes two (FP64 above 7260 cells, FP32 above
 # 14520) or one (FP64 above 14520), or keeps its rows in global memory (FP64 above 28900, FP32 above 57800); the
 # recurrences go sixteen rows at a time
