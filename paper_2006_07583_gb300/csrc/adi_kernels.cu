@@ -400,69 +400,167 @@ __global__ void prologue_mfd_kernel(const LineDesc<T> *__restrict__ descs, int n
 // window that starts inside the line eliminates from its first row as if it had no
 // predecessor; those rows are interior rows, and the start-up factors of that elimination (the
 // last kProH values of the factor buffer) join the whole line's factors within kProH rows.
-constexpr int kProR = 64, kProH = 32;
+constexpr int kProR = 64, kProH = 32, kProU = 16;  // kProU rows at a time
 
-// q(r) gives the right-hand side of row r.  The forward values of rows r0..r1-1 go to
-// tmp[(r - t0) * ts] and are read back by the backward sweep just before out(r, x) is called for
-// the row.
-template <typename T, typename QF, typename Out>
-__host__ __device__ __forceinline__ void prologue_win_solve(int n, int r0, int r1, QF q, const T *lo, const T *cu,
-                                                            const T *id, const T *su_id, T *tmp, long long ts,
-                                                            Out out, int t0 = 0) {
-    const int s = r0 > 0 ? r0 - kProH : 0;
-    const int e = r1 + kProH < n ? r1 + kProH : n;
-    T dd = T(0);
-#pragma unroll 8
-    for (int r = s; r < r0; ++r) dd = (q(r) - dd) * su_id[r - s];  // start-up rows
-#pragma unroll 8
-    for (int r = r0; r < r1; ++r) {
-        dd = (q(r) - lo[r] * dd) * id[r];
-        tmp[(long long)(r - t0) * ts] = dd;
-    }
-    T hh[kProH];
-#pragma unroll
-    for (int k = 0; k < kProH; ++k) {
-        const int r = r1 + k;
-        if (r < e) {
-            dd = (q(r) - lo[r] * dd) * id[r];
-            hh[k] = dd;
-        }
-    }
-    T x = T(0);
-#pragma unroll
-    for (int k = kProH - 1; k >= 0; --k) {
-        const int r = r1 + k;
-        if (r < e) x = hh[k] - cu[r] * x;
-    }
-#pragma unroll 8
-    for (int r = r1 - 1; r >= r0; --r) {
-        x = tmp[(long long)(r - t0) * ts] - cu[r] * x;
-        out(r, x);
-    }
-}
-
-// A warp takes 32 consecutive lines and one chunk of P (N+1 rows) or Pbar (N-1 rows); grid.y times the
-// block's warps: the chunks of P first, then those of Pbar.  The lines' natural fields are row-major, so
-// lane = line reads them coalesced, and the right-hand sides Q u / h and Qbar w / h are formed row by row
-// from them (two reads, one of them still in the L1 from the row before, instead of a pass of its own
-// that wrote them and a read of that), without a branch, so that the rows' loads run ahead of the recurrence: the
-// two boundary rows' values are formed beforehand.  The outputs (w*, a) and alpha are contiguous along each
-// line, so they go through shared memory and move along each line in turn, lane = row, eight lines' loads at
-// a time (one line after the other made a warp wait for alpha 64 times).  Every value is rounded as the two-pass
-// form rounded it.  4096 lines of 4097 rows: 531 -> 305 us with the stencil pass that this replaces; 640 lines of 641 rows 46
-// -> 25 us.
-template <typename T>
-constexpr int kProWarps = sizeof(T) == 4 ? 2 : 1;
+// Products and fused products rounded as written: the compiler may otherwise fuse a product into the sum that follows,
+// or not, as the loop around it happens to be unrolled.
+#ifdef __CUDA_ARCH__
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float fma_of(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_of(double a, double b, double c) { return __fma_rn(a, b, c); }
+#else
+inline float mul_rn(float a, float b) { return a * b; }
+inline double mul_rn(double a, double b) { return a * b; }
+inline float fma_of(float a, float b, float c) { return std::fma(a, b, c); }
+inline double fma_of(double a, double b, double c) { return std::fma(a, b, c); }
+#endif
+
+// One window.  rows.start(r), then rows.next(r, q) for every batch of kProU rows, gives the right-hand sides in order;
+// rows.back_start(r) and rows.back(r, y) the values that out(r, x, y) takes beside the solution, from the last batch
+// down.  lo, cu, id: the factors of row r0 on; su: the start-up factors.  The chunk's forward values go to tmp, those of the
+// rows after it to halo (which out may overwrite).  Every batch is one trip of a rolled loop: a warp runs through
+// this code once, so that straight-line code waits for its instructions, and what a batch loads is asked for a batch ahead.
+// INNER: a whole chunk whose window holds no boundary row, so that the factors of all rows from r0 on are those of row r0
+// (the elimination's factors settle within some 15 rows).
+template <bool INNER, typename T, typename Rows, typename Out>
+__host__ __device__ __forceinline__ void prologue_win_rows(int n, int r0, int r1, Rows rows, const T *lo, const T *cu,
+                                                           const T *id, const T *su, T *tmp, T *halo, long long ts,
+                                                           Out out) {
+    constexpr int U = kProU, S = 8;  // the start-up's value is rounded after every S rows
+    static_assert(kProH % U == 0 && kProR % U == 0 && U % S == 0, "whole batches");
+    const int nr = INNER ? kProR : r1 - r0;
+    const int m = INNER ? kProR + kProH : (r1 + kProH < n ? r1 + kProH : n) - r0;  // m > nr only for nr = kProR
+    const T lo0 = lo[0], id0 = id[0], cu0 = cu[0];
+    T q[U], dd = T(0);
+    rows.start(r0 > 0 ? r0 - kProH : 0);
+    if (r0 > 0) {
+        T t = T(0);
+#pragma unroll 1
+        for (int k = 0; k < kProH; k += U) {
+            rows.next(r0 - kProH + k, q);
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                t = i % S == 0 ? q[i] - dd : fma_of(-t, su[k + i - 1], q[i]);
+                if (i % S == S - 1) dd = mul_rn(t, su[k + i]);
+            }
+        }
+    }
+#pragma unroll 1
+    for (int o = 0; o < m; o += U) {
+        rows.next(r0 + o, q);
+        T *to = o < kProR ? tmp + o * ts : halo + (o - kProR) * ts;
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+            if (INNER || o + i < m) {
+                dd = mul_rn(fma_of(-(INNER ? lo0 : lo[o + i]), dd, q[i]), INNER ? id0 : id[o + i]);
+                to[i * ts] = dd;
+            }
+    }
+    T x = T(0);
+    const int top = (m - 1) / U * U;
+    rows.back_start(r0 + top);
+#pragma unroll 1
+    for (int o = top; o >= 0; o -= U) {
+        const T *from = o < kProR ? tmp + o * ts : halo + (o - kProR) * ts;
+        T f[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) f[i] = INNER || o + i < m ? from[i * ts] : T(0);
+        rows.back(r0 + o, q);
+#pragma unroll
+        for (int i = U - 1; i >= 0; --i)
+            if (INNER || o + i < m) {
+                x = fma_of(-(INNER ? cu0 : cu[o + i]), x, f[i]);
+                if (o < kProR && (INNER || o + i < nr)) out(r0 + o + i, x, q[i]);
+            }
+    }
+}
+
+// The same with right-hand sides q(r) and out(r, x); lo, cu, id of the whole line, forward values in tmp[(r - t0) * ts].
+template <typename T, typename QF>
+struct ProRowsOf {
+    QF q;
+    int n;
+    __host__ __device__ void start(int) {}
+    __host__ __device__ void next(int r, T (&v)[kProU]) {
+        for (int i = 0; i < kProU; ++i) v[i] = r + i < n ? q(r + i) : T(0);
+    }
+    __host__ __device__ void back_start(int) {}
+    __host__ __device__ void back(int, T (&)[kProU]) {}
+};
+template <typename T, typename QF, typename Out>
+__host__ __device__ __forceinline__ void prologue_win_solve(int n, int r0, int r1, QF q, const T *lo, const T *cu,
+                                                            const T *id, const T *su_id, T *tmp, long long ts,
+                                                            Out out, int t0 = 0) {
+    prologue_win_rows<false, T>(n, r0, r1, ProRowsOf<T, QF>{q, n}, lo + r0, cu + r0, id + r0, su_id, tmp + (r0 - t0) * ts,
+                         tmp + (r0 - t0 + kProR) * ts, ts, [&](int r, T x, T) { out(r, x); });
+}
+
+// The rows of the kernel below: q(r) = (3 x(r + 1) - 3 x(r - 1)) ih but for the boundary rows 0 and n - 1, x(k) for k0 <=
+// k <= k1 loaded once each, and y(r).
+template <typename T, bool INNER>
+struct ProRows {
+    const T *x, *y;
+    int xs, ys, k0, k1, n, r0, r1;
+    T ih, first, last, below, at, v[kProU];
+    __device__ T ld(int k) const { return x[(long long)(INNER ? k : min(max(k, k0), k1)) * xs]; }
+    __device__ void start(int s) {
+        below = ld(s - 1);
+        at = ld(s);
+#pragma unroll
+        for (int i = 0; i < kProU; ++i) v[i] = ld(s + 1 + i);
+    }
+    __device__ void next(int r, T (&q)[kProU]) {
+        T w[kProU];
+#pragma unroll
+        for (int i = 0; i < kProU; ++i) w[i] = ld(r + kProU + 1 + i);
+#pragma unroll
+        for (int i = 0; i < kProU; ++i) {
+            q[i] = mul_rn(fma_of(T(3), v[i], mul_rn(T(-3), below)), ih);
+            below = at;
+            at = v[i];
+        }
+#pragma unroll
+        for (int i = 0; i < kProU; ++i) v[i] = w[i];
+        if (INNER) return;
+        if (r == 0) q[0] = first;
+        if (r + kProU >= n)
+#pragma unroll
+            for (int i = 0; i < kProU; ++i)
+                if (r + i == n - 1) q[i] = last;
+    }
+    __device__ void back_start(int r) { ask(r); }
+    __device__ void back(int r, T (&out)[kProU]) {
+#pragma unroll
+        for (int i = 0; i < kProU; ++i) out[i] = v[i];
+        ask(r - kProU);
+    }
+    __device__ void ask(int r) {
+        if (r < r0 || r >= r1) return;  // no batch of the chunk
+#pragma unroll
+        for (int i = 0; i < kProU; ++i) v[i] = y[(long long)(INNER ? r + i : min(r + i, r1 - 1)) * ys];
+    }
+};
+
+// A warp takes 32 consecutive lines and one chunk of P (N+1 rows) or Pbar (N-1 rows); grid.y times the
+// block's warps: the chunks of P first, then those of Pbar.  The lines' natural fields are row-major, so
+// lane = line reads them coalesced, and the right-hand sides Q u / h and Qbar w / h are formed row by row
+// from them instead of in a pass of its own; the two boundary rows' values are formed beforehand.  The outputs
+// (w*, a) and alpha are contiguous along each line, so they go through shared memory and move along each line
+// in turn, lane = row, eight lines' loads at a time (one line after the other made a warp wait for alpha 64
+// times).  Every value is rounded as the two-pass form rounded it.  Few warps are in flight, so latency and, on
+// small grids, the first fetch of the code bound it: with a loop per kind of row unrolled in full and loads where
+// they are used it took 305 us for 4096 lines of 4097 rows, 25 for 640 of 641 and 22 for 63 of 65; now 215, 19 and 17 (the two
+// passes 531 and 46).  Batches of 8 rows: 241 and 21; of 32: as 16 with spills.
+template <typename T>
+constexpr int kProWarps = sizeof(T) == 4 ? 2 : 1;
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kProWarps<T>) prologue_cfd_kernel(const LineDesc<T> *__restrict__ descs, int nlines,
                                                                          int N, const T *__restrict__ fac) {
-    __shared__ T stile[kProWarps<T>][kProR][33];  // per line: the forward values, then the chunk's outputs
-    __shared__ T stu[kProWarps<T>][kProR][33];    // Pbar chunks: u at the chunk's nodes
+    __shared__ T stile[kProWarps<T>][kProR][33];  // per line: the forward values, then the solution
+    __shared__ T stu[kProWarps<T>][kProR][33];    // forward values after the chunk, then w or u at its points
+    __shared__ T sfac[kProWarps<T>][3][kProR + kProH], ssu[kProWarps<T>][kProH];
     __shared__ __align__(16) unsigned char sdesc[32 * sizeof(LineDesc<T>)];
     static_assert(sizeof(LineDesc<T>) % 16 == 0, "descriptor size");
     const int lane = threadIdx.x, warp = threadIdx.y;
@@ -483,86 +581,96 @@ __global__ void __launch_bounds__(32 * kProWarps<T>) prologue_cfd_kernel(const L
     const bool isP = ch < chP;
     const int c = isP ? ch : ch - chP;
     const int r0 = c * kProR, r1 = min(isP ? nP : nB, r0 + kProR), nr = r1 - r0;
-    const T *su_id = fac + 3 * (N + 1) + 3 * (N - 1);
+    // P g = (Q u)/h over rows 0..N, w*_r = w_r - beta g_r; or Pbar e = (Qbar w)/h over nodes 1..N-1 (rows 0..N-2),
+    // a_j = u_j - alpha_j e_j (+ source)
+    const int n = isP ? nP : nB;
+    {
+        const T *f = isP ? fac : fac + 3 * nP, *su = fac + 3 * nP + 3 * nB;
+        const int m = min(r1 + kProH, n) - r0;
+        for (int k = lane; k < m; k += 32) {
+            sfac[warp][0][k] = f[r0 + k];
+            sfac[warp][1][k] = f[n + r0 + k];
+            sfac[warp][2][k] = f[2 * n + r0 + k];
+        }
+        ssu[warp][lane] = su[lane];
+    }
+    __syncwarp();
     if (lane < nl) {
         const LineDesc<T> &d = sd[lane];
-        const T beta = (T)d.beta, ih = (T)d.inv_h;
         const T *__restrict__ un = d.u_out, *__restrict__ wn = d.w_out;
-        const long long snp = d.snp, snv = d.snv;
-        double w[8];
-        int c0;
-        auto row_dot = [&](const T *x, long long st, int n) {
-            T acc = T(0);
-            for (int t = 0; t < n; ++t) acc += (T)w[t] * x[(c0 + t) * st];
-            return mul_rn(acc, ih);
+        const int xs = (int)(isP ? d.snp : d.snv), ys = (int)(isP ? d.snv : d.snp);
+        const T *x = isP ? un : wn + xs, *y = isP ? wn : un + ys;
+        const int k1 = isP ? N : N - 1;
+        const T ih = (T)d.inv_h;
+        auto out = [&](int r, T g, T y_r) {
+            tile[r - r0][lane] = g;
+            tu[r - r0][lane] = y_r;
         };
-        // rows r0 - kProH .. r1 + kProH - 1 at most: inside the line (no boundary row, no clamped address) or not
-        const bool inner = r0 - kProH >= 1 && r1 + kProH <= (isP ? N : N - 2);
-        if (isP) {
-            // P g = (Q u)/h over rows 0..N; w*_r = w_r - beta g_r
-            const T *lo = fac, *cu = fac + (N + 1), *id = fac + 2 * (N + 1);
-            auto qi = [&](int lo_r, int hi_r) -> T {
-                return mul_rn(fma_of(T(3), un[hi_r * snp], mul_rn(T(-3), un[lo_r * snp])), ih);
-            };
-            auto out = [&](int r, T g) { tile[r - r0][lane] = wn[r * snv] - beta * g; };
-            if (inner) {
-                prologue_win_solve<T>(nP, r0, r1, [&](int r) -> T { return qi(r - 1, r + 1); }, lo, cu, id, su_id, &tile[0][lane],
-                                      33, out, r0);
-            } else {
-                const T first = row_dot(un, snp, cfd_Q_row(N, 0, &c0, w)), last = row_dot(un, snp, cfd_Q_row(N, N, &c0, w));
-                prologue_win_solve<T>(nP, r0, r1, [&](int r) -> T {
-                    const T q = qi(max(r - 1, 0), min(r + 1, N));
-                    return r == 0 ? first : r == N ? last : q;
-                }, lo, cu, id, su_id, &tile[0][lane], 33, out, r0);
-            }
+        const T *lo = sfac[warp][0], *cu = sfac[warp][1], *id = sfac[warp][2], *su = ssu[warp];
+        if (r0 > 0 && r1 + kProH < n) {
+            ProRows<T, true> rows{x, y, xs, ys, 0, k1, n, r0, r1, ih};
+            prologue_win_rows<true, T>(n, r0, r1, rows, lo, cu, id, su, &tile[0][lane], &tu[0][lane], 33, out);
         } else {
-            // Pbar e = (Qbar w)/h over nodes 1..N-1 (rows 0..N-2); a_j = u_j - alpha_j e_j (+ source)
-            const T *fb = fac + 3 * (N + 1);
-            const T *lo = fb, *cu = fb + (N - 1), *id = fb + 2 * (N - 1);
-            auto qi = [&](int r) -> T {
-                return mul_rn(fma_of(T(3), wn[(r + 2) * snv], mul_rn(T(-3), wn[r * snv])), ih);
+            auto boundary = [&](int j) {  // the first or last row of Q or Qbar
+                double w[8];
+                int c0;
+                const int cnt = isP ? cfd_Q_row(N, j, &c0, w) : cfd_Qbar_row(N, j, &c0, w);
+                const T *b = isP ? un : wn;
+                T acc = T(0);
+                for (int t = 0; t < cnt; ++t) acc += (T)w[t] * b[(long long)(c0 + t) * xs];
+                return mul_rn(acc, ih);
             };
-            auto out = [&](int r, T e) {
-                tile[r - r0][lane] = e;
-                tu[r - r0][lane] = un[(r + 1) * snp];
-            };
-            if (inner) {
-                prologue_win_solve<T>(nB, r0, r1, qi, lo, cu, id, su_id, &tile[0][lane], 33, out, r0);
-            } else {
-                const T first = row_dot(wn, snv, cfd_Qbar_row(N, 1, &c0, w)), last = row_dot(wn, snv, cfd_Qbar_row(N, N - 1, &c0, w));
-                prologue_win_solve<T>(nB, r0, r1, [&](int r) -> T {
-                    const T q = qi(r);
-                    return r == 0 ? first : r == N - 2 ? last : q;
-                }, lo, cu, id, su_id, &tile[0][lane], 33, out, r0);
-            }
-            if (c == 0) {
-                d.po[0] = un[0];
-                d.po[(long long)N * d.spo] = un[(long long)N * snp];
-            }
+            ProRows<T, false> rows{x, y, xs, ys, isP ? 0 : -1, k1, n, r0, r1, ih};
+            rows.first = r0 == 0 ? boundary(isP ? 0 : 1) : T(0);
+            rows.last = r1 + kProH >= n ? boundary(isP ? N : N - 1) : T(0);
+            prologue_win_rows<false, T>(n, r0, r1, rows, lo, cu, id, su, &tile[0][lane], &tu[0][lane], 33, out);
+        }
+        if (!isP && c == 0) {
+            d.po[0] = un[0];
+            d.po[(long long)N * d.spo] = un[(long long)N * d.snp];
         }
     }
     __syncwarp();
-    for (int k = lane; k < nr; k += 32)
-        for (int l0 = 0; l0 < nl; l0 += 8) {
-            if (isP) {
+    // the chunk's outputs, lane = row, a line's two halves and some lines' loads at a time
+    constexpr int L = 8, K = kProR / 32;
+    for (int l0 = 0; l0 < nl; l0 += L) {
+        if (isP) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (l0 + i < nl) sd[l0 + i].v[(r0 + k) * sd[l0 + i].sv] = tile[k][l0 + i];
-            } else {
-                const long long j = r0 + k + 1;
-                T al[8];
+            for (int i = 0; i < L; ++i) {
+                if (l0 + i >= nl) break;
+                const LineDesc<T> &dl = sd[l0 + i];
+                T *w = dl.v + (r0 + lane) * dl.sv;
+                const T beta = (T)dl.beta;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) al[i] = l0 + i < nl ? sd[l0 + i].alpha[j * sd[l0 + i].sp] : T(0);
+                for (int k = 0; k < K; ++k)
+                    if (lane + 32 * k < nr)
+                        w[32 * k * dl.sv] = fma_of(-beta, tile[lane + 32 * k][l0 + i], tu[lane + 32 * k][l0 + i]);
+            }
+        } else {
+            const long long j = r0 + lane + 1;
+            T al[L][K];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    if (l0 + i >= nl) break;
-                    const LineDesc<T> &dl = sd[l0 + i];
-                    T val = tu[k][l0 + i] - al[i] * tile[k][l0 + i];
-                    if (j == dl.src_k) val += prologue_src(dl);
-                    dl.po[j * dl.spo] = val;
+            for (int i = 0; i < L; ++i) {
+                const LineDesc<T> &dl = sd[min(l0 + i, nl - 1)];
+                const T *a = dl.alpha + j * dl.sp;
+#pragma unroll
+                for (int k = 0; k < K; ++k) al[i][k] = lane + 32 * k < nr ? a[32 * k * dl.sp] : T(0);
+            }
+#pragma unroll
+            for (int i = 0; i < L; ++i) {
+                if (l0 + i >= nl) break;
+                const LineDesc<T> &dl = sd[l0 + i];
+                T *po = dl.po + j * dl.spo;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    if (lane + 32 * k >= nr) break;
+                    T val = fma_of(-al[i][k], tile[lane + 32 * k][l0 + i], tu[lane + 32 * k][l0 + i]);
+                    if (j + 32 * k == dl.src_k) val += prologue_src(dl);
+                    po[32 * k * dl.spo] = val;
                 }
             }
         }
+    }
 }
 
 // Sets *flag if any x[i] is NaN or infinite: 16-byte loads over the aligned body of x (when x
