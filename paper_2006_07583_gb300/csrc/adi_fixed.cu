@@ -183,14 +183,12 @@ __host__ __device__ inline int fp_pitch(int N) { return (N + 2) | 1; }
 // Explicit right-hand side of a stage along its explicit direction:
 //   ov = vl - beta Du(ul)   (all N+1 velocities),   oa = ul - alpha Dv(vl)   (interior)
 // ul0 / ul1 (and vl0 / vl1): the iterate's buffers, picked by the parity of st->k (st may be null).
-// FAR: a line's rows do not fit shared memory and go through the block's part of far_rows instead.
-template <typename T, bool FAR>
+template <typename T>
 __global__ void __launch_bounds__(kFpThreads) fp_rhs_kernel(int method, FpLines g, T ih, T beta, const T *ul0, const T *ul1,
                                                             const T *vl0, const T *vl1, const T *__restrict__ alpha, T *ov,
-                                                            T *oa, FpTri<T> P, FpTri<T> Pb, const FpState *st, int lines,
-                                                            T *far_rows) {
+                                                            T *oa, FpTri<T> P, FpTri<T> Pb, const FpState *st, int lines) {
     extern __shared__ __align__(16) unsigned char fp_smem[];
-    T *x = FAR ? far_rows + (size_t)blockIdx.x * lines * fp_pitch(g.N) : (T *)fp_smem;
+    T *x = (T *)fp_smem;
     const bool odd = st && (st->k & 1);
     const T *ul = odd ? ul1 : ul0, *vl = odd ? vl1 : vl0;
     const FpShare sh(g, lines);
@@ -225,14 +223,14 @@ __device__ __forceinline__ double fp_diff(float x, float y) {
 //   v_{k+1} = vb - beta Du(u_{k+1}),
 // with the squared norms of the two updates; the last block to finish does the stopping test (the
 // paper's: the sum of the two Frobenius norms against eps, or kmax sweeps).
-template <typename T, bool FAR>
+template <typename T>
 __global__ void __launch_bounds__(kFpThreads) fp_sweep_kernel(int method, FpLines g, T ih, T beta, const T *__restrict__ a,
                                                               T *u0, T *u1, T *v0, T *v1, const T *__restrict__ vb,
                                                               const T *__restrict__ alpha, FpTri<T> P, FpTri<T> Pb,
-                                                              FpState *st, double eps, int kmax, int lines, T *far_rows) {
+                                                              FpState *st, double eps, int kmax, int lines) {
     if (st->done) return;
     extern __shared__ __align__(16) unsigned char fp_smem[];
-    T *x = FAR ? far_rows + (size_t)blockIdx.x * lines * fp_pitch(g.N) : (T *)fp_smem;
+    T *x = (T *)fp_smem;
     const bool odd = st->k & 1;
     const T *uk = odd ? u1 : u0, *vk = odd ? v1 : v0;
     T *un = odd ? u0 : u1, *vn = odd ? v0 : v1;
@@ -400,29 +398,20 @@ int run_fixed(int method, int nx, int ny, double h, double dt, const double *c_f
     FpLines rows{1, piy, nx, cfd ? nx : nx + 1, (long long)cu, 1, (long long)cv, 1};
     FpLines cols{1, pix, ny, cfd ? ny : ny + 1, 1, (long long)cu, 1, (long long)cw};
     const T ih = (T)(1.0 / h), beta = (T)(0.5 * dt);
-    // lines per block: four, fewer where their rows would not fit shared memory (beside the norms' 128 bytes); lines that
-    // do not fit alone keep their rows in global memory
+    // lines per block: four, fewer where their rows would not fit shared memory beside the norms' 128 bytes (the longest
+    // line, ADI_MAX_CELLS in FP64, takes 131 KB)
     constexpr size_t kSmem = 226 * 1024;
-    auto far = [&](const FpLines &g) { return fp_pitch(g.N) * sizeof(T) > kSmem; };
+    static_assert((ADI_MAX_CELLS + 3) * sizeof(double) <= kSmem, "one line fits");
     auto lines_of = [&](const FpLines &g) {
         int n = kFpLines;
-        while (!far(g) && n > 1 && (size_t)n * fp_pitch(g.N) * sizeof(T) > kSmem) n /= 2;
+        while (n > 1 && (size_t)n * fp_pitch(g.N) * sizeof(T) > kSmem) n /= 2;
         return n;
     };
-    auto smem = [&](const FpLines &g) { return far(g) ? 0 : (size_t)lines_of(g) * fp_pitch(g.N) * sizeof(T); };
+    auto smem = [&](const FpLines &g) { return (size_t)lines_of(g) * fp_pitch(g.N) * sizeof(T); };
     auto grid = [&](const FpLines &g) { return (unsigned)((g.n + lines_of(g) - 1) / lines_of(g)); };
-    auto rhs = [&](const FpLines &g) { return far(g) ? fp_rhs_kernel<T, true> : fp_rhs_kernel<T, false>; };
-    auto sweep = [&](const FpLines &g) { return far(g) ? fp_sweep_kernel<T, true> : fp_sweep_kernel<T, false>; };
-    DevArr far_mem;
-    size_t far_n = 0;
-    for (const FpLines *g : {&rows, &cols})
-        if (far(*g)) far_n = std::max(far_n, (size_t)grid(*g) * lines_of(*g) * fp_pitch(g->N));
-    if (far_n && cudaMalloc(&far_mem.p, far_n * sizeof(T)) != cudaSuccess) { (void)cudaGetLastError(); return ADI_ENOMEM; }
-    T *far_rows = (T *)far_mem.p;
     const int most = (int)std::max(smem(rows), smem(cols));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_rhs_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fp_sweep_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_rhs_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) { (void)cudaGetLastError(); return ADI_ECUDA; }
     FpState *st = (FpState *)state.p;
     auto copy = [&](int dst, int src0, int src1, size_t n, const FpState *s) {
@@ -444,29 +433,29 @@ int run_fixed(int method, int nx, int ny, double h, double dt, const double *c_f
         copy(dVs, dV, dV, nV, nullptr);
         copy(dUk, dU, dU, nU, nullptr);
         copy(dVk, dV, dV, nV, nullptr);
-        rhs(cols)<<<grid(cols), kFpThreads, smem(cols)>>>(method, cols, ih, beta, P(dU), P(dU), P(dW), P(dW), P(dAl),
-                                                                 P(dWs), P(dA), Py, Pby, nullptr, lines_of(cols), far_rows);
+        fp_rhs_kernel<T><<<grid(cols), kFpThreads, smem(cols)>>>(method, cols, ih, beta, P(dU), P(dU), P(dW), P(dW), P(dAl),
+                                                                 P(dWs), P(dA), Py, Pby, nullptr, lines_of(cols));
         if (src) fp_source_kernel<T><<<1, 1>>>(P(dA), sp, sscale, src[2], src[3], src[4], t);
         fp_reset_kernel<<<1, 1>>>(st);
         for (int k = 0; k < kmax; ++k)
-            sweep(rows)<<<grid(rows), kFpThreads, smem(rows)>>>(method, rows, ih, beta, P(dA), P(dUk), P(dUs), P(dVk),
+            fp_sweep_kernel<T><<<grid(rows), kFpThreads, smem(rows)>>>(method, rows, ih, beta, P(dA), P(dUk), P(dUs), P(dVk),
                                                                        P(dVs), P(dV), P(dAl), Px, Pbx, st, eps, kmax,
-                                                                       lines_of(rows), far_rows);
+                                                                       lines_of(rows));
         // ---- stage 2: v^{m+1} and C explicit along x (rows), then y-line sweeps from u* and w^m,
         // alternating between (Uk, Wk) and (Un, Wn) ----
         copy(dVn, dVk, dVs, nV, st);
         copy(dUn, dUk, dUs, nU, st);
-        rhs(rows)<<<grid(rows), kFpThreads, smem(rows)>>>(method, rows, ih, beta, P(dUk), P(dUs), P(dVk), P(dVs),
-                                                                 P(dAl), P(dVn), P(dA), Px, Pbx, st, lines_of(rows), far_rows);
+        fp_rhs_kernel<T><<<grid(rows), kFpThreads, smem(rows)>>>(method, rows, ih, beta, P(dUk), P(dUs), P(dVk), P(dVs),
+                                                                 P(dAl), P(dVn), P(dA), Px, Pbx, st, lines_of(rows));
         if (src) fp_source_kernel<T><<<1, 1>>>(P(dA), sp, sscale, src[2], src[3], src[4], t + dt);
         copy(dUk, dUn, dUn, nU, nullptr);
         copy(dWn, dWs, dWs, nW, nullptr);
         copy(dWk, dW, dW, nW, nullptr);
         fp_reset_kernel<<<1, 1>>>(st);
         for (int k = 0; k < kmax; ++k)
-            sweep(cols)<<<grid(cols), kFpThreads, smem(cols)>>>(method, cols, ih, beta, P(dA), P(dUk), P(dUn), P(dWk),
+            fp_sweep_kernel<T><<<grid(cols), kFpThreads, smem(cols)>>>(method, cols, ih, beta, P(dA), P(dUk), P(dUn), P(dWk),
                                                                        P(dWn), P(dWs), P(dAl), Py, Pby, st, eps, kmax,
-                                                                       lines_of(cols), far_rows);
+                                                                       lines_of(cols));
         copy(dU, dUk, dUn, nU, st);
         copy(dV, dVn, dVn, nV, nullptr);
         copy(dW, dWk, dWn, nW, st);

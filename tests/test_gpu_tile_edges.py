@@ -128,13 +128,13 @@ def test_short_lines_alone_and_in_a_wide_batch(adi, method, nx, ny, layers, fp64
         _check(got, want, fp64)
 
 
-# line counts around a block's four lines; lines so long that a block takes two (FP64 above 7260 cells, FP32 above
-# 14520) or one (FP64 above 14520), or keeps its rows in global memory (FP64 above 28900, FP32 above 57800); the
-# recurrences go sixteen rows at a time
+# line counts around a block's four lines; lines so long that a block takes two (FP64 above about 7230 cells, FP32 above
+# 14460) or one (FP64 above 14460; 14522 would fit twice but for the block's other shared memory); the recurrences go
+# sixteen rows at a time
 @pytest.mark.parametrize("method,nx,ny,fp64", [(CFD, 16, 17, True), (CFD, 17, 18, False), (MFD, 18, 19, True),
                                                (CFD, 23, 24, True), (CFD, 25, 320, False), (CFD, 7300, 16, True),
                                                (CFD, 16, 14600, True), (MFD, 15000, 16, False),
-                                               (CFD, 29000, 16, True), (MFD, 16, 58000, False)])
+                                               (CFD, 14522, 16, True)])
 def test_fixed_point_blocks(adi, method, nx, ny, fp64):
     h, dt, c, U, V, W = _case(method, nx, ny, 21, cfl=0.6)
     src = (ny // 2, nx // 3, 0.01, 15.0, 0.0)
