@@ -208,8 +208,9 @@ struct Plan {
         const void *ydesc[2];     // y-line descriptors of the next step's parity
         int nlines = 0, N = 0, method = 0;
         const void *fac = nullptr;  // CFD: the prologue's Thomas factors
-        void *A3 = nullptr, *A0 = nullptr;
-        int rows_u = 0, ldu = 0, ldc = 0, lda = 0;
+        const void *alpha = nullptr;
+        void *A0 = nullptr;       // the rebuilt a, row-major
+        int rows_u = 0, ldu = 0, lda = 0;
         int harm = -1;            // index of the member's harmonic record, or -1
     };
     std::vector<SpongeStep> sponges;
@@ -462,13 +463,13 @@ __global__ void transpose_kernel(const T *__restrict__ src, int rows, int cols, 
 // The entries of the carried arrays that no line writes, from the natural fields: the outer rows and columns
 // of the pressure arrays (the Dirichlet data), the first and last columns of both w* copies and the first and
 // last rows of the v copy that the next step writes.  Everything else of these arrays is written before
-// it is read (A[1] and A[2] by stage 1, A[3] and the current w* by the prologue, the other w* and v copies by
+// it is read (A[1] and A[2] by stage 1, A[0] and the current w* by the prologue, A[3] by stage 2, the other w* and v copies by
 // the step), so loading new fields copies edges only: at 4096^2 four transposes and three copies of whole
 // fields (300 us) became one launch of 5 us.
 template <typename T>
 struct EdgeRec {
     const T *u, *w, *v;     // natural u (rows_u x ldu), w (rows_w x ldw); the current v (leading dimension ldvp)
-    T *a1, *a2, *a3;        // A[1] (column-major, ldc), A[2] (row-major, lda), A[3] (as A[1])
+    T *a0, *a1, *a2, *a3;   // A[0], A[2] (row-major, lda), A[1], A[3] (column-major, ldc)
     T *w0, *w1, *vo;        // both w* copies (column-major, ldwc), the other v copy
     int rows_u, ldu, rows_w, ldw, rows_v, ldv, lda, ldc, ldwc, ldvp;
 };
@@ -478,12 +479,14 @@ __global__ void edges_kernel(EdgeRec<T> r) {
     const size_t lr = r.rows_u - 1, lc = r.ldu - 1, wc = r.ldw - 1, vr = r.rows_v - 1;
     if (k <= lc) {  // first and last rows of u
         const T a = r.u[k], b = r.u[lr * r.ldu + k];
+        r.a0[k] = a; r.a0[lr * r.lda + k] = b;
         r.a2[k] = a; r.a2[lr * r.lda + k] = b;
         r.a1[k * r.ldc] = a; r.a1[k * r.ldc + lr] = b;
         r.a3[k * r.ldc] = a; r.a3[k * r.ldc + lr] = b;
     }
     if (k <= lr) {  // first and last columns
         const T a = r.u[k * r.ldu], b = r.u[k * r.ldu + lc];
+        r.a0[k * r.lda] = a; r.a0[k * r.lda + lc] = b;
         r.a2[k * r.lda] = a; r.a2[k * r.lda + lc] = b;
         r.a1[k] = a; r.a1[lc * r.ldc + k] = b;
         r.a3[k] = a; r.a3[lc * r.ldc + k] = b;
@@ -971,8 +974,8 @@ int plan_build(Plan &p, const std::vector<adi_sim *> &members, cudaStream_t stre
         }
         sp.nlines = s->nlines[1]; sp.N = g.ny; sp.method = g.method;
         sp.fac = s->sp_fac.p;
-        sp.A3 = s->A[3].p; sp.A0 = s->A[0].p;
-        sp.rows_u = g.rows_u; sp.ldu = g.ldu; sp.ldc = g.ldc; sp.lda = g.lda;
+        sp.alpha = s->alpha.p; sp.A0 = s->A[0].p;
+        sp.rows_u = g.rows_u; sp.ldu = g.ldu; sp.lda = g.lda;
         sp.harm = my_h;
         p.sponges.push_back(sp);
     }
@@ -1075,13 +1078,8 @@ cudaError_t enqueue_stage(const Plan &p, int q, int dir, int natural, cudaStream
             e = launch_sponge<T>(sp.rec[q], stream);
             if (e == cudaSuccess)
                 e = launch_prologue_lines<T>((const LineDesc<T> *)sp.ydesc[q], sp.nlines, sp.N, sp.method,
-                                             (const T *)sp.fac, stream);
-            if (e == cudaSuccess) {  // the prologue wrote a column-major (A[3]); a row-major copy
-                dim3 grid((unsigned)((sp.rows_u + 31) / 32), (unsigned)((sp.ldu + 31) / 32)), block(32, 8);
-                transpose_kernel<T><<<grid, block, 0, stream>>>((const T *)sp.A3, sp.ldu, sp.rows_u, sp.ldc,
-                                                                (T *)sp.A0, sp.lda);
-                e = cudaGetLastError();
-            }
+                                             (const T *)sp.fac, (const T *)sp.alpha + 1, sp.lda, (T *)sp.A0 + 1, sp.lda,
+                                             stream);
             if (e == cudaSuccess && sp.harm >= 0)
                 e = launch_harmonic<T>((const HarmDesc *)p.hdesc.p + sp.harm, 1, (size_t)sp.rows_u * sp.ldu, 3, stream);
         }
@@ -1166,14 +1164,8 @@ int run_prologue_t(adi_sim *s) {
         if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);  // ft leaves scope
     }
     if (e == cudaSuccess)
-        e = launch_prologue_lines<T>(cols, s->nlines[1], N, s->g.method, (const T *)s->pro.p, s->stream);
-    // the prologue wrote a column-major (A[3]); the row-major copy that stage 1 reads
-    if (e == cudaSuccess && s->plan.tcount[1]) {
-        e = enqueue_transposes<T>(s->plan, 1, s->stream);
-    } else if (e == cudaSuccess) {  // no transposes in a plan whose lines store a there at once
-        const int rc = transpose(s, s->A[3].p, s->g.ldu, s->g.rows_u, s->g.ldc, s->A[0].p, s->g.lda);
-        if (rc) return rc;
-    }
+        e = launch_prologue_lines<T>(cols, s->nlines[1], N, s->g.method, (const T *)s->pro.p, (const T *)s->alpha.p + 1,
+                                     s->g.lda, (T *)s->A[0].p + 1, s->g.lda, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     return cuda_status(e);
 }
@@ -1335,7 +1327,7 @@ int set_edges(adi_sim *s) {
     const int cur = s->parity;
     EdgeRec<T> r;
     r.u = (const T *)s->Uo.p; r.w = (const T *)s->Wo.p; r.v = (const T *)s->V[cur].p;
-    r.a1 = (T *)s->A[1].p; r.a2 = (T *)s->A[2].p; r.a3 = (T *)s->A[3].p;
+    r.a0 = (T *)s->A[0].p; r.a1 = (T *)s->A[1].p; r.a2 = (T *)s->A[2].p; r.a3 = (T *)s->A[3].p;
     r.w0 = (T *)s->W[0].p; r.w1 = (T *)s->W[1].p; r.vo = (T *)s->V[1 - cur].p;
     r.rows_u = g.rows_u; r.ldu = g.ldu; r.rows_w = g.rows_w; r.ldw = g.ldw; r.rows_v = g.rows_v; r.ldv = g.ldv;
     r.lda = g.lda; r.ldc = g.ldc; r.ldwc = g.ldwc; r.ldvp = g.ldvp;

@@ -62,10 +62,11 @@ void prologue_factors(int N, std::vector<double> &out);
 void prologue_factors(int N, double *out);
 size_t prologue_factor_count(int N);
 // The prologue over the y-lines of one simulation (N cells each), spread over the lines' elements;
-// fac: the Thomas factors of prologue_factors() in T (CFD; nullptr for MFD).
+// fac: the Thomas factors of prologue_factors() in T (CFD; nullptr for MFD).  al, a: the first line's column of the row-major
+// alpha (leading dimension ald) and of the row-major carried a that is written (lda); line k is k columns on.
 template <typename T>
-cudaError_t launch_prologue_lines(const LineDesc<T> *col_lines, int nlines, int N, int method, const T *fac,
-                                  cudaStream_t s);
+cudaError_t launch_prologue_lines(const LineDesc<T> *col_lines, int nlines, int N, int method, const T *fac, const T *al,
+                                  int ald, T *a, int lda, cudaStream_t s);
 template <typename T>
 cudaError_t launch_finite_check(const T *x, size_t n, int *flag, cudaStream_t s);
 

@@ -288,10 +288,10 @@ __global__ void __launch_bounds__(32) line_solve_short_kernel(const LineDesc<T> 
 
 // ---------------------------------------------------------------------------------------
 // Prologue: carried state from natural fields, along the stage-2 (y) lines.
-//   a_k  = u_k - alpha_k (Dv w)_k + dt/2 f(t_m)   (interior pressure points) -> d.po
+//   a_k  = u_k - alpha_k (Dv w)_k + dt/2 f(t_m)   (interior pressure points) -> a
 //   w*_j = w_j - beta (Du u)_j                      (all velocity points)     -> d.v
-// (d.po of a stage-2 line is the stage-1 input buffer; d.v is the stage-2 input; the
-// natural u and w are read through d.u_out and d.w_out.)
+// (a is the row-major stage-1 input; d.v is the stage-2 input; the natural u and w are read through d.u_out
+// and d.w_out.)
 // CFD derivatives solve Pbar e = Qbar w and P g = Q u by the Thomas algorithm, with the
 // factors of the two constant matrices precomputed (fac: P's sub-diagonal, eliminated
 // super-diagonal and inverse pivots, N+1 each, then Pbar's, N-1 each).
@@ -319,10 +319,11 @@ __device__ __forceinline__ T mfd_interior_dot(const T *p, long long s) {
 }
 
 template <typename T>
-__global__ void prologue_mfd_kernel(const LineDesc<T> *__restrict__ descs, int nlines, int N) {
+__global__ void prologue_mfd_kernel(const LineDesc<T> *__restrict__ descs, int nlines, int N, const T *__restrict__ al,
+                                    int ald, T *__restrict__ a, int lda) {
     // block (32 lines, 8): elements j0 .. j0 + 31 of 32 consecutive lines; lane = line reads the
-    // row-major natural fields coalesced; w* and a, which are contiguous along each line, are written
-    // through shared memory, along each line in turn.
+    // row-major natural fields and alpha and writes the row-major a coalesced; w*, which is contiguous along each
+    // line, is written through shared memory, along each line in turn.
     __shared__ T tv[32][33], tp[32][33], tu[32][33];
     // the block's 32 descriptors, copied once with 16-byte loads (each thread would otherwise
     // read its own descriptor's fields, 32 scattered sectors per load)
@@ -362,7 +363,7 @@ __global__ void prologue_mfd_kernel(const LineDesc<T> *__restrict__ descs, int n
             }
             tu[jj][x] = un[j * snp];
             if (j >= 1 && j <= N) {
-                // a = u - alpha (D w)/h (+ source), formed below along the line
+                // a = u - alpha (D w)/h (+ source), formed below
                 T acc = T(0);
                 if (j >= 2 && j <= N - 1) {
                     acc = mfd_interior_dot(wn + (long long)(j - 2) * snv, snv);
@@ -375,18 +376,24 @@ __global__ void prologue_mfd_kernel(const LineDesc<T> *__restrict__ descs, int n
         }
     }
     __syncthreads();
-    // lane = element: 8 lines at a time, 32 consecutive elements each
+    // w*, lane = element: 8 lines at a time, 32 consecutive elements each
     for (int l = y; l < 32 && line0 + l < nlines; l += 8) {
         const LineDesc<T> &dl = sd[l];
         const int j = j0 + x;
-        if (j > N + 1) continue;
         if (j <= N) dl.v[(long long)j * dl.sv] = tv[x][l];
-        T val = tu[x][l];  // j = 0 or N+1: Dirichlet, u itself
+    }
+    // a, lane = line
+    if (line >= nlines) return;
+    const LineDesc<T> &d = sd[x];
+    for (int jj = y; jj < 32; jj += 8) {
+        const int j = j0 + jj;
+        if (j > N + 1) break;
+        T val = tu[jj][x];  // j = 0 or N+1: Dirichlet, u itself
         if (j >= 1 && j <= N) {
-            val = val - dl.alpha[(long long)j * dl.sp] * tp[x][l] * (T)dl.inv_h;
-            if (j == dl.src_k) val += prologue_src(dl);
+            val = val - al[(long long)j * ald + line] * tp[jj][x] * (T)d.inv_h;
+            if (j == d.src_k) val += prologue_src(d);
         }
-        dl.po[(long long)j * dl.spo] = val;
+        a[(long long)j * lda + line] = val;
     }
 }
 
@@ -545,19 +552,21 @@ struct ProRows {
 // A warp takes 32 consecutive lines and one chunk of P (N+1 rows) or Pbar (N-1 rows); grid.y times the
 // block's warps: the chunks of P first, then those of Pbar.  The lines' natural fields are row-major, so
 // lane = line reads them coalesced, and the right-hand sides Q u / h and Qbar w / h are formed row by row
-// from them instead of in a pass of its own; the two boundary rows' values are formed beforehand.  The outputs
-// (w*, a) and alpha are contiguous along each line, so they go through shared memory and move along each line
-// in turn, lane = row, eight lines' loads at a time (one line after the other made a warp wait for alpha 64
-// times).  Every value is rounded as the two-pass form rounded it.  Few warps are in flight, so latency and, on
-// small grids, the first fetch of the code bound it: with a loop per kind of row unrolled in full and loads where
-// they are used it took 305 us for 4096 lines of 4097 rows, 25 for 640 of 641 and 22 for 63 of 65; now 215, 19 and 17 (the two
-// passes 531 and 46).  Batches of 8 rows: 241 and 21; of 32: as 16 with spills.
+// from them instead of in a pass of its own; the two boundary rows' values are formed beforehand.  a, in the
+// layout that stage 1 reads, and alpha are row-major too; w* is contiguous along each line and is written through
+// shared memory, lane = row.  (a in the y-lines' layout went the same way, with a transpose after it: 20 steps and
+// the read of 640 x 640 cells with absorbing layers 1042 us, now 975.)  Every value is rounded as the two-pass form
+// rounded it.  Few warps are in flight, so latency and, on small grids, the first fetch of the code bound it:
+// with a loop per kind of row unrolled in full and loads where they are used it took 305 us for 4096 lines of 4097
+// rows, 25 for 640 of 641 and 22 for 63 of 65; now 208, 17 and 16 (the two passes 531 and 46).  Rows in batches of 8: 11 %
+// slower; of 32: as 16, with spills.
 template <typename T>
 constexpr int kProWarps = sizeof(T) == 4 ? 2 : 1;
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kProWarps<T>) prologue_cfd_kernel(const LineDesc<T> *__restrict__ descs, int nlines,
-                                                                         int N, const T *__restrict__ fac) {
+                                                                         int N, const T *__restrict__ fac, const T *__restrict__ al,
+                                                                         int ald, T *__restrict__ a, int lda) {
     __shared__ T stile[kProWarps<T>][kProR][33];  // per line: the forward values, then the solution
     __shared__ T stu[kProWarps<T>][kProR][33];    // forward values after the chunk, then w or u at its points
     __shared__ T sfac[kProWarps<T>][3][kProR + kProH], ssu[kProWarps<T>][kProH];
@@ -626,48 +635,37 @@ __global__ void __launch_bounds__(32 * kProWarps<T>) prologue_cfd_kernel(const L
             prologue_win_rows<false, T>(n, r0, r1, rows, lo, cu, id, su, &tile[0][lane], &tu[0][lane], 33, out);
         }
         if (!isP && c == 0) {
-            d.po[0] = un[0];
-            d.po[(long long)N * d.spo] = un[(long long)N * d.snp];
+            a[line0 + lane] = un[0];
+            a[(long long)N * lda + line0 + lane] = un[(long long)N * d.snp];
         }
     }
     __syncwarp();
-    // the chunk's outputs, lane = row, a line's two halves and some lines' loads at a time
-    constexpr int L = 8, K = kProR / 32;
-    for (int l0 = 0; l0 < nl; l0 += L) {
-        if (isP) {
+    if (isP) {  // w*, lane = row, a line's two halves at a time
+#pragma unroll 8
+        for (int l = 0; l < nl; ++l) {
+            const LineDesc<T> &dl = sd[l];
+            T *w = dl.v + (r0 + lane) * dl.sv;
+            const T beta = (T)dl.beta;
 #pragma unroll
-            for (int i = 0; i < L; ++i) {
-                if (l0 + i >= nl) break;
-                const LineDesc<T> &dl = sd[l0 + i];
-                T *w = dl.v + (r0 + lane) * dl.sv;
-                const T beta = (T)dl.beta;
+            for (int k = 0; k < kProR / 32; ++k)
+                if (lane + 32 * k < nr) w[32 * k * dl.sv] = fma_of(-beta, tile[lane + 32 * k][l], tu[lane + 32 * k][l]);
+        }
+    } else if (lane < nl) {  // a, lane = line, some rows' loads at a time
+        const LineDesc<T> &d = sd[lane];
+        const T *al_r = al + (long long)(r0 + 1) * ald + line0 + lane;
+        T *a_r = a + (long long)(r0 + 1) * lda + line0 + lane;
+        const int src = d.src_k - (r0 + 1);
+#pragma unroll 1
+        for (int k = 0; k < nr; k += kProU) {
+            T v[kProU];
 #pragma unroll
-                for (int k = 0; k < K; ++k)
-                    if (lane + 32 * k < nr)
-                        w[32 * k * dl.sv] = fma_of(-beta, tile[lane + 32 * k][l0 + i], tu[lane + 32 * k][l0 + i]);
-            }
-        } else {
-            const long long j = r0 + lane + 1;
-            T al[L][K];
+            for (int i = 0; i < kProU; ++i) v[i] = k + i < nr ? al_r[(long long)(k + i) * ald] : T(0);
 #pragma unroll
-            for (int i = 0; i < L; ++i) {
-                const LineDesc<T> &dl = sd[min(l0 + i, nl - 1)];
-                const T *a = dl.alpha + j * dl.sp;
-#pragma unroll
-                for (int k = 0; k < K; ++k) al[i][k] = lane + 32 * k < nr ? a[32 * k * dl.sp] : T(0);
-            }
-#pragma unroll
-            for (int i = 0; i < L; ++i) {
-                if (l0 + i >= nl) break;
-                const LineDesc<T> &dl = sd[l0 + i];
-                T *po = dl.po + j * dl.spo;
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    if (lane + 32 * k >= nr) break;
-                    T val = fma_of(-al[i][k], tile[lane + 32 * k][l0 + i], tu[lane + 32 * k][l0 + i]);
-                    if (j + 32 * k == dl.src_k) val += prologue_src(dl);
-                    po[32 * k * dl.spo] = val;
-                }
+            for (int i = 0; i < kProU; ++i) {
+                if (k + i >= nr) break;
+                T val = fma_of(-v[i], tile[k + i][lane], tu[k + i][lane]);
+                if (k + i == src) val += prologue_src(d);
+                a_r[(long long)(k + i) * lda] = val;
             }
         }
     }
@@ -729,14 +727,16 @@ cudaError_t launch_line_solve_short(const LineDesc<T> *d, int nlines, int method
 }
 
 template <typename T>
-cudaError_t launch_prologue_lines(const LineDesc<T> *d, int nlines, int N, int method, const T *fac, cudaStream_t s) {
+cudaError_t launch_prologue_lines(const LineDesc<T> *d, int nlines, int N, int method, const T *fac, const T *al, int ald,
+                                  T *a, int lda, cudaStream_t s) {
     if (nlines <= 0) return cudaSuccess;
     const unsigned gx = (unsigned)((nlines + 31) / 32);
     if (method == kCFD) {
         const int chunks = (N + 1 + kProR - 1) / kProR + (N - 1 + kProR - 1) / kProR, w = kProWarps<T>;
-        prologue_cfd_kernel<T><<<dim3(gx, (unsigned)((chunks + w - 1) / w)), dim3(32, w), 0, s>>>(d, nlines, N, fac);
+        prologue_cfd_kernel<T><<<dim3(gx, (unsigned)((chunks + w - 1) / w)), dim3(32, w), 0, s>>>(d, nlines, N, fac, al, ald,
+                                                                                                  a, lda);
     } else {
-        prologue_mfd_kernel<T><<<dim3(gx, (unsigned)((N + 2 + 31) / 32)), dim3(32, 8), 0, s>>>(d, nlines, N);
+        prologue_mfd_kernel<T><<<dim3(gx, (unsigned)((N + 2 + 31) / 32)), dim3(32, 8), 0, s>>>(d, nlines, N, al, ald, a, lda);
     }
     return cudaGetLastError();
 }
@@ -794,7 +794,7 @@ cudaError_t launch_finite_check(const T *x, size_t n, int *flag, cudaStream_t s)
     template cudaError_t launch_line_solve_v1<T>(const LineDesc<T> *, int, T *, long long,   \
                                                  int, cudaStream_t);                         \
     template cudaError_t launch_line_solve_short<T>(const LineDesc<T> *, int, int, int, int, cudaStream_t); \
-    template cudaError_t launch_prologue_lines<T>(const LineDesc<T> *, int, int, int, const T *, cudaStream_t); \
+    template cudaError_t launch_prologue_lines<T>(const LineDesc<T> *, int, int, int, const T *, const T *, int, T *, int, cudaStream_t); \
     template cudaError_t launch_finite_check<T>(const T *, size_t, int *, cudaStream_t);
 ADI_INST(float)
 ADI_INST(double)

@@ -212,7 +212,8 @@ int step_static(int method, int nx, int ny, double h, double dt, const T *c, con
     if (e == cudaSuccess) e = cudaMemcpyAsync(w_out, w, g.nW * esz, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = launch_precompute<T>(dd, nl, tab, status, s);
     // carried state a, w* from the natural fields (read through the y-lines' u_out/w_out)
-    if (e == cudaSuccess) e = launch_prologue_lines<T>(dd + g.piy, g.pix, ny, method, (const T *)(base + L.fac), s);
+    if (e == cudaSuccess) e = launch_prologue_lines<T>(dd + g.piy, g.pix, ny, method, (const T *)(base + L.fac), alpha + 1,
+                                                       g.ldu, A + 1, g.ldu, s);
     if (e == cudaSuccess) e = launch_line_solve_short<T>(dd, g.piy, method, nx, 0, s);
     if (e == cudaSuccess) e = launch_line_solve_short<T>(dd + g.piy, g.pix, method, ny, 1, s);
     int singular = 0;
