@@ -469,8 +469,8 @@ def peak_leg(adi, torch, side, steps, peak):
 
 def paper_leg(adi, side, steps=2, kmax=6):
     """The paper's own stage solver on this GPU for comparison: the fixed-point iteration of
-    Eq. 9 with kmax sweeps per stage (no early stop), one thread per line, on the same two
-    simulations, FP32; device time of the steps."""
+    Eq. 9 with kmax sweeps per stage (no early stop), on the same two simulations, FP32; device
+    time of the steps."""
     pts, ms = 0, 0.0
     for sp in make_specs(side, steps):
         from paper_2006_07583_gb300 import workloads as wl
@@ -481,8 +481,8 @@ def paper_leg(adi, side, steps=2, kmax=6):
                                              kmax=kmax, eps=0.0, precision=adi.ADI_FP32)
         pts += sp.nx * sp.ny
         ms += t / steps
-    return {"workload": "the paper's fixed-point stage solver (Eq. 9, %d sweeps per stage, one thread "
-                        "per line), same two %dx%d simulations, FP32, one after the other" % (kmax, side, side),
+    return {"workload": "the paper's fixed-point stage solver (Eq. 9, %d sweeps per stage), "
+                        "same two %dx%d simulations, FP32, one after the other" % (kmax, side, side),
             "value": pts / (ms / 1e3), "unit": UNIT, "ms_per_step": ms, "steps": steps}
 
 

@@ -193,7 +193,7 @@ int adi_set_harmonic(adi_handle sim, const double *B, const double *F, double om
  * A simulation with layers writes its natural fields every step and rebuilds its carried state
  * from the damped fields (the work of adi_set_fields' prologue), about one more stage's worth
  * of memory traffic per step.  Works with batches, graphs, sources and adi_set_harmonic.
- * Device memory: the y-line descriptors of both parities and the prologue's scratch.
+ * Device memory: the y-line descriptors of both parities, the prologue's factors and the axes' tables.
  * Errors: ADI_EINVAL (negative or non-finite values), ADI_EBUSY in a batch, ADI_ENOMEM,
  * ADI_ECUDA.
  */

@@ -463,8 +463,8 @@ __global__ void transpose_kernel(const T *__restrict__ src, int rows, int cols, 
 // The entries of the carried arrays that no line writes, from the natural fields: the outer rows and columns
 // of the pressure arrays (the Dirichlet data), the first and last columns of both w* copies and the first and
 // last rows of the v copy that the next step writes.  Everything else of these arrays is written before
-// it is read (A[1] and A[2] by stage 1, A[0] and the current w* by the prologue, A[3] by stage 2, the other w* and v copies by
-// the step), so loading new fields copies edges only: at 4096^2 four transposes and three copies of whole
+// it is read (A[1] and A[2] by stage 1, A[0] and the current w* by the prologue, A[3] by stage 2, the other w* and v
+// copies by the step), so loading new fields copies edges only: at 4096^2 four transposes and three copies of whole
 // fields (300 us) became one launch of 5 us.
 template <typename T>
 struct EdgeRec {
