@@ -483,6 +483,9 @@ __host__ __device__ __forceinline__ void prologue_win_rows(int n, int r0, int r1
     }
 }
 
+// Whether the chunk [r0, r1) of an n-row system is INNER.
+__host__ __device__ inline bool prologue_inner(int n, int r0, int r1) { return r0 > 0 && r1 + kProH < n; }
+
 // The same with right-hand sides q(r) and out(r, x); lo, cu, id of the whole line, forward values in tmp[(r - t0) * ts].
 template <typename T, typename QF>
 struct ProRowsOf {
@@ -505,30 +508,35 @@ __host__ __device__ __forceinline__ void prologue_win_solve(int n, int r0, int r
 
 // The rows of the kernel below: q(r) = (3 x(r + 1) - 3 x(r - 1)) ih but for the boundary rows 0 and n - 1, x(k) for k0 <=
 // k <= k1 loaded once each, and y(r).
-template <typename T, bool INNER>
+template <typename T, bool INNER, typename P = const T *>
 struct ProRows {
-    const T *x, *y;
+    P x, y;
     int xs, ys, k0, k1, n, r0, r1;
     T ih, first, last, below, at, v[kProU];
-    __device__ T ld(int k) const { return x[(long long)(INNER ? k : min(max(k, k0), k1)) * xs]; }
-    __device__ void start(int s) {
+    __host__ __device__ T ld(int k) const { return x[(long long)(INNER ? k : min(max(k, k0), k1)) * xs]; }
+    __host__ __device__ void start(int s) {
         below = ld(s - 1);
         at = ld(s);
 #pragma unroll
         for (int i = 0; i < kProU; ++i) v[i] = ld(s + 1 + i);
     }
-    __device__ void next(int r, T (&q)[kProU]) {
+    __host__ __device__ void next(int r, T (&q)[kProU]) {
         T w[kProU];
+        // an INNER window's last batch asks for nothing: what would come next lies up to 16 rows beyond the window and
+        // is not used, and the field may end with the window's last row
+        const bool more = !INNER || r + kProU < r1 + kProH;
+        if (more)
 #pragma unroll
-        for (int i = 0; i < kProU; ++i) w[i] = ld(r + kProU + 1 + i);
+            for (int i = 0; i < kProU; ++i) w[i] = ld(r + kProU + 1 + i);
 #pragma unroll
         for (int i = 0; i < kProU; ++i) {
             q[i] = mul_rn(fma_of(T(3), v[i], mul_rn(T(-3), below)), ih);
             below = at;
             at = v[i];
         }
+        if (more)
 #pragma unroll
-        for (int i = 0; i < kProU; ++i) v[i] = w[i];
+            for (int i = 0; i < kProU; ++i) v[i] = w[i];
         if (INNER) return;
         if (r == 0) q[0] = first;
         if (r + kProU >= n)
@@ -536,13 +544,13 @@ struct ProRows {
             for (int i = 0; i < kProU; ++i)
                 if (r + i == n - 1) q[i] = last;
     }
-    __device__ void back_start(int r) { ask(r); }
-    __device__ void back(int r, T (&out)[kProU]) {
+    __host__ __device__ void back_start(int r) { ask(r); }
+    __host__ __device__ void back(int r, T (&out)[kProU]) {
 #pragma unroll
         for (int i = 0; i < kProU; ++i) out[i] = v[i];
         ask(r - kProU);
     }
-    __device__ void ask(int r) {
+    __host__ __device__ void ask(int r) {
         if (r < r0 || r >= r1) return;  // no batch of the chunk
 #pragma unroll
         for (int i = 0; i < kProU; ++i) v[i] = y[(long long)(INNER ? r + i : min(r + i, r1 - 1)) * ys];
@@ -616,7 +624,7 @@ __global__ void __launch_bounds__(32 * kProWarps<T>) prologue_cfd_kernel(const L
             tu[r - r0][lane] = y_r;
         };
         const T *lo = sfac[warp][0], *cu = sfac[warp][1], *id = sfac[warp][2], *su = ssu[warp];
-        if (r0 > 0 && r1 + kProH < n) {
+        if (prologue_inner(n, r0, r1)) {
             ProRows<T, true> rows{x, y, xs, ys, 0, k1, n, r0, r1, ih};
             prologue_win_rows<true, T>(n, r0, r1, rows, lo, cu, id, su, &tile[0][lane], &tu[0][lane], 33, out);
         } else {
