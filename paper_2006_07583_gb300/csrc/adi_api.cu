@@ -1300,7 +1300,8 @@ int stage_fields(adi_sim *s, const void *const f[3], bool f32, const void *stage
     }
     int flags[2] = {0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(flags, s->plan.fault.p, sizeof(flags), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    const cudaError_t waited = cudaStreamSynchronize(s->stream);  // after an error too: no copy outlives the call
+    if (e == cudaSuccess) e = waited;
     if (e != cudaSuccess) return s->sticky = cuda_status(e);
     if (flags[0]) return s->sticky = ADI_ETIMEOUT;
     return flags[1] ? ADI_EINVAL : ADI_OK;
@@ -1869,7 +1870,8 @@ namespace {
 // adi_read_fields / adi_read_fields_f32.  A field whose host type or row length differs from the device
 // array's is first converted or packed into its slot of the staging buffer (a pitched device-to-host
 // copy runs at about half the speed of a contiguous one).  One wait covers the work before and all copies; the
-// fault word comes with them.
+// fault word comes with them.  Nothing is queued before the staging buffer is there, and an error waits too, so that no
+// copy into the caller's arrays outlives the call.
 int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
     if (!s) return ADI_EINVAL;
     if (s->in_batch && s->batch_stream) {
@@ -1885,14 +1887,17 @@ int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
     const bool dev32 = s->precision == ADI_FP32;
     size_t off[4];
     xfer_slots(g, off);
+    auto staged = [&](int k) { return parts[k].dst && (dev32 != f32 || parts[k].ld != parts[k].cols); };
+    if (staged(0) || staged(1) || staged(2)) {
+        int rc = xfer_buffer(s);
+        if (rc) return rc;
+    }
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
         auto &pt = parts[k];
         if (!pt.dst) continue;
         const void *src = pt.src;
-        if (dev32 != f32 || pt.ld != pt.cols) {
-            int rc = xfer_buffer(s);
-            if (rc) return rc;
+        if (staged(k)) {
             void *slot = (unsigned char *)s->xfer.p + off[k];
             const dim3 grid = conv_grid(pt.rows, pt.cols);
             if (dev32 && f32)
@@ -1912,7 +1917,8 @@ int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
     }
     int fault = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&fault, s->plan.fault.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    const cudaError_t waited = cudaStreamSynchronize(s->stream);
+    if (e == cudaSuccess) e = waited;
     if (e != cudaSuccess) return s->sticky = cuda_status(e);
     if (fault) s->sticky = ADI_ETIMEOUT;
     return s->sticky;

@@ -1,0 +1,86 @@
+"""CPU: the library's host code on a CUDA runtime without a GPU (tests/fake_cudart.cpp), where allocations fail, waits run
+out and copies stay queued until their stream is waited for."""
+import ctypes as ct
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2006_07583_gb300 import build as _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CFD, MFD, FP32, FP64 = 0, 1, 0, 1
+OK, EINVAL, ENOMEM, ECUDA, ETIMEOUT = 0, 1, 2, 3, 5
+
+
+@pytest.fixture(scope="module")
+def lib():
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    _build.build()
+    out = os.path.join(HERE, "_build")  # git-ignored
+    os.makedirs(out, exist_ok=True)
+    so = os.path.join(out, "libadi_host.so")
+    objs = [os.path.join(_build.BUILD, os.path.basename(s)[:-3] + ".o") for s in _build.sources()]
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    r = subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + inc, "-Wl,-Bsymbolic", "-o", so,
+                        os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-lpthread"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    return ct.CDLL(so)
+
+
+def _ptr(a):
+    return a.ctypes.data_as(ct.c_void_p)
+
+
+def _sim(lib, method, nx, ny, precision):
+    n = (nx + 1) * (ny + 1) if method == CFD else (nx + 2) * (ny + 2)
+    c, h = np.ones(n), ct.c_void_p()
+    assert lib.adi_create(ct.byref(h), method, nx, ny, ct.c_double(1.0 / nx), ct.c_double(0.5 / nx), _ptr(c), None, None,
+                          None, precision) == OK
+    return h
+
+
+def _arrays(method, nx, ny, dtype):
+    if method == CFD:
+        shapes = [(ny + 1, nx + 1)] * 3
+    else:
+        shapes = [(ny + 2, nx + 2), (ny + 2, nx + 1), (ny + 1, nx + 2)]
+    return [np.full(s, 7.0, dtype) for s in shapes]
+
+
+@pytest.mark.parametrize("method", [CFD, MFD])
+@pytest.mark.parametrize("precision", [FP32, FP64])
+@pytest.mark.parametrize("f32", [False, True])
+def test_read_without_staging_memory_leaves_nothing_behind(lib, method, precision, f32):
+    """The staging buffer's allocation fails: no copy into the caller's arrays is on its way when the call returns, and
+    none was made.  The handle stays usable."""
+    h = _sim(lib, method, 20, 18, precision)
+    read = lib.adi_read_fields_f32 if f32 else lib.adi_read_fields
+    out = _arrays(method, 20, 18, np.float32 if f32 else np.float64)
+    lib.fake_fail_alloc(0)
+    rc = read(h, *[_ptr(a) for a in out])
+    lib.fake_fail_alloc(-1)
+    assert rc == ENOMEM
+    assert lib.fake_host_writes() == 0
+    lib.fake_run_all()
+    assert all((a == 7.0).all() for a in out)
+    assert read(h, *[_ptr(a) for a in out]) == OK
+    assert all((a == 0.0).all() for a in out)
+    assert lib.adi_destroy(h) == OK
+
+
+@pytest.mark.parametrize("launch", [0, 1, 2])
+def test_read_error_leaves_no_copy_on_its_way(lib, launch):
+    """A conversion's launch fails after other fields' copies were queued: they have ended when the call returns."""
+    h = _sim(lib, MFD, 20, 18, FP32)
+    out = _arrays(MFD, 20, 18, np.float64)
+    lib.fake_fail_launch(launch)
+    rc = lib.adi_read_fields(h, *[_ptr(a) for a in out])
+    lib.fake_fail_launch(-1)
+    assert rc == ECUDA
+    assert lib.fake_host_writes() == 0
+    assert lib.adi_destroy(h) == OK
