@@ -287,6 +287,7 @@ struct adi_sim {
     // adi_set_source after creation and kept until adi_destroy (adi_create frees its own)
     DevBuf xfer, pro;
     int parity = 0;                           // which V/W copy is current
+    bool unchecked = false;                   // the own plan has stepped since its fault word was read
     int plan_base = 0;                        // parity at which the own plan was built
     std::vector<unsigned char> h_desc[2][2];  // host descriptors [parity][0 = x-lines, 1 = y-lines]
     int nlines[2] = {0, 0};
@@ -1853,6 +1854,7 @@ int adi_step(adi_handle s, int nsteps) {
     if (e != cudaSuccess) return s->sticky = cuda_status(e);
     s->steps += nsteps;
     s->parity ^= nsteps & 1;
+    s->unchecked = true;
     return ADI_OK;
 }
 
@@ -1863,15 +1865,17 @@ int adi_sync(adi_handle s) {
     if (e != cudaSuccess) return s->sticky = cuda_status(e);
     int rc = plan_fault(s->plan, s->stream);
     if (rc) s->sticky = rc;
+    s->unchecked = false;
     return s->sticky;
 }
 
 namespace {
 // adi_read_fields / adi_read_fields_f32.  A field whose host type or row length differs from the device
 // array's is first converted or packed into its slot of the staging buffer (a pitched device-to-host
-// copy runs at about half the speed of a contiguous one).  One wait covers the work before and all copies; the
-// fault word comes with them.  Nothing is queued before the staging buffer is there, and an error waits too, so that no
-// copy into the caller's arrays outlives the call.
+// copy runs at about half the speed of a contiguous one).  The caller's arrays are written only once the solves before
+// are known to have ended: after steps that no call has waited for, the fault word is read first; else (a member of a
+// batch, or after adi_sync) one wait covers the conversions and all copies.  Nothing is queued before the staging
+// buffer is there, and an error waits too, so that no copy into the caller's arrays outlives the call.
 int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
     if (!s) return ADI_EINVAL;
     if (s->in_batch && s->batch_stream) {
@@ -1895,7 +1899,6 @@ int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
         auto &pt = parts[k];
-        if (!pt.dst) continue;
         const void *src = pt.src;
         if (staged(k)) {
             void *slot = (unsigned char *)s->xfer.p + off[k];
@@ -1909,18 +1912,23 @@ int read_fields_any(adi_handle s, void *u, void *v, void *w, bool f32) {
             else
                 convert_out<double, double><<<grid, 256, 0, s->stream>>>((const double *)src, (double *)slot, pt.rows, pt.cols, pt.ld);
             e = cudaGetLastError();
-            src = slot;
+            pt.src = slot;
         }
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(pt.dst, src, pt.rows * pt.cols * (f32 ? sizeof(float) : sizeof(double)), cudaMemcpyDeviceToHost,
+    }
+    if (e == cudaSuccess && s->unchecked) {
+        const int rc = plan_fault(s->plan, s->stream);
+        if (rc) return s->sticky = rc;
+        s->unchecked = false;
+    }
+    for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+        const auto &pt = parts[k];
+        if (pt.dst)
+            e = cudaMemcpyAsync(pt.dst, pt.src, pt.rows * pt.cols * (f32 ? sizeof(float) : sizeof(double)), cudaMemcpyDeviceToHost,
                                 s->stream);
     }
-    int fault = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&fault, s->plan.fault.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream);
     const cudaError_t waited = cudaStreamSynchronize(s->stream);
     if (e == cudaSuccess) e = waited;
-    if (e != cudaSuccess) return s->sticky = cuda_status(e);
-    if (fault) s->sticky = ADI_ETIMEOUT;
+    if (e != cudaSuccess) s->sticky = cuda_status(e);
     return s->sticky;
 }
 

@@ -84,3 +84,23 @@ def test_read_error_leaves_no_copy_on_its_way(lib, launch):
     assert rc == ECUDA
     assert lib.fake_host_writes() == 0
     assert lib.adi_destroy(h) == OK
+
+
+@pytest.mark.parametrize("method", [CFD, MFD])
+@pytest.mark.parametrize("precision", [FP32, FP64])
+@pytest.mark.parametrize("f32", [False, True])
+def test_read_after_a_timeout_leaves_the_arrays_alone(lib, method, precision, f32):
+    """A solve's bounded wait ran out: the read says so and the caller's arrays hold what they held, in the first call
+    and in later ones; a simulation whose solves ended reads as usual."""
+    read = lib.adi_read_fields_f32 if f32 else lib.adi_read_fields
+    for fault in (0, 1):
+        h = _sim(lib, method, 20, 18, precision)
+        out = _arrays(method, 20, 18, np.float32 if f32 else np.float64)
+        lib.fake_raise_fault(fault)
+        assert lib.adi_step(h, 1) == OK
+        lib.fake_raise_fault(0)
+        for _ in range(2):
+            assert read(h, *[_ptr(a) for a in out]) == (ETIMEOUT if fault else OK)
+            lib.fake_run_all()
+            assert all((a == (7.0 if fault else 0.0)).all() for a in out)
+        assert lib.adi_destroy(h) == OK
