@@ -409,9 +409,9 @@ int run_fixed(int method, int nx, int ny, double h, double dt, const double *c_f
     };
     auto smem = [&](const FpLines &g) { return (size_t)lines_of(g) * fp_pitch(g.N) * sizeof(T); };
     auto grid = [&](const FpLines &g) { return (unsigned)((g.n + lines_of(g) - 1) / lines_of(g)); };
-    const int most = (int)std::max(smem(rows), smem(cols));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_rhs_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    // the limit is the process's, not this call's: the same for every size, so that no call lowers it under another's
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_rhs_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fp_sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) { (void)cudaGetLastError(); return ADI_ECUDA; }
     FpState *st = (FpState *)state.p;
     auto copy = [&](int dst, int src0, int src1, size_t n, const FpState *s) {

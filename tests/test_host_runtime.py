@@ -104,3 +104,22 @@ def test_read_after_a_timeout_leaves_the_arrays_alone(lib, method, precision, f3
             lib.fake_run_all()
             assert all((a == (7.0 if fault else 0.0)).all() for a in out)
         assert lib.adi_destroy(h) == OK
+
+
+@pytest.mark.parametrize("precision", [FP32, FP64])
+@pytest.mark.parametrize("method", [CFD, MFD])
+def test_fixed_point_keeps_its_shared_memory_limit(lib, method, precision):
+    """The dynamic shared memory limit of a kernel belongs to the process: a call with short lines leaves it where a
+    call with long lines, which another thread may be in the middle of, needs it."""
+    for n in (4000, 16):
+        shapes = [a.shape for a in _arrays(method, n, 16, np.float64)]
+        c, u, v, w = [np.ones(s) for s in shapes[:1] + shapes]
+        sweeps, ms = ct.c_longlong(), ct.c_double()
+        rc = lib.adi_fixed_point(method, n, 16, ct.c_double(1.0 / n), ct.c_double(0.1 / n), _ptr(c), _ptr(u), _ptr(v), _ptr(w), 1,
+                                 ct.c_double(0.0), None, 2, ct.c_double(0.0), precision, ct.byref(sweeps), ct.byref(ms))
+        assert rc == OK
+        for kernel in (b"fp_sweep_kernel", b"fp_rhs_kernel"):
+            name = kernel + (b"IdE" if precision == FP64 else b"IfE")
+            limit, used = ct.c_longlong(), ct.c_longlong()
+            lib.fake_smem(name, ct.byref(limit), ct.byref(used))
+            assert limit.value >= used.value >= 48 * 1024
