@@ -2028,14 +2028,16 @@ cudaError_t launch_fac_inst(const LineDesc<T> *d, const FacGroup *groups, int ng
                             int grid, int natural, int q, int *fault, cudaStream_t s) {
     auto kern = line_solve_factored_kernel<T, BS, MM, SPLIT, NT>;
     // the host sizes the ring with fac_static_smem, an upper bound of the kernel's own static
-    // shared memory: check it against the compiled kernel once
-    static const bool static_ok = [&] {
+    // shared memory: check it against the compiled kernel once.  The dynamic limit is the process's, so it is
+    // all that the static part leaves, whatever this launch needs: no thread lowers it under another's launch
+    static const int dyn_max = [&] {
         cudaFuncAttributes a{};
-        return cudaFuncGetAttributes(&a, kern) == cudaSuccess && a.sharedSizeBytes <= fac_static_smem(sizeof(T), BS);
+        if (cudaFuncGetAttributes(&a, kern) != cudaSuccess || a.sharedSizeBytes > fac_static_smem(sizeof(T), BS)) return -1;
+        return (int)(kFacSmemLimit - a.sharedSizeBytes);
     }();
-    if (!static_ok) return cudaErrorInvalidConfiguration;
     const size_t dyn = (size_t)stages * stage_bytes;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    if (dyn_max < 0 || dyn > (size_t)dyn_max) return cudaErrorInvalidConfiguration;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max);
     if (e != cudaSuccess) return e;
     kern<<<grid, NT, dyn, s>>>(d, groups, ngroups, natural, (unsigned)stage_bytes, stages, q, fault);
     return cudaGetLastError();

@@ -123,3 +123,14 @@ def test_fixed_point_keeps_its_shared_memory_limit(lib, method, precision):
             limit, used = ct.c_longlong(), ct.c_longlong()
             lib.fake_smem(name, ct.byref(limit), ct.byref(used))
             assert limit.value >= used.value >= 48 * 1024
+
+
+@pytest.mark.parametrize("precision,kernel", [(FP32, b"IfLi2ELi9ELb0E"), (FP64, b"IdLi2ELi9ELb0E")])
+def test_line_solves_keep_their_shared_memory_limit(lib, precision, kernel):
+    """The same for the factored solver's launches: simulations of different sizes are stepped from several threads."""
+    for n in (4000, 16):
+        h = _sim(lib, CFD, n, 16, precision)
+        assert lib.adi_step(h, 1) == OK and lib.adi_sync(h) == OK and lib.adi_destroy(h) == OK
+        limit, used = ct.c_longlong(), ct.c_longlong()
+        lib.fake_smem(b"line_solve_factored_kernel" + kernel, ct.byref(limit), ct.byref(used))
+        assert limit.value >= used.value >= 48 * 1024
