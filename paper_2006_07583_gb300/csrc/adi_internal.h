@@ -57,16 +57,17 @@ constexpr int kV1ShortCells = 128;
 template <typename T>
 cudaError_t launch_line_solve_short(const LineDesc<T> *d, int nlines, int method, int N, int write_natural, cudaStream_t s);
 // CFD: 3 (N+1) + 3 (N-1) Thomas factors of P and Pbar, then the start-up factors of the
-// chunked solves (prologue_factor_count(N) values in all)
+// chunked solves (prologue_factor_count(N) values in all); pivots: pivots in place of their inverses
 void prologue_factors(int N, std::vector<double> &out);
-void prologue_factors(int N, double *out);
+void prologue_factors(int N, double *out, bool pivots = false);
 size_t prologue_factor_count(int N);
 // The prologue over the y-lines of one simulation (N cells each), spread over the lines' elements;
 // fac: the Thomas factors of prologue_factors() in T (CFD; nullptr for MFD).  al, a: the first line's column of the row-major
-// alpha (leading dimension ald) and of the row-major carried a that is written (lda); line k is k columns on.
+// alpha (leading dimension ald) and of the row-major carried a that is written (lda); line k is k columns on.  pivots: fac
+// holds pivots (lines of at most kV1ShortCells cells).
 template <typename T>
 cudaError_t launch_prologue_lines(const LineDesc<T> *col_lines, int nlines, int N, int method, const T *fac, const T *al,
-                                  int ald, T *a, int lda, cudaStream_t s);
+                                  int ald, T *a, int lda, cudaStream_t s, bool pivots = false);
 template <typename T>
 cudaError_t launch_finite_check(const T *x, size_t n, int *flag, cudaStream_t s);
 

@@ -191,7 +191,7 @@ int step_static(int method, int nx, int ny, double h, double dt, const T *c, con
     if (method == ADI_CFD) {
         nfac = prologue_factor_count(ny);
         if (nfac > kMaxFactors) return ADI_ENOMEM;
-        prologue_factors(ny, g_host_factors);
+        prologue_factors(ny, g_host_factors, true);
         T *hf = (T *)(g_host_descs + (L.fac - L.desc));
         for (size_t k = 0; k < nfac; ++k) hf[k] = (T)g_host_factors[k];
     }
@@ -213,7 +213,7 @@ int step_static(int method, int nx, int ny, double h, double dt, const T *c, con
     if (e == cudaSuccess) e = launch_precompute<T>(dd, nl, tab, status, s);
     // carried state a, w* from the natural fields (read through the y-lines' u_out/w_out)
     if (e == cudaSuccess) e = launch_prologue_lines<T>(dd + g.piy, g.pix, ny, method, (const T *)(base + L.fac), alpha + 1,
-                                                       g.ldu, A + 1, g.ldu, s);
+                                                       g.ldu, A + 1, g.ldu, s, true);
     if (e == cudaSuccess) e = launch_line_solve_short<T>(dd, g.piy, method, nx, 0, s);
     if (e == cudaSuccess) e = launch_line_solve_short<T>(dd + g.piy, g.pix, method, ny, 1, s);
     int singular = 0;

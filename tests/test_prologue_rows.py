@@ -1,5 +1,5 @@
-"""CPU: tests/prologue_rows_check.cu runs the prologue kernel's windows on the host for every line of 16 to 4096 cells
-(no GPU needed).  GPU: fields loaded into CFD grids around the first windows with constant factors."""
+"""CPU: tests/prologue_rows_check.cu runs the prologue kernel's windows on the host for every line of 16 to 4096 cells, and
+tests/static_prologue_check.cu measures the error of those of the allocation-free step (no GPU needed).  GPU: fields loaded into CFD grids around the first windows with constant factors."""
 import os
 import shutil
 import subprocess
@@ -14,19 +14,27 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 
 
-def test_prologue_rows_host_check():
+def _build_and_run(name):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not available")
     out = os.path.join(HERE, "_build")  # git-ignored
     os.makedirs(out, exist_ok=True)
-    exe = os.path.join(out, "prologue_rows_check")
+    exe = os.path.join(out, name)
     r = subprocess.run([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-I" + os.path.join(ROOT, "include"),
-                        "-diag-suppress", "20011,20013,20014", "-o", exe, os.path.join(HERE, "prologue_rows_check.cu")],
+                        "-diag-suppress", "20011,20013,20014", "-o", exe, os.path.join(HERE, name + ".cu")],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
     r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "bad 0" in r.stdout, r.stdout[-2000:]
+
+
+def test_prologue_rows_host_check():
+    _build_and_run("prologue_rows_check")
+
+
+def test_static_prologue_error_host_check():
+    _build_and_run("static_prologue_check")
 
 
 # P has such a window from ny = 160 on (its rows 64 to 127), Pbar from 162 on; 224 | 226 give a second one, and 208 is
