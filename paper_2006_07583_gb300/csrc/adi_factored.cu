@@ -310,7 +310,9 @@ __device__ __forceinline__ float fac_rcp(float x) {
 }
 // FP64: the hardware approximation r0 (about 20 bits) and one step of Householder's cubic iteration, r0 (1 + e
 // + e^2) with e = 1 - x r0: three FMAs against a division's ten or so operations on the FP64 pipe that bounds these kernels;
-// the error left is e^3 = 2^-60 and one rounding (measured against 1 / x: at most 1 ulp).
+// the error left is e^3 = 2^-60 and one rounding (measured against 1 / x: at most 1 ulp).  For the pivots of MfdBand only,
+// where divisions made 1001 lines of 1001 cells 299 in place of 288 us a step and the step's error against extended precision, over grids
+// of 48 to 1001 cells a side, no smaller (9.38e-16, 9.33e-16 and 7.80e-16 for u, v and w with either).
 __device__ __forceinline__ double fac_rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -918,18 +920,21 @@ __device__ __forceinline__ void seg_scan(Map<T, BS> a, bool forward, int Tl, T (
     }
 }
 
-// Block inverse of the line kernel.
+// Block inverse of the line kernel.  CFD in FP64 divides: with fac_rcp a step's error was no smaller (v and w 0.03 %
+// larger) for 2 % of its time (512 x 512 cells: 108 us, 106 with it).
+__device__ __forceinline__ float fac_block_rcp(float x) { return fac_rcp(x); }
+__device__ __forceinline__ double fac_block_rcp(double x) { return 1.0 / x; }
 template <typename T, int BS>
 __device__ __forceinline__ void fac_inv(const T (&S)[BS][BS], T (&R)[BS][BS]) {
     if constexpr (BS == 2) {
-        const T id = fac_rcp(S[0][0] * S[1][1] - S[0][1] * S[1][0]);
+        const T id = fac_block_rcp(S[0][0] * S[1][1] - S[0][1] * S[1][0]);
         R[0][0] = S[1][1] * id; R[0][1] = -S[0][1] * id;
         R[1][0] = -S[1][0] * id; R[1][1] = S[0][0] * id;
     } else {
         const T c00 = S[1][1] * S[2][2] - S[1][2] * S[2][1];
         const T c01 = S[1][2] * S[2][0] - S[1][0] * S[2][2];
         const T c02 = S[1][0] * S[2][1] - S[1][1] * S[2][0];
-        const T id = fac_rcp(S[0][0] * c00 + S[0][1] * c01 + S[0][2] * c02);
+        const T id = fac_block_rcp(S[0][0] * c00 + S[0][1] * c01 + S[0][2] * c02);
         R[0][0] = c00 * id;
         R[0][1] = (S[0][2] * S[2][1] - S[0][1] * S[2][2]) * id;
         R[0][2] = (S[0][1] * S[1][2] - S[0][2] * S[1][1]) * id;
