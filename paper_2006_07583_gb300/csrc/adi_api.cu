@@ -410,7 +410,9 @@ __global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restri
     for (int q = threadIdx.x; q < 32 * KV; q += 256) {
         const int jj = q / KV, kv = (q % KV) * V, j = jb + jj, k = k0 + kv;
         if (j < 1 || j >= j1) continue;
-        Vec va{}, vc{}, vn{}, vi{};
+        Vec va, vc{}, vn{}, vi{};
+#pragma unroll
+        for (int i = 0; i < V; ++i) va.x[i] = T(-0.0);  // plus c is c, its zeros' signs included
         if (k < ku1) {
             if (!a_row) va = *reinterpret_cast<const Vec *>(a + j * ldc + k);
             vc = *reinterpret_cast<const Vec *>(c + j * ldc + k);
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restri
         }
 #pragma unroll
         for (int i = 0; i < V; ++i) {
-            tu[jj][kv + i] = T(0.5) * (va.x[i] + vc.x[i]);
+            tu[jj][kv + i] = va.x[i] + vc.x[i];
             tw[jj][kv + i] = T(0.5) * (vn.x[i] + vi.x[i]);
         }
     }
@@ -434,7 +436,8 @@ __global__ void __launch_bounds__(256) naturalize_kernel(const NatDesc *__restri
         const int k = k0 + kk;
         if (k >= ku0 && k < ku1) {
             T u = tu[threadIdx.x & 31][kk];
-            if (a_row) u += T(0.5) * a_row[(long long)k * d.lda + j];  // halves are exact: the same sum
+            if (a_row) u = a_row[(long long)k * d.lda + j] + u;
+            u *= T(0.5);  // of the sum: a subnormal value's half is not exact
             if (k == src_i)  // the point source's dt/2 f is not part of u
                 u -= T(0.5) * (T)(d.src_scale * ricker(d.src_amp, d.src_f0, d.src_td,
                                                        (double)(*d.clock + d.clock_ahead) * d.dt));
