@@ -655,61 +655,75 @@ __device__ bool fac_run(const LineDesc<TS> &d, const FacGeom &g, const double *d
     return true;
 }
 
+__host__ __device__ __forceinline__ float fac_abs(float x) { return x < 0.f ? -x : x; }
+__host__ __device__ __forceinline__ double fac_abs(double x) { return x < 0.0 ? -x : x; }
+
 // Reach of the windowed scans over the windows that start at the chunks [e0, e1) (see the header): the
 // largest number of consecutive stored transfers (forward: F_e F_{e-1} ..., backward: H_s H_{s+1} ...)
 // whose product first has infinity norm at most tau, or that reaches the end of the line; at most
 // kFacMaxReach + 1 (which selects the full scan).
-// A window's products are formed in FP32, and in FP64 only where a norm comes so near tau that FP32's rounding could
-// decide (the FP64 pipe is what the records wait for).
+// A window's products are formed in FP32 with an entrywise bound on what its roundings have done, and again in FP64 where
+// the bound leaves open on which side of tau a norm lies (the FP64 pipe is what the records wait for), so that the reach
+// is FP64's.  The bound: with |P^ - P| <= E, the product P^ M^ of M^ = M (1 + 2^-24) as BS products and sums differs from P M
+// by at most (E + (BS + 1) 2^-24 |P^|) |M|; 2^-21 in its place leaves room for FP64's roundings, 1e-36 for what FP32
+// flushes, and 1 % and 2^-20 of the norm for the roundings of the bound and the norm themselves.  (Entrywise, because the
+// rows of a CFD transfer differ in size: bounds by norms left so much open that most windows ran again.  1023 CFD lines of
+// 1024 cells: 269 us for their records, 364 with such bounds, 367 in FP64 throughout, 267 without a bound.)
 template <typename TS, int BS, typename R>
-__device__ int fac_window(const TS *maps, int tact, double tau, bool forward, int first, bool &unsure) {
+__host__ __device__ int fac_window(const TS *maps, int tact, double tau, bool forward, int first, bool &unsure) {
     constexpr int B2 = BS * BS;
-    R P[BS][BS];
+    constexpr bool kBound = sizeof(R) == 4;
+    R P[BS][BS], E[BS][BS];
 #pragma unroll
     for (int p = 0; p < BS; ++p)
 #pragma unroll
-        for (int q = 0; q < BS; ++q) P[p][q] = p == q ? R(1) : R(0);
+        for (int q = 0; q < BS; ++q) { P[p][q] = p == q ? R(1) : R(0); E[p][q] = R(0); }
     unsure = false;
-    const R lo = (R)(tau * 0.999), hi = (R)(tau * 1.001);
     for (int r = 0;;) {
         const int k = forward ? first - r : first + r;
-        R M[BS][BS], T1[BS][BS], nrm = R(0);
+        R M[BS][BS], T1[BS][BS], E1[BS][BS], nrm = R(0), err = R(0);
 #pragma unroll
         for (int p = 0; p < BS; ++p)
 #pragma unroll
             for (int q = 0; q < BS; ++q) M[p][q] = (R)maps[(size_t)k * B2 + p * BS + q];
 #pragma unroll
         for (int p = 0; p < BS; ++p) {
-            R rs = R(0);
+            R rs = R(0), es = R(0);
 #pragma unroll
             for (int q = 0; q < BS; ++q) {
-                R t = R(0);
+                R t = R(0), b = R(1e-36);
 #pragma unroll
-                for (int m = 0; m < BS; ++m) t += P[p][m] * M[m][q];
+                for (int m = 0; m < BS; ++m) {
+                    t += P[p][m] * M[m][q];
+                    if (kBound) b += (E[p][m] + R(0x1p-21) * fac_abs(P[p][m])) * fac_abs(M[m][q]);
+                }
                 T1[p][q] = t;
-                rs += t < R(0) ? -t : t;
+                E1[p][q] = b;
+                rs += fac_abs(t);
+                es += b;
             }
             nrm = rs > nrm ? rs : nrm;
+            err = es > err ? es : err;
         }
 #pragma unroll
         for (int p = 0; p < BS; ++p)
 #pragma unroll
-            for (int q = 0; q < BS; ++q) P[p][q] = T1[p][q];
+            for (int q = 0; q < BS; ++q) { P[p][q] = T1[p][q]; E[p][q] = E1[p][q]; }
         ++r;
+        if (kBound && !(fac_abs(nrm - (R)tau) > R(1.01) * err + R(0x1p-20) * nrm)) { unsure = true; return r; }
         const bool at_end = forward ? (k == 0) : (k == tact - 1);
-        if (nrm > lo && nrm < hi) unsure = true;
         if (nrm <= (R)tau || at_end || r > kFacMaxReach) return r;
     }
 }
 template <typename TS, int BS>
-__device__ int fac_reach(const TS *maps, int tact, double tau, bool forward, int e0, int e1) {
+__host__ __device__ int fac_reach(const TS *maps, int tact, double tau, bool forward, int e0, int e1) {
     int reach = 0;
     for (int e = e0; e < e1 && e < tact - 1 && reach <= kFacMaxReach; ++e) {
         const int first = forward ? e : e + 1;  // chunk whose transfer the window starts with
         bool unsure;
         int r = fac_window<TS, BS, float>(maps, tact, tau, forward, first, unsure);
         if (unsure) r = fac_window<TS, BS, double>(maps, tact, tau, forward, first, unsure);
-        reach = max(reach, r);
+        reach = r > reach ? r : reach;
     }
     return reach;
 }
