@@ -18,10 +18,10 @@ __device__ __forceinline__ int cfd_idx_e(int j) { return 2 * j - 1; }
 // Reciprocal: IEEE round-to-nearest in both precisions (the FP32 intrinsic avoids the
 // general division sequence).
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__host__ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
 template <typename T, int BS>
-__device__ __forceinline__ void mat_inv(const T (&S)[BS][BS], T (&R)[BS][BS]) {
+__host__ __device__ __forceinline__ void mat_inv(const T (&S)[BS][BS], T (&R)[BS][BS]) {
     if constexpr (BS == 2) {
         T det = S[0][0] * S[1][1] - S[0][1] * S[1][0];
         T id = recip(det);

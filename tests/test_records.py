@@ -1,5 +1,6 @@
 """CPU checks of how the factored solver's records are built (no GPU needed), from the CUDA sources run on the host:
-tests/reach_check.cu, the windowed scans' reach against the same products in FP64."""
+tests/reach_check.cu, the windowed scans' reach against the same products in FP64; tests/records_check.cu, the records of
+lines built by several runs against extended precision."""
 import os
 import shutil
 import subprocess
@@ -26,3 +27,7 @@ def _build_and_run(name):
 
 def test_reach_host_check():
     _build_and_run("reach_check")
+
+
+def test_records_host_check():
+    _build_and_run("records_check")
