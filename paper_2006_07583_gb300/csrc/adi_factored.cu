@@ -37,6 +37,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 
 #include "../../include/adi.h"
 #include "adi_internal.h"
@@ -180,9 +181,11 @@ constexpr size_t kDescBytes = sizeof(LineDesc<float>);
 static_assert(sizeof(LineDesc<float>) == sizeof(LineDesc<double>), "descriptor sizes differ");
 static_assert(kDescBytes % 16 == 0, "descriptor size");
 __host__ __device__ inline size_t fac_desc_area(int nl) { return ((size_t)nl * kDescBytes + 127) & ~(size_t)127; }
-// A stage: the group (192 bytes), the descriptors, then the lines.
-constexpr size_t kFacGroupBytes = 192;
-static_assert(sizeof(FacGroup) % 16 == 0 && sizeof(FacGroup) <= kFacGroupBytes, "group header");
+// A stage: the group's header (its fields before the base addresses, which only the staging warp reads, from global
+// memory), the descriptors, then the lines.  With the whole 192-byte record staged, lines of 703-706 MFD cells went four
+// instead of five to a CTA.
+constexpr size_t kFacGroupBytes = offsetof(FacGroup, gp);
+static_assert(kFacGroupBytes == 128 && alignof(FacGroup) == 16, "group header");
 __host__ __device__ inline size_t fac_head_bytes(int nl) { return kFacGroupBytes + fac_desc_area(nl); }
 
 size_t fac_stage_bytes(int method, int N, int nl, size_t esz) {
@@ -1069,7 +1072,7 @@ __device__ void fac_issue(const LineDesc<T> *__restrict__ descs, const FacGroup 
     const unsigned bv = round16((unsigned)gr.vn * (unsigned)sizeof(T));
     const unsigned br = (unsigned)(gr.info + 4) * (unsigned)sizeof(T);  // the staged record
     const unsigned bd = (unsigned)(gr.nl * kDescBytes);
-    const unsigned bg = (unsigned)sizeof(FacGroup);
+    const unsigned bg = (unsigned)kFacGroupBytes;
     if (lane == 0) {
         mbar_expect_tx(bar, bg + bd + (unsigned)gr.nl * (2 * bp + bv + br));
         bulk_to_smem(stage, gp, bg, bar);

@@ -6,6 +6,7 @@ import subprocess
 import numpy as np
 import pytest
 
+import oracle
 from paper_2006_07583_gb300 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -64,3 +65,25 @@ def test_natural_pressure_of_subnormal_fields(adi, method, nx, ny):
     for alone, shared in zip(*got):
         assert np.count_nonzero(alone) > alone.size // 2
         assert np.array_equal(alone.view(np.uint32), shared.view(np.uint32))
+
+
+# 16 | 17 chunks a line: the last lengths whose lines store the carried pressure in the next stage's layout and the first
+# ones that do not; and lengths whose lines just fit a CTA's shared memory together
+@pytest.mark.parametrize("method,n,fp64", [(m, n, f) for m, n in ((CFD, 157), (CFD, 158), (MFD, 160), (MFD, 161)) for f in (True, False)]
+                         + [(CFD, 122, False), (CFD, 930, True), (MFD, 150, False), (MFD, 706, False)])
+def test_lines_at_layout_limits(adi, method, n, fp64):
+    """The path's own tolerances: FP64 max |difference| <= 1e-12 x max |field|, FP32 relative L2 <= 1e-4."""
+    rng = np.random.default_rng(n)
+    for nx, ny in ((n, 24), (24, n)):
+        c, *F = [rng.uniform(0.6, 1.4, wl.shapes(method, nx, ny)[0])] + [rng.standard_normal(s) for s in wl.shapes(method, nx, ny)]
+        h = 1.0 / n
+        dt = 0.8 * h / c.max()
+        sim = adi.Sim(method, nx, ny, h, dt, c, *F, precision=adi.ADI_FP64 if fp64 else adi.ADI_FP32)
+        sim.step(3)
+        got = sim.read()
+        sim.close()
+        for g, o in zip(got, oracle.run(method, nx, ny, h, dt, c ** 2, *F, 3)):
+            if fp64:
+                assert np.max(np.abs(g - o)) <= 1e-12 * np.max(np.abs(o))
+            else:
+                assert np.linalg.norm(g - o) <= 1e-4 * np.linalg.norm(o)

@@ -1,6 +1,6 @@
 """CPU checks of how the factored solver's records are built (no GPU needed), from the CUDA sources run on the host:
 tests/reach_check.cu, the windowed scans' reach against the same products in FP64; tests/records_check.cu, the records of
-lines built by several runs against extended precision."""
+lines built by several runs against extended precision; tests/lines_per_cta_check.cu, the lines that fit a CTA."""
 import os
 import shutil
 import subprocess
@@ -31,3 +31,7 @@ def test_reach_host_check():
 
 def test_records_host_check():
     _build_and_run("records_check")
+
+
+def test_lines_per_cta_host_check():
+    _build_and_run("lines_per_cta_check")
