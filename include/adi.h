@@ -225,7 +225,8 @@ int adi_sync(adi_handle sim);
  * handle's current time.  Fields that need converting or packing (FP64 arrays, a padded
  * velocity array) pass through a device staging buffer of three fields in FP64, allocated on
  * its first use and kept until adi_destroy.  Errors: the handle's sticky error, ADI_ENOMEM (the
- * staging buffer), ADI_ECUDA.
+ * staging buffer), ADI_ETIMEOUT, ADI_ECUDA; the buffers are left as they were with the first three, and
+ * in no case written after the call has returned.
  */
 int adi_read_fields(adi_handle sim, double *u, double *v, double *w);
 

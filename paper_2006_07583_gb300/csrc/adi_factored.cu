@@ -103,8 +103,9 @@ __host__ __device__ inline int fac_geom_T(int method, int N) {
 // MFD lines of at most 224 chunks run in FP64 in CTAs of 256 threads: twice the registers a thread (the
 // band form's 72 FP64 values do not fit 128 registers and spilled 0.5 KB a thread, more than the L1 beside the staged
 // lines holds), and seven warps keep the FP64 pipe as busy as fifteen: 1001 lines of 1001 cells 200 ->
-// 144 us with the band form.  CFD, whose lines of 512 cells then made two rounds instead of one, gained nothing (55.7
-// -> 58.0 us) and keeps the wide CTAs.
+// 144 us with the band form; a step at 20 to 2024 cells a side 5 to 16 % faster than in wide CTAs, 1.4 % slower at 881 to 934,
+// where a CTA takes one line in place of two.  CFD, whose lines of 512 cells then made two rounds instead of one, gained
+// nothing (55.7 -> 58.0 us) and keeps the wide CTAs.
 __host__ __device__ inline bool fac_narrow(int method, int T, size_t esz) {
     return method == kMFD && esz == 8 && T <= kFacNarrow - 32;
 }

@@ -437,7 +437,9 @@ template <bool INNER, typename T, bool DIV = false, typename Rows, typename Out>
 __host__ __device__ __forceinline__ void prologue_win_rows(int n, int r0, int r1, Rows rows, const T *lo, const T *cu,
                                                            const T *id, const T *su, T *tmp, T *halo, long long ts,
                                                            Out out) {
-    constexpr int U = kProU, S = 8;  // the start-up's value is rounded after every S rows
+    // The start-up forms each row from the row before's unrounded product and rounds it after every S rows.  There is no
+    // numerical reason for the eight: it is how an unrolled loop was once contracted, kept so that the results are the same bits
+    constexpr int U = kProU, S = 8;
     static_assert(kProH % U == 0 && kProR % U == 0 && U % S == 0, "whole batches");
     const int nr = INNER ? kProR : r1 - r0;
     const int m = INNER ? kProR + kProH : (r1 + kProH < n ? r1 + kProH : n) - r0;  // m > nr only for nr = kProR

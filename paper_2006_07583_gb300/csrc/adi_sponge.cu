@@ -26,7 +26,7 @@ __device__ __forceinline__ double cell_coord(int method, bool staggered, int k, 
     return (double)k - 0.5;
 }
 
-// The factor at distance d of one axis.  It falls with d, so the factor at the nearest wall's distance is
+// The factor at distance d of one axis.  It rises with d, so the factor at the nearest wall's distance is
 // the smaller of the two axes' factors.
 __device__ __forceinline__ double damping(double x, int n, double width, double a) {
     const double d = fmin(x, (double)n - x);
