@@ -1671,7 +1671,13 @@ int adi_autotune(adi_handle s, int trials, int force, int *chosen, double *ms_pe
     }
     s->fac_nl_cap = res.solver == ADI_SOLVER_FACTORED ? res.nl_cap : 0;
     s->fac_ring_cap = res.solver == ADI_SOLVER_FACTORED ? res.ring_cap : 0;
-    rc = adi_set_solver(s, res.solver);  // rebuilds the plan with the chosen parameters
+    const bool same = res.solver == s->solver;  // adi_set_solver then leaves the plan of the last launch tried
+    rc = adi_set_solver(s, res.solver);
+    if (!rc && same) {
+        rc = plan_build(s->plan, std::vector<adi_sim *>{s}, s->stream);
+        s->plan_base = s->parity;
+        if (rc) s->sticky = rc;
+    }
     if (rc) return rc;
     if (chosen) *chosen = res.solver;
     if (ms_per_step)

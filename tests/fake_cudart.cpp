@@ -26,7 +26,7 @@ std::recursive_mutex mu;
 std::set<CUstream_st *> streams;
 CUstream_st legacy;
 std::map<const void *, std::string> names;     // kernels by their host stub
-std::map<const void *, size_t> limits, largest;  // dynamic shared memory: the limit set, the largest launch
+std::map<const void *, size_t> limits, largest, recent;  // dynamic shared memory: the limit set, the largest and the last launch
 std::map<const void *, std::pair<void *, size_t>> vars;
 thread_local cudaError_t last = cudaSuccess;
 int fail_alloc = -1;     // allocations until one fails (-1: none)
@@ -72,6 +72,14 @@ void fake_smem(const char *part, long long *limit, long long *used) {
         if (largest.count(n.first) && (long long)largest[n.first] > *used) *used = (long long)largest[n.first];
         if (limits.count(n.first) && (*limit < 0 || (long long)limits[n.first] < *limit)) *limit = (long long)limits[n.first];
     }
+}
+
+// the dynamic shared memory of the last launch of the kernel whose name contains `part`
+long long fake_last_smem(const char *part) {
+    Lock l(mu);
+    for (auto &n : names)
+        if (n.second.find(part) != std::string::npos && recent.count(n.first)) return (long long)recent[n.first];
+    return -1;
 }
 
 // ---- the runtime ----
@@ -170,6 +178,7 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **args, size_t s
     if (fail_launch >= 0 && fail_launch-- == 0) return set(cudaErrorLaunchFailure);
     const size_t limit = limits.count(k) ? limits[k] : 48 * 1024;
     if (smem > largest[k]) largest[k] = smem;
+    recent[k] = smem;
     if (smem > limit) return set(cudaErrorInvalidValue);
     if (raise_fault && names[k].find("line_solve_factored_kernel") != std::string::npos && !of(s)->capturing) {
         int *fault = *(int **)args[7];  // (descs, groups, ngroups, natural, stage_bytes, stages, q, fault)

@@ -29,7 +29,9 @@ def lib():
     r = subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + inc, "-Wl,-Bsymbolic", "-o", so,
                         os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-lpthread"], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-2000:]
-    return ct.CDLL(so)
+    lib = ct.CDLL(so)
+    lib.fake_last_smem.restype = ct.c_longlong
+    return lib
 
 
 def _ptr(a):
@@ -134,3 +136,22 @@ def test_line_solves_keep_their_shared_memory_limit(lib, precision, kernel):
         limit, used = ct.c_longlong(), ct.c_longlong()
         lib.fake_smem(b"line_solve_factored_kernel" + kernel, ct.byref(limit), ct.byref(used))
         assert limit.value >= used.value >= 48 * 1024
+
+
+def test_autotune_leaves_the_chosen_launch(lib):
+    """Every candidate takes the same time here, so the automatic launch is chosen; the steps after the call run it and
+    not the last one tried, the first time and from the cached choice."""
+    def smem_of_a_step(h):
+        assert lib.adi_step(h, 1) == OK and lib.adi_sync(h) == OK
+        return lib.fake_last_smem(b"line_solve_factored_kernelIfLi2ELi9ELb0E")
+
+    sims = [_sim(lib, CFD, 100, 100, FP32) for _ in range(3)]
+    want = smem_of_a_step(sims[0])
+    for h in sims[1:]:
+        chosen, cap, ring = ct.c_int(-1), ct.c_int(-1), ct.c_int(-1)
+        assert lib.adi_autotune(h, 2, 0, ct.byref(chosen), None) == OK
+        assert lib.adi_get_launch(h, ct.byref(cap), ct.byref(ring)) == OK
+        assert (chosen.value, cap.value, ring.value) == (2, 0, 0)
+        assert smem_of_a_step(h) == want
+    for h in sims:
+        assert lib.adi_destroy(h) == OK
